@@ -402,7 +402,8 @@ __global__ void __launch_bounds__(kBlock) k_pcg_step(DevProblem P, int zc, int j
 #pragma unroll
     for (int i = 0; i < kStepSums; ++i) acc[i].add(part[i]);
     double out[kStepSums];
-    if (grid_reduce<kStepSums>(acc, red, out) && tid == 0) step_scalars(out, j, want_rr, hdr, resid);
+    if (grid_reduce<kStepSums>(acc, red, out, hw_grid(), want_rr ? kStepSums : kSumRR) && tid == 0)
+        step_scalars(out, j, want_rr, hdr, resid);
 }
 
 // -------------------------------------------------------------- PCG final

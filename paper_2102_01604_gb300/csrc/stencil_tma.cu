@@ -391,7 +391,8 @@ __device__ __forceinline__ void step_body(
         __syncthreads();
     }
     double out[kStepSums];
-    if (grid_reduce<kStepSums>(acc, red, out, vg) && tid == 0) step_scalars(out, j, want_rr, hdr, resid);
+    if (grid_reduce<kStepSums>(acc, red, out, vg, want_rr ? kStepSums : kSumRR) && tid == 0)
+        step_scalars(out, j, want_rr, hdr, resid);
 }
 
 template <int K, int TX, int TY, int MODE>
