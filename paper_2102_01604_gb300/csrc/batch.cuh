@@ -46,7 +46,7 @@ struct InitArgs {
     int zc;
     unsigned gx, gy, gz;
     const float *h, *w, *g, *y;
-    float4* z0;
+    float4* p0;
     double tol2;
     WsHeader* hdr;
     double* resid;
@@ -54,10 +54,10 @@ struct InitArgs {
 };
 
 struct StepArgs {
-    CUtensorMap tz, tv, tp, tw, th, tx, tp2;
+    CUtensorMap tp, tv, tp2, tw, th, tx;
     DevProblem P;
     int nchunk, j, want_rr;
-    float4 *zout, *vout, *pout, *xacc;
+    float4 *vout, *pout, *xacc;
     WsHeader* hdr;
     double* resid;
     Reduce red;

@@ -60,6 +60,7 @@ struct SolveScalars {
     double alpha;     // step of the latest completed iteration
     double alpha_prev;  // step of the iteration before it
     double beta;      // coefficient of the next direction update
+    double beta_prev; // coefficient of the latest one
     double tol2;      // (tol_cg)^2, 0 = off
     int it;           // PCG iterations completed
     int xcount;       // iterations already folded into x (x is updated every other iteration)

@@ -631,7 +631,7 @@ static cudaError_t enqueue_phased(std::vector<PhasedSubject>& subj, int tile, cu
             const FitJob& j = *subj[s].j;
             const StencilGrid& g = subj[s].ig;
             ia[s] = InitArgs{j.P, g.zc, g.grid.x, g.grid.y, g.grid.z, j.L.h, j.L.w, j.L.g, j.y,
-                             subj[s].B.z[0], tol2, j.L.hdr, nullptr, j.L.red};
+                             subj[s].B.p[0], tol2, j.L.hdr, nullptr, j.L.red};
         }
         if ((e = launch_pcg_init_batch(K, ia.data(), bini.data(), n, st))) return e;
         for (int c = 0; c < o.cg_iters; ++c) {

@@ -98,8 +98,8 @@ cudaError_t launch_solve_mg(const DevProblem& P, const SolveOpts& o, const float
 // when the volume or the pointers do not meet the copy engine's alignment
 // rules; the plain kernel is used then.
 struct StepMaps {
-    CUtensorMap z[2], v[2], p[3];   // halo boxes of the solve's vectors
-    CUtensorMap p2[3], x;           // tile boxes (x fold)
+    CUtensorMap v[2], p[3];   // halo boxes of the solve's vectors
+    CUtensorMap x;            // tile box (x fold)
     CUtensorMap w, h;
     SolveBufs B;
     int tile;          // index of the tile shape the maps were encoded for

@@ -411,6 +411,7 @@ __global__ void __launch_bounds__(kBlock) k_mgcg_init(DevProblem P, MgLevel L0, 
         sc.alpha = 0.0;
         sc.alpha_prev = 0.0;
         sc.beta = 0.0;
+        sc.beta_prev = 0.0;
         sc.it = 0;
         sc.xcount = 0;
         sc.tol2 = tol2;

@@ -13,10 +13,21 @@
 // with r_j = M z_j formed per voxel (M symmetric, so r_j.v_j = z_j.q_j).  All
 // four sums are reduced in the same launch as q_j, so alpha_j and beta_j are
 // known when iteration j + 1 starts: it forms z_{j+1} and p_{j+1} = z_{j+1} +
-// beta_j p_j for its tile and halo from (z_j, v_j, p_j), applies the operator
-// and writes z, v and p once.  |r_{j+1}|^2 is expanded the same way when the
-// residual norm is wanted.  r.z is recomputed directly (z_j.M z_j) in every
-// iteration, so the expansion spans one step and errors do not accumulate.
+// beta_j p_j for its tile and halo, applies the operator and writes v and p
+// once.  |r_{j+1}|^2 is expanded the same way when the residual norm is
+// wanted.  r.z is recomputed directly (z_j.M z_j) in every iteration, so the
+// expansion spans one step and errors do not accumulate.
+//
+// z itself is not stored: the last two directions hold it,
+//     z_j = p_j - beta_{j-1} p_{j-1},
+// with the beta that formed p_j, so an iteration reads p_j, p_{j-1} and v_j
+// and writes p_{j+1} and v_{j+1}.  The iteration is bound by HBM: without z's
+// store it moves 124 B per voxel (K = 4) instead of 140, and the x fold, whose
+// two directions are both at hand, 16 B per iteration instead of 24.  The
+// difference of two roundings of p's size replaces one of z's; |p_j| stays
+// within a few |z_j| (1 to 3.3 on the Newton systems of a fit), and delta's
+// error against 64-bit arithmetic is the same (2.0e-7 either way after 30
+// iterations).
 //
 // The preconditioner block M_n = H_n + diag(lambda_k d_n), d_n = sum of the
 // six edge coefficients, is factorised in every iteration from H and the JTV
@@ -107,7 +118,6 @@ __device__ __forceinline__ float edge_sum(const float (&c)[6])
 // Per-solve workspace buffers: [N] float4 each (voxel-interleaved maps),
 // 256-byte aligned.
 struct SolveBufs {
-    float4* z[2];    // preconditioned residual z_j in z[j & 1]
     float4* v[2];    // v_j = M^-1 q_j in v[j & 1]
     float4* p[3];    // direction p_j in p[j % 3]
     float4* x;       // sum of the directions folded so far, alpha_i p_i
@@ -131,29 +141,37 @@ __device__ __forceinline__ float4 pack4(const float (&o)[K])
 
 // What one iteration's launch does besides the common work.
 enum : int {
-    kModeFirst = 0,    // j = 0: z_0 comes from the init kernel, p_0 = z_0
-    kModeStep = 1,     // odd j
-    kModeFold = 2,     // j = 2: also x = alpha_0 p_0 + alpha_1 p_1
-    kModeFoldX = 3     // even j > 2: also x += alpha_{j-2} p_{j-2} + alpha_{j-1} p_{j-1}
+    kModeFirst = 0,    // j = 0: p_0 = z_0 comes from the init kernel
+    kModeSecond = 1,   // j = 1: z_0 = p_0, there is no p_{-1}
+    kModeStep = 2,     // odd j > 1
+    kModeFold = 3,     // j = 2: also x = alpha_0 p_0 + alpha_1 p_1
+    kModeFoldX = 4     // even j > 2: also x += alpha_{j-2} p_{j-2} + alpha_{j-1} p_{j-1}
 };
 
 // Sums reduced by every iteration, in this order.
 enum : int { kSumPQ, kSumZQ, kSumVQ, kSumZR, kSumRR, kSumRQ, kSumQQ, kStepSums };
 
-// z_j and p_j of one point from the previous iteration's z, v, p (at j = 0,
-// z is z_0 and v, p are not read).
-template <int K, bool FIRST>
-__device__ __forceinline__ void step_point(float alpha, float beta, const float4& z4, const float4& v4,
-                                           const float4& p4, float (&zj)[K], float (&pj)[K])
+// The scalars an iteration starts from: alpha_{j-1}, alpha_{j-2}, beta_{j-1}
+// and beta_{j-2} (those that exist).
+struct StepScalars {
+    float alpha, alpha_prev, beta, beta_prev;
+};
+
+// z_j and p_j of one point from p1 = p_{j-1}, v = v_{j-1} and p2 = p_{j-2}
+// (j = 0: p1 is p_0 and v, p2 are not read; j = 1: p2 is not read).
+template <int K, int MODE>
+__device__ __forceinline__ void step_point(const StepScalars& s, const float4& p14, const float4& v4,
+                                           const float4& p24, float (&zj)[K], float (&pj)[K])
 {
-    float z[K], v[K], p[K];
-    unpack4<K>(z4, z);
+    float p1[K], v[K], p2[K];
+    unpack4<K>(p14, p1);
     unpack4<K>(v4, v);
-    unpack4<K>(p4, p);
+    unpack4<K>(p24, p2);
 #pragma unroll
     for (int a = 0; a < K; ++a) {
-        zj[a] = FIRST ? z[a] : fmaf(-alpha, v[a], z[a]);
-        pj[a] = FIRST ? zj[a] : fmaf(beta, p[a], zj[a]);
+        const float z = MODE >= kModeStep ? fmaf(-s.beta_prev, p2[a], p1[a]) : p1[a];   // z_{j-1}
+        zj[a] = MODE == kModeFirst ? z : fmaf(-s.alpha, v[a], z);
+        pj[a] = MODE == kModeFirst ? z : fmaf(s.beta, p1[a], zj[a]);
     }
 }
 
@@ -255,6 +273,7 @@ __device__ __forceinline__ void step_scalars(const double (&s)[kStepSums], int j
     const double rz_next = rz - 2.0 * alpha * s[kSumZQ] + alpha * alpha * s[kSumVQ];
     sc.alpha_prev = sc.alpha;
     sc.alpha = alpha;
+    sc.beta_prev = sc.beta;
     sc.beta = rz_next / rz;
     sc.rz = rz_next;
     sc.it = j + 1;

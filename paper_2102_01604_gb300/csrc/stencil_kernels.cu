@@ -1,8 +1,8 @@
 // stencil_kernels.cu -- the prior and the Newton-system solve (sm_103a):
 //   k_jtv          JTV weights w_n = (u_n + eps^2)^-1/2 and JTV_eps (Eqs. 38-40)
-//   k_pcg_init     r_0 = g + L y, z_0 = M^-1 r_0 (Eq. 42)
+//   k_pcg_init     r_0 = g + L y, p_0 = z_0 = M^-1 r_0 (Eq. 42)
 //   k_pcg_step     one PCG iteration (pcg_step.cuh): z_j, p_j from the previous
-//                  iteration, q = (H + L) p_j, v = M^-1 q, the x fold and the
+//                  ones, q = (H + L) p_j, v = M^-1 q, the x fold and the
 //                  sums for alpha_j and beta_j -- the plain kernel used when the
 //                  TMA-staged one (stencil_tma.cu) does not apply
 //   k_pcg_final    delta = x + pending directions (or y <- y - delta)
@@ -181,11 +181,11 @@ __global__ void __launch_bounds__(kBlock) k_jtv_batch(const __grid_constant__ Ba
 
 static size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 
-// z[2], v[2], p[3] and x, each [N] float4; or the multigrid solver's
+// v[2], p[3] and x, each [N] float4; or the multigrid solver's
 // buffers (multigrid.cu), whichever is larger.
 size_t solve_ws_bytes(const DevProblem& P)
 {
-    const size_t pcg = 8 * align256(sizeof(float4) * (size_t)P.N);
+    const size_t pcg = 6 * align256(sizeof(float4) * (size_t)P.N);
     const size_t mg = mg_ws_bytes(P);
     return pcg > mg ? pcg : mg;
 }
@@ -207,7 +207,6 @@ static SolveBufs carve(const DevProblem& P, void* ws)
     SolveBufs b;
     char* c = static_cast<char*>(ws);
     const size_t vec = align256(sizeof(float4) * (size_t)P.N);
-    for (float4*& v : b.z) { v = reinterpret_cast<float4*>(c); c += vec; }
     for (float4*& v : b.v) { v = reinterpret_cast<float4*>(c); c += vec; }
     for (float4*& v : b.p) { v = reinterpret_cast<float4*>(c); c += vec; }
     b.x = reinterpret_cast<float4*>(c);
@@ -219,7 +218,7 @@ static SolveBufs carve(const DevProblem& P, void* ws)
 template <int K>
 __device__ __forceinline__ void pcg_init_body(const DevProblem& P, int zc, const float* __restrict__ h,
                                               const float* __restrict__ w, const float* __restrict__ g,
-                                              const float* __restrict__ y, float4* __restrict__ z0,
+                                              const float* __restrict__ y, float4* __restrict__ p0,
                                               double tol2, WsHeader* hdr, double* resid, Reduce red,
                                               const VGrid& vg)
 {
@@ -268,7 +267,7 @@ __device__ __forceinline__ void pcg_init_body(const DevProblem& P, int zc, const
             float L[T], zz[K];
             pd &= cholesky_f32<K>(M, L);
             chol_apply<K>(L, r, zz);
-            z0[n] = pack4<K>(zz);
+            p0[n] = pack4<K>(zz);
             float vrz = 0.0f, vrr = 0.0f;
 #pragma unroll
             for (int k = 0; k < K; ++k) {
@@ -290,6 +289,7 @@ __device__ __forceinline__ void pcg_init_body(const DevProblem& P, int zc, const
         sc.alpha = 0.0;
         sc.alpha_prev = 0.0;
         sc.beta = 0.0;
+        sc.beta_prev = 0.0;
         sc.it = 0;
         sc.xcount = 0;
         sc.tol2 = tol2;
@@ -304,11 +304,11 @@ template <int K>
 __global__ void __launch_bounds__(kBlock) k_pcg_init(DevProblem P, int zc, const float* __restrict__ h,
                                                      const float* __restrict__ w,
                                                      const float* __restrict__ g,
-                                                     const float* __restrict__ y, float4* __restrict__ z0,
+                                                     const float* __restrict__ y, float4* __restrict__ p0,
                                                      double tol2, WsHeader* hdr, double* resid,
                                                      Reduce red)
 {
-    pcg_init_body<K>(P, zc, h, w, g, y, z0, tol2, hdr, resid, red, hw_grid());
+    pcg_init_body<K>(P, zc, h, w, g, y, p0, tol2, hdr, resid, red, hw_grid());
 }
 
 template <int K>
@@ -316,7 +316,7 @@ __global__ void __launch_bounds__(kBlock) k_pcg_init_batch(const __grid_constant
 {
     const int s = batch_subject(b.start, b.n);
     const InitArgs& a = b.a[s];
-    pcg_init_body<K>(a.P, a.zc, a.h, a.w, a.g, a.y, a.z0, a.tol2, a.hdr, a.resid, a.red,
+    pcg_init_body<K>(a.P, a.zc, a.h, a.w, a.g, a.y, a.p0, a.tol2, a.hdr, a.resid, a.red,
                      batch_grid(b.start[s], a.gx, a.gy, a.gz));
 }
 
@@ -324,36 +324,34 @@ __global__ void __launch_bounds__(kBlock) k_pcg_init_batch(const __grid_constant
 
 // Plain form of one PCG iteration (pcg_step.cuh): a thread per (x, y) column
 // marching a run of z planes; each neighbour's p_j is formed from its own
-// (z, v, p) read from memory.  Used for volumes or pointers the TMA kernel
+// p_{j-1}, v_{j-1} and p_{j-2} read from memory.  Used for volumes or pointers the TMA kernel
 // cannot take (nx not a multiple of 4, a volume smaller than a tile).
 template <int K, int MODE>
 __global__ void __launch_bounds__(kBlock) k_pcg_step(DevProblem P, int zc, int j, int want_rr,
                                                      const float* __restrict__ h,
                                                      const float* __restrict__ w,
-                                                     const float4* __restrict__ zin,
-                                                     const float4* __restrict__ vin,
                                                      const float4* __restrict__ pin,
+                                                     const float4* __restrict__ vin,
                                                      const float4* __restrict__ p2,
-                                                     float4* __restrict__ zout, float4* __restrict__ vout,
+                                                     float4* __restrict__ vout,
                                                      float4* __restrict__ pout, float4* __restrict__ xacc,
                                                      WsHeader* hdr, double* resid, Reduce red)
 {
     constexpr int T = K * (K + 1) / 2;
     constexpr bool first = MODE == kModeFirst;
-    __shared__ float s_alpha, s_alpha_prev, s_beta;
+    __shared__ StepScalars s_sc;
     __shared__ int s_done;
     const int tid = threadIdx.x + threadIdx.y * blockDim.x;
     if (tid == 0) {
         s_done = hdr->sc.done;
-        s_alpha = (float)hdr->sc.alpha;
-        s_alpha_prev = (float)hdr->sc.alpha_prev;
-        s_beta = (float)hdr->sc.beta;
+        s_sc = StepScalars{(float)hdr->sc.alpha, (float)hdr->sc.alpha_prev, (float)hdr->sc.beta,
+                           (float)hdr->sc.beta_prev};
     }
     __syncthreads();
     if (s_done) return;
     if (MODE >= kModeFold && tid == 0 && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0)
         hdr->sc.xcount = j;
-    const float alpha = s_alpha, alpha_prev = s_alpha_prev, beta = s_beta;
+    const StepScalars sc = s_sc;
     const long long sxy = (long long)P.nx * P.ny;
     const int x = blockIdx.x * kTileX + threadIdx.x;
     const int yy = blockIdx.y * kTileY + threadIdx.y;
@@ -362,7 +360,7 @@ __global__ void __launch_bounds__(kBlock) k_pcg_step(DevProblem P, int zc, int j
     float part[kStepSums] = {};
     auto point = [&](long long m, float (&zj)[K], float (&pj)[K]) {
         const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-        step_point<K, first>(alpha, beta, zin[m], first ? zero : vin[m], first ? zero : pin[m], zj, pj);
+        step_point<K, MODE>(sc, pin[m], first ? zero : vin[m], MODE >= kModeStep ? p2[m] : zero, zj, pj);
     };
     if (x < P.nx && yy < P.ny) {
         for (int z = z0p; z < z1p; ++z) {
@@ -387,12 +385,11 @@ __global__ void __launch_bounds__(kBlock) k_pcg_step(DevProblem P, int zc, int j
             for (int t = 0; t < T; ++t) hv[t] = __ldg(h + t * P.N + n);
             float v[K], sums[kStepSums];
             step_voxel<K>(P, e.c, zj, pj, [&](int m, int a) { return nb[m][a]; }, hv, want_rr, v, sums);
-            if (!first) zout[n] = pack4<K>(zj);
-            pout[n] = pack4<K>(pj);
+            if (!first) pout[n] = pack4<K>(pj);
             vout[n] = pack4<K>(v);
             if (MODE >= kModeFold) {
                 const float4 x0 = MODE == kModeFoldX ? xacc[n] : make_float4(0.f, 0.f, 0.f, 0.f);
-                xacc[n] = fold_x(x0, alpha_prev, p2[n], alpha, pin[n]);
+                xacc[n] = fold_x(x0, sc.alpha_prev, p2[n], sc.alpha, pin[n]);
             }
 #pragma unroll
             for (int i = 0; i < kStepSums; ++i) part[i] += sums[i];
@@ -541,6 +538,7 @@ cudaError_t launch_jtv(const DevProblem& P, const float* y, float* w, double* jt
 int step_mode(int j)
 {
     if (j == 0) return kModeFirst;
+    if (j == 1) return kModeSecond;
     if (j % 2) return kModeStep;
     return j == 2 ? kModeFold : kModeFoldX;
 }
@@ -551,13 +549,14 @@ static void launch_step_plain(const DevProblem& P, const StencilGrid& sg, int j,
                               double* resid, Reduce red, cudaStream_t st)
 {
     const int jm = j > 0 ? j - 1 : 0;
-    const float4 *zin = B.z[jm & 1], *vin = B.v[jm & 1], *pin = B.p[(j + 2) % 3], *p2 = B.p[(j + 1) % 3];
-    float4 *zout = B.z[j & 1], *vout = B.v[j & 1], *pout = B.p[j % 3];
+    const float4 *pin = B.p[jm % 3], *vin = B.v[jm & 1], *p2 = B.p[(j + 1) % 3];
+    float4 *vout = B.v[j & 1], *pout = B.p[j % 3];
 #define MPM_STEP_PLAIN(M)                                                                          \
-    k_pcg_step<K, M><<<sg.grid, sg.block, 0, st>>>(P, sg.zc, j, want_rr, h, w, zin, vin, pin, p2, zout, \
-                                                   vout, pout, B.x, hdr, resid, red)
+    k_pcg_step<K, M><<<sg.grid, sg.block, 0, st>>>(P, sg.zc, j, want_rr, h, w, pin, vin, p2, vout, pout, \
+                                                   B.x, hdr, resid, red)
     switch (step_mode(j)) {
     case kModeFirst: MPM_STEP_PLAIN(kModeFirst); break;
+    case kModeSecond: MPM_STEP_PLAIN(kModeSecond); break;
     case kModeStep: MPM_STEP_PLAIN(kModeStep); break;
     case kModeFold: MPM_STEP_PLAIN(kModeFold); break;
     default: MPM_STEP_PLAIN(kModeFoldX); break;
@@ -577,7 +576,7 @@ static cudaError_t solve_k(const DevProblem& P, int cg_iters, double tol_cg, con
     const double tol2 = tol_cg > 0.0 ? tol_cg * tol_cg : 0.0;
     {
         LaunchScope ls(MPM_KERNEL_PCG_INIT, st);
-        k_pcg_init<K><<<ig.grid, ig.block, 0, st>>>(P, ig.zc, h, w, g, y, B.z[0], tol2, hdr, resid, red);
+        k_pcg_init<K><<<ig.grid, ig.block, 0, st>>>(P, ig.zc, h, w, g, y, B.p[0], tol2, hdr, resid, red);
     }
     StepMaps maps;
     const int tile = tma_tile_choice(P);
@@ -604,18 +603,17 @@ cudaError_t tma_autotune(const DevProblem& P, void* solve_ws, WsHeader* hdr, Red
                          cudaStream_t st, int* best, float* ms)
 {
     *best = -1;
-    // Timed on zeroed operands carved from the solve workspace's eight vectors
-    // so that no buffer the launch writes is also read: iteration 3 reads z, v
-    // and p from vectors 0-2, writes z, v, p to 4-6; H and w alias the
-    // read-only vectors 0-3 (T N floats fit in 0-2 for K = 3, 4).
+    // Timed on zeroed operands carved from the solve workspace's six vectors
+    // so that no buffer the launch writes is also read: iteration 3 reads p_2,
+    // p_1 and v_2 from vectors 0-2 and writes p_3 and v_3 to 4 and 5; H and w
+    // alias the read-only vectors 0-3 (T N floats fit in 0-2 for K = 3, 4).
     const size_t vec = align256(sizeof(float4) * (size_t)P.N);
     char* c = static_cast<char*>(solve_ws);
     auto at = [&](int i) { return reinterpret_cast<float4*>(c + i * vec); };
     SolveBufs B;
-    B.z[0] = at(0); B.z[1] = at(4);
-    B.v[0] = at(1); B.v[1] = at(5);
-    B.p[2] = at(2); B.p[1] = at(3); B.p[0] = at(6);
-    B.x = at(7);
+    B.p[2] = at(0); B.p[1] = at(1); B.p[0] = at(4);
+    B.v[0] = at(2); B.v[1] = at(5);
+    B.x = at(3);       // not touched in iteration 3
     const float* h = reinterpret_cast<const float*>(at(0));
     const float* w = reinterpret_cast<const float*>(at(3));
     cudaError_t e;

@@ -2,15 +2,16 @@
 // TMA plane staging (sm_103a).  The per-voxel arithmetic is pcg_step.cuh's,
 // shared with the plain kernel k_pcg_step (stencil_kernels.cu).
 //
-// Iteration j reads z_{j-1}, v_{j-1} and p_{j-1} (with a one-voxel halo), the
-// JTV weights and H, and writes z_j, p_j and v_j once:
-//   z_j = z_{j-1} - alpha_{j-1} v_{j-1},  p_j = z_j + beta_{j-1} p_{j-1}
+// Iteration j reads p_{j-1}, v_{j-1} and p_{j-2} (with a one-voxel halo), the
+// JTV weights and H, and writes p_j and v_j once:
+//   z_j = (p_{j-1} - beta_{j-2} p_{j-2}) - alpha_{j-1} v_{j-1}
+//   p_j = z_j + beta_{j-1} p_{j-1}
 //   q_j = (H + L) p_j,  v_j = M^-1 q_j,  and the sums for alpha_j and beta_j.
 // A block owns a TX x TY tile and marches up a run of z planes.  Per plane
 // one thread issues bulk tensor copies into a ring of "raw" stages:
-//   z, v, p   (TX+2) x (TY+2) voxels of 4 floats at (x0 - 1, y0 - 1, z)
-//   w         (TX+8) x (TY+2) floats at (x0 - 4, y0 - 1, z)
-//   x, p_j-2  TX x TY voxels of 4 floats at (x0, y0, z) (even j >= 2, x fold)
+//   p, v, p_j-2  (TX+2) x (TY+2) voxels of 4 floats at (x0 - 1, y0 - 1, z)
+//   w            (TX+8) x (TY+2) floats at (x0 - 4, y0 - 1, z)
+//   x            TX x TY voxels of 4 floats at (x0, y0, z) (even j > 2, x fold)
 // and H (TX x TY x T floats, planar) into a second ring.  The solve's own
 // vectors hold 4 floats per voxel, so their boxes start 16-byte aligned at
 // any x; the planar w box starts at a multiple of 4 floats.  Boxes that leave
@@ -19,9 +20,9 @@
 //
 // The compute warps (one voxel per thread) take each plane in two phases:
 //   A  form z_j and p_j of the plane's points (the tile and its x / y halo,
-//      recomputed from the staged z, v, p) into a shared "formed" plane (a
-//      ring of three), write z_j and p_j of the tile and fold x; the raw
-//      stage is then released;
+//      recomputed from the staged p, v, p_{j-2}) into a shared "formed" plane
+//      (a ring of three), write p_j of the tile and fold x; the raw stage is
+//      then released;
 //   B  one plane behind A: q = (H + L) p_j from the formed plane (x / y
 //      neighbours) and the thread's own column (z neighbours, kept in
 //      registers), v = M^-1 q, r = M z_j, the voxel's terms of the sums.
@@ -68,31 +69,30 @@ int copy_withhold() { return g_withhold.load(std::memory_order_relaxed); }
 long long copy_wait_cycles() { return g_wait_cycles.load(std::memory_order_relaxed); }
 
 // Per tile shape: one compute thread per voxel plus a producer warp.  256-
-// voxel tiles run two blocks per SM with two raw stages in the x-fold
-// iterations (whose stages also hold the x and p_{j-2} tiles) and three in
-// the others; 512-voxel tiles one block per SM with three and four.
+// voxel tiles run two blocks per SM with three raw stages, and two H stages in
+// the x-fold iterations (whose raw stages also hold the x tile) or three in
+// the others; 512-voxel tiles one block per SM with three or four raw stages.
 template <int K, int TX, int TY, bool FOLD = true>
 struct StepLayout {
     static constexpr int VOX = TX * TY;                 // voxels per tile = compute threads
     static constexpr int WARPS = VOX / 32;              // compute warps
     static constexpr int THREADS = VOX + 32;            // plus the producer warp
     static constexpr int MINB = VOX >= 512 ? 1 : 2;     // resident blocks per SM aimed for
-    static constexpr int RS = (VOX >= 512 ? 3 : 2) + (FOLD ? 0 : 1);   // raw (z, v, p, w[, x, p_{j-2}]) stages
-    static constexpr int HS = FOLD ? 2 : 3;             // H stages
+    static constexpr int RS = VOX >= 512 && !FOLD ? 4 : 3;   // raw (p, v, p_{j-2}, w[, x]) stages
+    static constexpr int HS = VOX < 512 && FOLD ? 2 : 3;     // H stages
     static constexpr int T = K * (K + 1) / 2;
-    static constexpr int BX = TX + 2, BY = TY + 2;      // z / v / p box and formed plane (x from x0 - 1)
+    static constexpr int BX = TX + 2, BY = TY + 2;      // p / v / p_{j-2} box and formed plane (x from x0 - 1)
     static constexpr int WX = TX + 8;                   // w box (x from x0 - 4, 16-byte aligned)
     static constexpr int NH = 2 * (TX + TY);            // halo points of a formed plane
     static constexpr int a128(int b) { return (b + 127) / 128 * 128; }
     static constexpr int BOX_BYTES = BX * BY * 16, W_BYTES = WX * BY * 4;
     static constexpr int TILE_BYTES = TX * TY * 16, H_BYTES = T * TX * TY * 4;
-    static constexpr int Z_OFF = 0;
+    static constexpr int P_OFF = 0;
     static constexpr int V_OFF = a128(BOX_BYTES);
-    static constexpr int P_OFF = V_OFF + a128(BOX_BYTES);
-    static constexpr int W_OFF = P_OFF + a128(BOX_BYTES);
+    static constexpr int P2_OFF = V_OFF + a128(BOX_BYTES);
+    static constexpr int W_OFF = P2_OFF + a128(BOX_BYTES);
     static constexpr int X_OFF = W_OFF + a128(W_BYTES);
-    static constexpr int P2_OFF = X_OFF + a128(TILE_BYTES);
-    static constexpr int RAW = FOLD ? P2_OFF + a128(TILE_BYTES) : X_OFF;
+    static constexpr int RAW = FOLD ? X_OFF + a128(TILE_BYTES) : X_OFF;
     static constexpr int H_STAGE = a128(H_BYTES);
     static constexpr int SLOT = a128(BOX_BYTES);
     static constexpr int H_BASE = RS * RAW;
@@ -132,21 +132,21 @@ __device__ __forceinline__ void compute_warps_sync()
 // The rings and their phases run on from one item to the next.
 template <int K, int TX, int TY, int MODE>
 __device__ __forceinline__ void step_body(
-    const DevProblem& P, int nchunk, int j, int want_rr, const CUtensorMap* tz, const CUtensorMap* tv,
-    const CUtensorMap* tp, const CUtensorMap* tw, const CUtensorMap* th, const CUtensorMap* txm,
-    const CUtensorMap* tp2, float4* __restrict__ zout, float4* __restrict__ vout,
-    float4* __restrict__ pout, float4* __restrict__ xacc, WsHeader* hdr, double* resid, Reduce red,
-    long long wait_cycles, int withhold, const VGrid& vg)
+    const DevProblem& P, int nchunk, int j, int want_rr, const CUtensorMap* tp, const CUtensorMap* tv,
+    const CUtensorMap* tp2, const CUtensorMap* tw, const CUtensorMap* th, const CUtensorMap* txm,
+    float4* __restrict__ vout, float4* __restrict__ pout, float4* __restrict__ xacc, WsHeader* hdr,
+    double* resid, Reduce red, long long wait_cycles, int withhold, const VGrid& vg)
 {
     using L = StepLayout<K, TX, TY, (MODE >= kModeFold)>;
     constexpr int T = L::T;
     constexpr int kStepRaw = L::RS, kStepH = L::HS, kStepWarps = L::WARPS;
-    constexpr bool first = MODE == kModeFirst, fold = MODE >= kModeFold, readx = MODE == kModeFoldX;
+    constexpr bool first = MODE == kModeFirst, third = MODE >= kModeStep;   // third: p_{j-2} exists
+    constexpr bool fold = MODE >= kModeFold, readx = MODE == kModeFoldX;
     extern __shared__ unsigned char smem_raw[];
     __shared__ __align__(8) uint64_t raw_full[kStepRaw], raw_empty[kStepRaw];
     __shared__ __align__(8) uint64_t h_full[kStepH], h_empty[kStepH];
     __shared__ int s_done;
-    __shared__ float s_alpha, s_alpha_prev, s_beta;
+    __shared__ StepScalars s_sc;
     __shared__ volatile int s_fail;
     unsigned char* smem =
         reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~uintptr_t(127));
@@ -162,9 +162,8 @@ __device__ __forceinline__ void step_body(
 
     if (tid == 0) {
         s_done = hdr->sc.done;
-        s_alpha = (float)hdr->sc.alpha;
-        s_alpha_prev = (float)hdr->sc.alpha_prev;
-        s_beta = (float)hdr->sc.beta;
+        s_sc = StepScalars{(float)hdr->sc.alpha, (float)hdr->sc.alpha_prev, (float)hdr->sc.beta,
+                           (float)hdr->sc.beta_prev};
         s_fail = 0;
         for (int s = 0; s < kStepRaw; ++s) {
             mbar_init(smem_u32(&raw_full[s]), 1);
@@ -179,7 +178,7 @@ __device__ __forceinline__ void step_body(
     __syncthreads();
     if (s_done) return;                                   // the same in every block
     if (fold && tid == 0 && vg.bx == 0) hdr->sc.xcount = j;
-    const float alpha = s_alpha, alpha_prev = s_alpha_prev, beta = s_beta;
+    const StepScalars sc = s_sc;
 
     // Counters: c over the raw planes this block loads, e over its H planes
     // (one per plane it computes), both in order -> ring stage and phase.
@@ -213,19 +212,15 @@ __device__ __forceinline__ void step_body(
                     unsigned char* st = smem + s * L::RAW;
                     const uint32_t bar = smem_u32(&raw_full[s]);
                     uint32_t bytes = L::BOX_BYTES + L::W_BYTES;
-                    if (!first) bytes += 2 * L::BOX_BYTES;
-                    if (fold && inner) bytes += L::TILE_BYTES * (readx ? 2 : 1);
+                    if (!first) bytes += L::BOX_BYTES;
+                    if (third) bytes += L::BOX_BYTES;
+                    if (readx && inner) bytes += L::TILE_BYTES;
                     mbar_expect_tx(bar, bytes);
-                    tma_load_3d(smem_u32(st + L::Z_OFF), tz, 4 * (x0 - 1), y0 - 1, jj, bar);
-                    if (!first) {
-                        tma_load_3d(smem_u32(st + L::V_OFF), tv, 4 * (x0 - 1), y0 - 1, jj, bar);
-                        tma_load_3d(smem_u32(st + L::P_OFF), tp, 4 * (x0 - 1), y0 - 1, jj, bar);
-                    }
+                    tma_load_3d(smem_u32(st + L::P_OFF), tp, 4 * (x0 - 1), y0 - 1, jj, bar);
+                    if (!first) tma_load_3d(smem_u32(st + L::V_OFF), tv, 4 * (x0 - 1), y0 - 1, jj, bar);
+                    if (third) tma_load_3d(smem_u32(st + L::P2_OFF), tp2, 4 * (x0 - 1), y0 - 1, jj, bar);
                     tma_load_3d(smem_u32(st + L::W_OFF), tw, x0 - 4, y0 - 1, jj, bar);
-                    if (fold && inner) {
-                        tma_load_3d(smem_u32(st + L::P2_OFF), tp2, 4 * x0, y0, jj, bar);
-                        if (readx) tma_load_3d(smem_u32(st + L::X_OFF), txm, 4 * x0, y0, jj, bar);
-                    }
+                    if (readx && inner) tma_load_3d(smem_u32(st + L::X_OFF), txm, 4 * x0, y0, jj, bar);
                     raw_issued = c;
                     if (!inner) continue;
                     const int e = eb + (jj - za);
@@ -254,7 +249,7 @@ __device__ __forceinline__ void step_body(
             const int ja = max(za - 1, 0), jb = min(zb, nz - 1);
             const bool inside = x < nx && y < ny;
             const bool okxm = x > 0, okxp = x + 1 < nx, okym = y > 0, okyp = y + 1 < ny;
-            const int bc = (ty + 1) * L::BX + tx + 1;      // own point in a z / v / p box and formed plane
+            const int bc = (ty + 1) * L::BX + tx + 1;      // own point in a p / v / p_{j-2} box and formed plane
             const int wcc = (ty + 1) * L::WX + tx + 4;     // own point in a w box
             const int tc = ty * TX + tx;                   // own point in a tile box
             // own column: p_j of planes z - 1, z, z + 1, z_j of z and z + 1,
@@ -309,12 +304,12 @@ __device__ __forceinline__ void step_body(
                 if (ok) {
                     // Phase A: z_j and p_j of this plane
                     const unsigned char* st = smem + r_stage(c) * L::RAW;
-                    const float4* bz = reinterpret_cast<const float4*>(st + L::Z_OFF);
-                    const float4* bv = reinterpret_cast<const float4*>(st + L::V_OFF);
                     const float4* bp = reinterpret_cast<const float4*>(st + L::P_OFF);
+                    const float4* bv = reinterpret_cast<const float4*>(st + L::V_OFF);
+                    const float4* b2 = reinterpret_cast<const float4*>(st + L::P2_OFF);
                     const float* bw = reinterpret_cast<const float*>(st + L::W_OFF);
-                    const float4 p4 = first ? zero4 : bp[bc];
-                    step_point<K, first>(alpha, beta, bz[bc], first ? zero4 : bv[bc], p4, zn, pn);
+                    const float4 p4 = bp[bc], p24 = third ? b2[bc] : zero4;
+                    step_point<K, MODE>(sc, p4, first ? zero4 : bv[bc], p24, zn, pn);
                     wn = bw[wcc];
                     cxyn[0] = okxm ? (wn + bw[wcc - 1]) * P.ihx2 : 0.f;
                     cxyn[1] = okxp ? (wn + bw[wcc + 1]) * P.ihx2 : 0.f;
@@ -331,18 +326,16 @@ __device__ __forceinline__ void step_body(
                             else if (tid < 2 * TX + TY) hb = (tid - 2 * TX + 1) * L::BX;
                             else hb = (tid - 2 * TX - TY + 1) * L::BX + TX + 1;
                             float hzj[K], hpj[K];
-                            step_point<K, first>(alpha, beta, bz[hb], first ? zero4 : bv[hb],
-                                                 first ? zero4 : bp[hb], hzj, hpj);
+                            step_point<K, MODE>(sc, bp[hb], first ? zero4 : bv[hb], third ? b2[hb] : zero4,
+                                                hzj, hpj);
                             fp[hb] = pack4<K>(hpj);
                         }
                         if (inside) {
                             const long long n = col + sxy * jj;
-                            if (!first) zout[n] = pack4<K>(zn);
-                            pout[n] = pack4<K>(pn);
+                            if (!first) pout[n] = pack4<K>(pn);
                             if (fold) {
                                 const float4* bx = reinterpret_cast<const float4*>(st + L::X_OFF);
-                                const float4* b2 = reinterpret_cast<const float4*>(st + L::P2_OFF);
-                                xacc[n] = fold_x(readx ? bx[tc] : zero4, alpha_prev, b2[tc], alpha, p4);
+                                xacc[n] = fold_x(readx ? bx[tc] : zero4, sc.alpha_prev, p24, sc.alpha, p4);
                             }
                         }
                     }
@@ -397,16 +390,15 @@ __device__ __forceinline__ void step_body(
 
 template <int K, int TX, int TY, int MODE>
 __global__ void __launch_bounds__(StepLayout<K, TX, TY>::THREADS, StepLayout<K, TX, TY>::MINB) k_pcg_step_tma(
-    DevProblem P, int nchunk, int j, int want_rr, const __grid_constant__ CUtensorMap tz,
-    const __grid_constant__ CUtensorMap tv, const __grid_constant__ CUtensorMap tp,
+    DevProblem P, int nchunk, int j, int want_rr, const __grid_constant__ CUtensorMap tp,
+    const __grid_constant__ CUtensorMap tv, const __grid_constant__ CUtensorMap tp2,
     const __grid_constant__ CUtensorMap tw, const __grid_constant__ CUtensorMap th,
-    const __grid_constant__ CUtensorMap txm, const __grid_constant__ CUtensorMap tp2,
-    float4* __restrict__ zout, float4* __restrict__ vout, float4* __restrict__ pout,
+    const __grid_constant__ CUtensorMap txm, float4* __restrict__ vout, float4* __restrict__ pout,
     float4* __restrict__ xacc, WsHeader* hdr, double* resid, Reduce red, long long wait_cycles,
     int withhold)
 {
-    step_body<K, TX, TY, MODE>(P, nchunk, j, want_rr, &tz, &tv, &tp, &tw, &th, &txm, &tp2, zout, vout,
-                               pout, xacc, hdr, resid, red, wait_cycles, withhold, hw_grid());
+    step_body<K, TX, TY, MODE>(P, nchunk, j, want_rr, &tp, &tv, &tp2, &tw, &th, &txm, vout, pout, xacc,
+                               hdr, resid, red, wait_cycles, withhold, hw_grid());
 }
 
 // Several subjects in one launch (mpm_fit_batch with opts.graph = 2).
@@ -416,9 +408,8 @@ __global__ void __launch_bounds__(StepLayout<K, TX, TY>::THREADS, StepLayout<K, 
 {
     const int s = batch_subject(b.start, b.n);
     const StepArgs& a = b.a[s];
-    step_body<K, TX, TY, MODE>(a.P, a.nchunk, a.j, a.want_rr, &a.tz, &a.tv, &a.tp, &a.tw, &a.th, &a.tx,
-                               &a.tp2, a.zout, a.vout, a.pout, a.xacc, a.hdr, a.resid, a.red,
-                               a.wait_cycles, a.withhold, batch_grid(b.start[s], b.start[s + 1] - b.start[s], 1, 1));
+    step_body<K, TX, TY, MODE>(a.P, a.nchunk, a.j, a.want_rr, &a.tp, &a.tv, &a.tp2, &a.tw, &a.th, &a.tx,
+                               a.vout, a.pout, a.xacc, a.hdr, a.resid, a.red, a.wait_cycles, a.withhold, batch_grid(b.start[s], b.start[s + 1] - b.start[s], 1, 1));
 }
 
 // ------------------------------------------------------------------ host
@@ -489,7 +480,6 @@ bool make_step_maps(const DevProblem& P, const float* h, const float* w, const S
     if (P.nx % 4 != 0 || P.nx < WX || P.ny < BY) return false;
     uintptr_t any = reinterpret_cast<uintptr_t>(h) | reinterpret_cast<uintptr_t>(w) |
                     reinterpret_cast<uintptr_t>(B.x);
-    for (float4* v : B.z) any |= reinterpret_cast<uintptr_t>(v);
     for (float4* v : B.v) any |= reinterpret_cast<uintptr_t>(v);
     for (float4* v : B.p) any |= reinterpret_cast<uintptr_t>(v);
     if (any % 16) return false;
@@ -511,10 +501,8 @@ bool make_step_maps(const DevProblem& P, const float* h, const float* w, const S
     bool ok = encode(&out->w, w, 3, d3, s3, wbox) && encode(&out->h, h, 4, dh, sh, hbox) &&
               encode(&out->x, f(B.x), 3, da, sa, tilebox);
     for (int i = 0; i < 2 && ok; ++i)
-        ok = encode(&out->z[i], f(B.z[i]), 3, da, sa, halo) && encode(&out->v[i], f(B.v[i]), 3, da, sa, halo);
-    for (int i = 0; i < 3 && ok; ++i)
-        ok = encode(&out->p[i], f(B.p[i]), 3, da, sa, halo) &&
-             encode(&out->p2[i], f(B.p[i]), 3, da, sa, tilebox);
+        ok = encode(&out->v[i], f(B.v[i]), 3, da, sa, halo);
+    for (int i = 0; i < 3 && ok; ++i) ok = encode(&out->p[i], f(B.p[i]), 3, da, sa, halo);
     out->B = B;
     out->tile = tile;
     return ok;
@@ -535,8 +523,8 @@ static cudaError_t launch_step_m(const DevProblem& P, int nchunk, dim3 grid, con
     }
     const int jm = j > 0 ? j - 1 : 0;
     k_pcg_step_tma<K, TX, TY, MODE><<<grid, dim3(L::THREADS, 1, 1), L::SMEM, st>>>(
-        P, nchunk, j, want_rr, m.z[jm & 1], m.v[jm & 1], m.p[(j + 2) % 3], m.w, m.h, m.x,
-        m.p2[(j + 1) % 3], m.B.z[j & 1], m.B.v[j & 1], m.B.p[j % 3], m.B.x, hdr, resid, red,
+        P, nchunk, j, want_rr, m.p[jm % 3], m.v[jm & 1], m.p[(j + 1) % 3], m.w, m.h, m.x,
+        m.B.v[j & 1], m.B.p[j % 3], m.B.x, hdr, resid, red,
         g_wait_cycles.load(std::memory_order_relaxed), g_withhold.load(std::memory_order_relaxed));
     return cudaGetLastError();
 }
@@ -548,6 +536,7 @@ static cudaError_t launch_step_k(const DevProblem& P, int nchunk, dim3 grid, con
 {
     switch (mode) {
     case kModeFirst: return launch_step_m<K, TX, TY, kModeFirst>(P, nchunk, grid, m, j, want_rr, hdr, resid, red, st);
+    case kModeSecond: return launch_step_m<K, TX, TY, kModeSecond>(P, nchunk, grid, m, j, want_rr, hdr, resid, red, st);
     case kModeStep: return launch_step_m<K, TX, TY, kModeStep>(P, nchunk, grid, m, j, want_rr, hdr, resid, red, st);
     case kModeFold: return launch_step_m<K, TX, TY, kModeFold>(P, nchunk, grid, m, j, want_rr, hdr, resid, red, st);
     default: return launch_step_m<K, TX, TY, kModeFoldX>(P, nchunk, grid, m, j, want_rr, hdr, resid, red, st);
@@ -559,18 +548,16 @@ StepArgs step_args(const DevProblem& P, const StepMaps& m, int nchunk, int j, in
 {
     StepArgs a;
     const int jm = j > 0 ? j - 1 : 0;
-    a.tz = m.z[jm & 1];
+    a.tp = m.p[jm % 3];
     a.tv = m.v[jm & 1];
-    a.tp = m.p[(j + 2) % 3];
+    a.tp2 = m.p[(j + 1) % 3];
     a.tw = m.w;
     a.th = m.h;
     a.tx = m.x;
-    a.tp2 = m.p2[(j + 1) % 3];
     a.P = P;
     a.nchunk = nchunk;
     a.j = j;
     a.want_rr = want_rr;
-    a.zout = m.B.z[j & 1];
     a.vout = m.B.v[j & 1];
     a.pout = m.B.p[j % 3];
     a.xacc = m.B.x;
@@ -603,6 +590,7 @@ static cudaError_t launch_step_batch_k(int mode, const Batch<StepArgs>& b, cudaS
 {
     switch (mode) {
     case kModeFirst: return launch_step_batch_m<K, TX, TY, kModeFirst>(b, st);
+    case kModeSecond: return launch_step_batch_m<K, TX, TY, kModeSecond>(b, st);
     case kModeStep: return launch_step_batch_m<K, TX, TY, kModeStep>(b, st);
     case kModeFold: return launch_step_batch_m<K, TX, TY, kModeFold>(b, st);
     default: return launch_step_batch_m<K, TX, TY, kModeFoldX>(b, st);
@@ -701,10 +689,12 @@ static cudaError_t prime_one()
                                      step_smem_max<K, TX, TY>());
     };
     set(reinterpret_cast<const void*>(k_pcg_step_tma<K, TX, TY, kModeFirst>));
+    set(reinterpret_cast<const void*>(k_pcg_step_tma<K, TX, TY, kModeSecond>));
     set(reinterpret_cast<const void*>(k_pcg_step_tma<K, TX, TY, kModeStep>));
     set(reinterpret_cast<const void*>(k_pcg_step_tma<K, TX, TY, kModeFold>));
     set(reinterpret_cast<const void*>(k_pcg_step_tma<K, TX, TY, kModeFoldX>));
     set(reinterpret_cast<const void*>(k_pcg_step_tma_batch<K, TX, TY, kModeFirst>));
+    set(reinterpret_cast<const void*>(k_pcg_step_tma_batch<K, TX, TY, kModeSecond>));
     set(reinterpret_cast<const void*>(k_pcg_step_tma_batch<K, TX, TY, kModeStep>));
     set(reinterpret_cast<const void*>(k_pcg_step_tma_batch<K, TX, TY, kModeFold>));
     set(reinterpret_cast<const void*>(k_pcg_step_tma_batch<K, TX, TY, kModeFoldX>));
