@@ -195,8 +195,30 @@ __device__ __forceinline__ VGrid batch_grid(unsigned first, unsigned gx, unsigne
     return VGrid{v % gx, (v / gx) % gy, v / (gx * gy), gx, gy, gz};
 }
 
+// The first nv (<= NV) pairs of a warp's lanes combined, side by side (lane 0
+// holds the results).
+template <int NV>
+__device__ __forceinline__ void warp_combine(Acc (&a)[NV], int nv = NV)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+#pragma unroll
+        for (int j = 0; j < NV; ++j) {
+            if (j < nv) {
+                Acc b;
+                b.hi = __shfl_down_sync(0xffffffffu, a[j].hi, o);
+                b.lo = __shfl_down_sync(0xffffffffu, a[j].lo, o);
+                a[j].add(b);
+            }
+        }
+    }
+}
+
+constexpr int kMaxWarps = 20;      // of a reducing block (640 threads)
+
 // Last-block-done reduction of the first nv (<= NV) values per block.  Every
-// thread calls it with its own compensated partials; returns true in exactly
+// thread calls it; of(j, w), w < nw, is warp w's compensated pair of value j in
+// shared memory (read after a block barrier).  Returns true in exactly
 // one block (the last to arrive), where out[j] (valid in thread 0) holds the
 // grid-wide sums in a fixed summation order.  The counter is reset for the
 // next launch.  The grid is the block's launch, or its subject's share of a
@@ -210,44 +232,23 @@ __device__ __forceinline__ VGrid batch_grid(unsigned first, unsigned gx, unsigne
 // float64 (2 lanes per clock and SM).  One value after another, with a
 // block-wide float64 sum and two barriers each, a PCG iteration took 29.3 us at
 // 64^3 and 290 us at 176x240x256 where this form took 20.6 and 280 us.
-template <int NV>
-__device__ __forceinline__ bool grid_reduce(const Acc (&v)[NV], Reduce red, double (&out)[NV],
-                                            const VGrid& vg, int nv = NV)
+template <int NV, class Of>
+__device__ __forceinline__ bool grid_reduce_warps(Of of, int nw, Reduce red, double (&out)[NV],
+                                                  const VGrid& vg, int nv)
 {
-    constexpr int kMaxWarps = 20;      // blocks of at most 640 threads
-    __shared__ float sh_hi[NV][kMaxWarps], sh_lo[NV][kMaxWarps];
     __shared__ double sh_part[kMaxWarps > NV ? kMaxWarps : NV];
     __shared__ bool am_last;
     const int tid = threadIdx.x + threadIdx.y * blockDim.x;
-    const int nw = (int)(blockDim.x * blockDim.y + 31) >> 5;
     const int warp = tid >> 5, lane = tid & 31;
     const unsigned bid = vg.id();
     const unsigned nblocks = vg.count();
-    Acc a[NV];
-#pragma unroll
-    for (int j = 0; j < NV; ++j) a[j] = v[j];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-#pragma unroll
-        for (int j = 0; j < NV; ++j) {
-            if (j < nv) {
-                Acc b;
-                b.hi = __shfl_down_sync(0xffffffffu, a[j].hi, o);
-                b.lo = __shfl_down_sync(0xffffffffu, a[j].lo, o);
-                a[j].add(b);
-            }
-        }
-    }
-    if (lane == 0) {
-#pragma unroll
-        for (int j = 0; j < NV; ++j) {
-            sh_hi[j][warp] = a[j].hi;
-            sh_lo[j][warp] = a[j].lo;
-        }
-    }
     __syncthreads();
     for (int j = warp; j < nv; j += nw) {
-        double s = lane < nw ? (double)sh_hi[j][lane] + (double)sh_lo[j][lane] : 0.0;
+        double s = 0.0;
+        if (lane < nw) {
+            const Acc a = of(j, lane);
+            s = (double)a.hi + (double)a.lo;
+        }
         for (int o = nw > 16 ? 16 : nw > 8 ? 8 : 4; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
         if (lane == 0) red.partials[(size_t)j * kMaxBlocks + bid] = s;
     }
@@ -291,6 +292,25 @@ __device__ __forceinline__ bool grid_reduce(const Acc (&v)[NV], Reduce red, doub
         *red.counter = 0u;
     }
     return true;
+}
+
+// The same from every thread's own compensated partials.
+template <int NV>
+__device__ __forceinline__ bool grid_reduce(const Acc (&v)[NV], Reduce red, double (&out)[NV],
+                                            const VGrid& vg, int nv = NV)
+{
+    __shared__ Acc sh[kMaxWarps][NV];
+    const int tid = threadIdx.x + threadIdx.y * blockDim.x;
+    const int nw = (int)(blockDim.x * blockDim.y + 31) >> 5;
+    Acc a[NV];
+#pragma unroll
+    for (int j = 0; j < NV; ++j) a[j] = v[j];
+    warp_combine<NV>(a, nv);
+    if ((tid & 31) == 0) {
+#pragma unroll
+        for (int j = 0; j < NV; ++j) sh[tid >> 5][j] = a[j];
+    }
+    return grid_reduce_warps<NV>([&](int j, int w) { return sh[w][j]; }, nw, red, out, vg, nv);
 }
 
 template <int NV>

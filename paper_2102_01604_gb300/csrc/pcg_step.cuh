@@ -151,6 +151,37 @@ enum : int {
 // Sums reduced by every iteration, in this order.
 enum : int { kSumPQ, kSumZQ, kSumVQ, kSumZR, kSumRR, kSumRQ, kSumQQ, kStepSums };
 
+// The four maps of a voxel as two pairs, for the paired float32 instructions
+// (each lane rounds as its scalar form): the iteration's instruction issue is
+// the bound next to HBM, and its per-map arithmetic pairs without moves.
+struct Maps {
+    float2 a, b;
+    __device__ __forceinline__ Maps() {}
+    __device__ __forceinline__ Maps(float2 x, float2 y) : a(x), b(y) {}
+    __device__ __forceinline__ Maps(const float4& v) : a(make_float2(v.x, v.y)), b(make_float2(v.z, v.w)) {}
+    __device__ __forceinline__ float operator[](int k) const
+    {
+        return k == 0 ? a.x : k == 1 ? a.y : k == 2 ? b.x : b.y;
+    }
+    __device__ __forceinline__ float4 vec() const { return make_float4(a.x, a.y, b.x, b.y); }
+};
+
+__device__ __forceinline__ float2 twice(float v) { return make_float2(v, v); }
+
+// s v + w, and v - w.
+__device__ __forceinline__ Maps axpy(float s, const Maps& v, const Maps& w)
+{
+    return Maps(__ffma2_rn(twice(s), v.a, w.a), __ffma2_rn(twice(s), v.b, w.b));
+}
+__device__ __forceinline__ Maps minus(const Maps& v, const Maps& w) { return axpy(-1.0f, w, v); }
+
+// sum_k v_k w_k (the padding of K = 3 is zero).
+__device__ __forceinline__ float dot(const Maps& v, const Maps& w)
+{
+    const float2 s = __ffma2_rn(v.b, w.b, __fmul2_rn(v.a, w.a));
+    return s.x + s.y;
+}
+
 // The scalars an iteration starts from: alpha_{j-1}, alpha_{j-2}, beta_{j-1}
 // and beta_{j-2} (those that exist).
 struct StepScalars {
@@ -159,63 +190,53 @@ struct StepScalars {
 
 // z_j and p_j of one point from p1 = p_{j-1}, v = v_{j-1} and p2 = p_{j-2}
 // (j = 0: p1 is p_0 and v, p2 are not read; j = 1: p2 is not read).
-template <int K, int MODE>
-__device__ __forceinline__ void step_point(const StepScalars& s, const float4& p14, const float4& v4,
-                                           const float4& p24, float (&zj)[K], float (&pj)[K])
+template <int MODE>
+__device__ __forceinline__ void step_point(const StepScalars& s, const Maps& p1, const Maps& v,
+                                           const Maps& p2, Maps& zj, Maps& pj)
 {
-    float p1[K], v[K], p2[K];
-    unpack4<K>(p14, p1);
-    unpack4<K>(v4, v);
-    unpack4<K>(p24, p2);
-#pragma unroll
-    for (int a = 0; a < K; ++a) {
-        const float z = MODE >= kModeStep ? fmaf(-s.beta_prev, p2[a], p1[a]) : p1[a];   // z_{j-1}
-        zj[a] = MODE == kModeFirst ? z : fmaf(-s.alpha, v[a], z);
-        pj[a] = MODE == kModeFirst ? z : fmaf(s.beta, p1[a], zj[a]);
-    }
+    const Maps z = MODE >= kModeStep ? axpy(-s.beta_prev, p2, p1) : p1;   // z_{j-1}
+    zj = MODE == kModeFirst ? z : axpy(-s.alpha, v, z);
+    pj = MODE == kModeFirst ? z : axpy(s.beta, p1, zj);
 }
 
 // x after folding in the two latest directions, in the order of two single
 // updates: x + alpha_{j-2} p_{j-2}, then + alpha_{j-1} p_{j-1} (all four
 // components; the padding of K = 3 stays zero).
-__device__ __forceinline__ float4 fold_x(const float4& x, float alpha_prev, const float4& p2, float alpha,
-                                         const float4& p1)
+__device__ __forceinline__ Maps fold_x(const Maps& x, const StepScalars& s, const Maps& p2, const Maps& p1)
 {
-    return make_float4(fmaf(alpha, p1.x, fmaf(alpha_prev, p2.x, x.x)),
-                       fmaf(alpha, p1.y, fmaf(alpha_prev, p2.y, x.y)),
-                       fmaf(alpha, p1.z, fmaf(alpha_prev, p2.z, x.z)),
-                       fmaf(alpha, p1.w, fmaf(alpha_prev, p2.w, x.w)));
+    return axpy(s.alpha, p1, axpy(s.alpha_prev, p2, x));
 }
 
 // One voxel of iteration j: q = (H + L) p_j with the weighted 7-point stencil
 //     (L p)_k = lambda_k sum_m c_m (p_k[n] - p_k[m]),  c_m = (w_n + w_m) / h^2
 // (c_m = 0 for neighbours outside the volume, whose values nb then only need
-// to be finite), v = M^-1 q, r = M z_j, and the voxel's terms of the sums.
-// nb(m, a) returns p_j of map a at neighbour m (order x-, x+, y-, y+, z-, z+).
+// to be finite), v = M^-1 q, r = M z_j, and the voxel's terms added to part.
+// nb(m) returns p_j at neighbour m (order x-, x+, y-, y+, z-, z+).
 template <int K, class NB>
-__device__ __forceinline__ void step_voxel(const DevProblem& P, const float (&c)[6],
-                                           const float (&zj)[K], const float (&pj)[K], NB nb,
-                                           const float (&hv)[K * (K + 1) / 2], bool resid,
-                                           float (&v)[K], float (&sums)[kStepSums])
+__device__ __forceinline__ void step_voxel(const DevProblem& P, const float (&c)[6], const Maps& zj,
+                                           const Maps& pj, NB nb, const float (&hv)[K * (K + 1) / 2],
+                                           bool resid, Maps& v, float (&part)[kStepSums])
 {
     float M[K][K];
     precond_block<K>(P, hv, edge_sum(c), M);
+    Maps s;
+    {
+        const Maps d = minus(pj, nb(0));
+        s = Maps(__fmul2_rn(twice(c[0]), d.a), __fmul2_rn(twice(c[0]), d.b));
+    }
+#pragma unroll
+    for (int m = 1; m < 6; ++m) s = axpy(c[m], minus(pj, nb(m)), s);
     float q[K];
 #pragma unroll
     for (int a = 0; a < K; ++a) {
-        const float pa = pj[a];
-        float s = c[0] * (pa - nb(0, a));
-#pragma unroll
-        for (int m = 1; m < 6; ++m) s = fmaf(c[m], pa - nb(m, a), s);
-        float acc = P.lambda[a] * s;
+        float acc = P.lambda[a] * s[a];
 #pragma unroll
         for (int b = 0; b < K; ++b) acc = fmaf(hv[a < b ? tri(K, a, b) : tri(K, b, a)], pj[b], acc);
         q[a] = acc;
     }
-    float L[K * (K + 1) / 2];
+    float L[K * (K + 1) / 2], vk[K], r[K];
     cholesky_f32<K>(M, L);
-    chol_apply<K>(L, q, v);
-    float r[K];
+    chol_apply<K>(L, q, vk);
 #pragma unroll
     for (int a = 0; a < K; ++a) {
         float acc = M[a][0] * zj[0];
@@ -223,33 +244,17 @@ __device__ __forceinline__ void step_voxel(const DevProblem& P, const float (&c)
         for (int b = 1; b < K; ++b) acc = fmaf(M[a][b], zj[b], acc);
         r[a] = acc;
     }
-    float pq = pj[0] * q[0], zq = zj[0] * q[0], vq = v[0] * q[0], zr = zj[0] * r[0];
-#pragma unroll
-    for (int a = 1; a < K; ++a) {
-        pq = fmaf(pj[a], q[a], pq);
-        zq = fmaf(zj[a], q[a], zq);
-        vq = fmaf(v[a], q[a], vq);
-        zr = fmaf(zj[a], r[a], zr);
-    }
-    sums[kSumPQ] = pq;
-    sums[kSumZQ] = zq;
-    sums[kSumVQ] = vq;
-    sums[kSumZR] = zr;
-    float rr = 0.0f, rq = 0.0f, qq = 0.0f;
+    const Maps q4 = Maps(pack4<K>(q)), r4 = Maps(pack4<K>(r));
+    v = Maps(pack4<K>(vk));
+    part[kSumPQ] += dot(pj, q4);
+    part[kSumZQ] += dot(zj, q4);
+    part[kSumVQ] += dot(v, q4);
+    part[kSumZR] += dot(zj, r4);
     if (resid) {
-        rr = r[0] * r[0];
-        rq = r[0] * q[0];
-        qq = q[0] * q[0];
-#pragma unroll
-        for (int a = 1; a < K; ++a) {
-            rr = fmaf(r[a], r[a], rr);
-            rq = fmaf(r[a], q[a], rq);
-            qq = fmaf(q[a], q[a], qq);
-        }
+        part[kSumRR] += dot(r4, r4);
+        part[kSumRQ] += dot(r4, q4);
+        part[kSumQQ] += dot(q4, q4);
     }
-    sums[kSumRR] = rr;
-    sums[kSumRQ] = rq;
-    sums[kSumQQ] = qq;
 }
 
 // Scalars of iteration j from its reduced sums (the last block of the launch):

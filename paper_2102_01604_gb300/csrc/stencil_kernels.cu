@@ -358,9 +358,9 @@ __global__ void __launch_bounds__(kBlock) k_pcg_step(DevProblem P, int zc, int j
     const int z0p = blockIdx.z * zc;
     const int z1p = min(P.nz, z0p + zc);
     float part[kStepSums] = {};
-    auto point = [&](long long m, float (&zj)[K], float (&pj)[K]) {
-        const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-        step_point<K, MODE>(sc, pin[m], first ? zero : vin[m], MODE >= kModeStep ? p2[m] : zero, zj, pj);
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    auto point = [&](long long m, Maps& zj, Maps& pj) {
+        step_point<MODE>(sc, pin[m], first ? zero : vin[m], MODE >= kModeStep ? p2[m] : zero, zj, pj);
     };
     if (x < P.nx && yy < P.ny) {
         for (int z = z0p; z < z1p; ++z) {
@@ -368,31 +368,22 @@ __global__ void __launch_bounds__(kBlock) k_pcg_step(DevProblem P, int zc, int j
             const float wn = __ldg(w + n);
             Edges e;
             make_edges(P, x, yy, z, n, w, wn, e);
-            float zj[K], pj[K], nb[6][K];
+            Maps zj, pj, nb[6];
             point(n, zj, pj);
 #pragma unroll
             for (int m = 0; m < 6; ++m) {
-                float zm[K];
-                if (e.ok[m]) {
-                    point(n + e.off[m], zm, nb[m]);
-                } else {
-#pragma unroll
-                    for (int a = 0; a < K; ++a) nb[m][a] = pj[a];
-                }
+                Maps zm;
+                if (e.ok[m]) point(n + e.off[m], zm, nb[m]);
+                else nb[m] = pj;
             }
             float hv[T];
 #pragma unroll
             for (int t = 0; t < T; ++t) hv[t] = __ldg(h + t * P.N + n);
-            float v[K], sums[kStepSums];
-            step_voxel<K>(P, e.c, zj, pj, [&](int m, int a) { return nb[m][a]; }, hv, want_rr, v, sums);
-            if (!first) pout[n] = pack4<K>(pj);
-            vout[n] = pack4<K>(v);
-            if (MODE >= kModeFold) {
-                const float4 x0 = MODE == kModeFoldX ? xacc[n] : make_float4(0.f, 0.f, 0.f, 0.f);
-                xacc[n] = fold_x(x0, sc.alpha_prev, p2[n], sc.alpha, pin[n]);
-            }
-#pragma unroll
-            for (int i = 0; i < kStepSums; ++i) part[i] += sums[i];
+            Maps v;
+            step_voxel<K>(P, e.c, zj, pj, [&](int m) { return nb[m]; }, hv, want_rr, v, part);
+            if (!first) pout[n] = pj.vec();
+            vout[n] = v.vec();
+            if (MODE >= kModeFold) xacc[n] = fold_x(MODE == kModeFoldX ? xacc[n] : zero, sc, p2[n], pin[n]).vec();
         }
     }
     Acc acc[kStepSums];

@@ -69,17 +69,19 @@ int copy_withhold() { return g_withhold.load(std::memory_order_relaxed); }
 long long copy_wait_cycles() { return g_wait_cycles.load(std::memory_order_relaxed); }
 
 // Per tile shape: one compute thread per voxel plus a producer warp.  256-
-// voxel tiles run two blocks per SM with three raw stages, and two H stages in
-// the x-fold iterations (whose raw stages also hold the x tile) or three in
-// the others; 512-voxel tiles one block per SM with three or four raw stages.
+// voxel tiles run two blocks per SM with three H stages and three raw stages,
+// in the x-fold iterations (whose raw stages also hold the x tile) two; 512-
+// voxel tiles one block per SM.  Solve of 176x240x256, 30 iterations: 7.46 ms;
+// with three raw stages in the fold iterations too 7.55, three raw and two H
+// stages there 7.86, four raw and two H in the others 8.18.
 template <int K, int TX, int TY, bool FOLD = true>
 struct StepLayout {
     static constexpr int VOX = TX * TY;                 // voxels per tile = compute threads
     static constexpr int WARPS = VOX / 32;              // compute warps
     static constexpr int THREADS = VOX + 32;            // plus the producer warp
     static constexpr int MINB = VOX >= 512 ? 1 : 2;     // resident blocks per SM aimed for
-    static constexpr int RS = VOX >= 512 && !FOLD ? 4 : 3;   // raw (p, v, p_{j-2}, w[, x]) stages
-    static constexpr int HS = VOX < 512 && FOLD ? 2 : 3;     // H stages
+    static constexpr int RS = VOX >= 512 ? (FOLD ? 3 : 4) : (FOLD ? 2 : 3);   // raw (p, v, p_{j-2}, w[, x]) stages
+    static constexpr int HS = 3;                        // H stages
     static constexpr int T = K * (K + 1) / 2;
     static constexpr int BX = TX + 2, BY = TY + 2;      // p / v / p_{j-2} box and formed plane (x from x0 - 1)
     static constexpr int WX = TX + 8;                   // w box (x from x0 - 4, 16-byte aligned)
@@ -179,18 +181,21 @@ __device__ __forceinline__ void step_body(
     if (s_done) return;                                   // the same in every block
     if (fold && tid == 0 && vg.bx == 0) hdr->sc.xcount = j;
     const StepScalars sc = s_sc;
+    const int sums = want_rr ? kStepSums : kSumRR;        // sums reduced by this launch
 
-    // Counters: c over the raw planes this block loads, e over its H planes
-    // (one per plane it computes), both in order -> ring stage and phase.
+    // Planes are counted in order, c over the raw planes this block loads and
+    // e over its H planes (one per plane it computes): count -> ring stage and
+    // phase.  The compute warps step a stage and a phase bit along instead.
     auto r_stage = [](int c) { return (int)((unsigned)c % (unsigned)kStepRaw); };
     auto r_phase = [](int c) { return (uint32_t)(((unsigned)c / (unsigned)kStepRaw) & 1u); };
     auto h_stage = [](int e) { return (int)((unsigned)e % (unsigned)kStepH); };
     auto h_phase = [](int e) { return (uint32_t)(((unsigned)e / (unsigned)kStepH) & 1u); };
-    auto formed = [&](int c) {
-        return reinterpret_cast<float4*>(smem + L::S_BASE + ((unsigned)c % 3u) * L::SLOT);
-    };
 
-    Acc acc[kStepSums];
+    // A warp's sums over its items so far: kept here and not in every thread's
+    // registers (nine warps a block leave 96, which the marching state fills).
+    __shared__ Acc s_acc[L::WARPS][kStepSums];
+    if (lane < kStepSums && !producer) s_acc[warp][lane] = Acc();
+    __syncwarp();
     int raw_issued = -1, h_issued = -1;   // last counters issued (producer lane 0)
     if (producer) {
         if (lane == 0 && !withhold) {
@@ -240,8 +245,29 @@ __device__ __forceinline__ void step_body(
             }
         }
     } else {
-        const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
-        int cb = 0, eb = 0;
+        const Maps zero = Maps(make_float4(0.f, 0.f, 0.f, 0.f));
+        const uint32_t rf0 = smem_u32(&raw_full[0]), re0 = smem_u32(&raw_empty[0]);
+        const uint32_t hf0 = smem_u32(&h_full[0]), he0 = smem_u32(&h_empty[0]);
+        unsigned rs = 0, hs = 0, fs = 0;           // next raw, H and formed stage
+        uint32_t rph = 0, hph = 0;                 // phase of the raw and H ring's current turn
+        bool bad = false;                          // a wait of this thread gave up
+        // a wait that is over costs one try; s_fail is read only where it is not
+        auto wait = [&](uint32_t bar, uint32_t parity) {
+            if (bad || mbar_try_wait(bar, parity)) return;
+            if (s_fail || !mbar_wait(bar, parity, wait_cycles)) {
+                bad = true;
+                s_fail = 1;
+            }
+        };
+        const int bc = (ty + 1) * L::BX + tx + 1;      // own point in a p / v / p_{j-2} box and formed plane
+        const int wcc = (ty + 1) * L::WX + tx + 4;     // own point in a w box
+        const int tc = ty * TX + tx;                   // own point in a tile box
+        // this thread's halo point, if any: y - 1 row, y + TY row, x - 1 column, x + TX column
+        const int hb = tid < TX ? tid + 1
+                     : tid < 2 * TX ? (TY + 1) * L::BX + tid - TX + 1
+                     : tid < 2 * TX + TY ? (tid - 2 * TX + 1) * L::BX
+                                         : (tid - 2 * TX - TY + 1) * L::BX + TX + 1;
+        const long long sxy = (long long)nx * ny;
         for (int i = (int)vg.bx; i < items; i += (int)vg.gx) {
             const int t = i % tiles, ch = i / tiles;
             const int za = (int)((long long)ch * nz / nchunk), zb = (int)((long long)(ch + 1) * nz / nchunk);
@@ -249,124 +275,112 @@ __device__ __forceinline__ void step_body(
             const int ja = max(za - 1, 0), jb = min(zb, nz - 1);
             const bool inside = x < nx && y < ny;
             const bool okxm = x > 0, okxp = x + 1 < nx, okym = y > 0, okyp = y + 1 < ny;
-            const int bc = (ty + 1) * L::BX + tx + 1;      // own point in a p / v / p_{j-2} box and formed plane
-            const int wcc = (ty + 1) * L::WX + tx + 4;     // own point in a w box
-            const int tc = ty * TX + tx;                   // own point in a tile box
             // own column: p_j of planes z - 1, z, z + 1, z_j of z and z + 1,
             // the weights of z - 1, z, z + 1 and the x / y coefficients of z, z + 1
-            float pm[K], pc[K], pn[K], zc[K], zn[K], cxy[4], cxyn[4];
+            Maps pm = zero, pc = zero, pn = zero, zc = zero, zn = zero;
+            float cxy[4], cxyn[4];
             float wm = 0.f, wc = 0.f, wn = 0.f;
-#pragma unroll
-            for (int a = 0; a < K; ++a) pm[a] = pc[a] = pn[a] = zc[a] = zn[a] = 0.f;
 #pragma unroll
             for (int m = 0; m < 4; ++m) cxy[m] = cxyn[m] = 0.f;
             float part[kStepSums] = {};
-            const long long col = (long long)x + (long long)nx * y;
-            const long long sxy = (long long)nx * ny;
+            long long n = (long long)x + (long long)nx * y + sxy * ja;   // own voxel in plane jj
+            const float4* fpc = nullptr;                                 // formed planes jj and jj - 1
+            const float4* fpm = nullptr;
 
-            // Phase B for plane z (counter cz of its formed plane, H counter e):
-            // `up` holds p_j of plane z + 1 (or of z itself at the top face).
-            auto phase_b = [&](int z, int cz, int e, const float (&up)[K], float wup) {
-                const bool ok = !s_fail && mbar_wait(smem_u32(&h_full[h_stage(e)]), h_phase(e), wait_cycles);
-                if (!ok) s_fail = 1;
-                if (ok && inside) {
-                    const float* hb = reinterpret_cast<const float*>(smem + L::H_BASE + h_stage(e) * L::H_STAGE);
+            // Phase B for plane z, voxel n (its formed plane fp): `up` holds
+            // p_j of plane z + 1 (or of z itself at the top face).
+            auto phase_b = [&](int z, long long nz_, const float4* fp, const Maps& up, float wup) {
+                wait(hf0 + 8 * hs, hph);
+                if (!bad && inside) {
+                    const float* hp = reinterpret_cast<const float*>(smem + L::H_BASE + hs * L::H_STAGE) + tc;
                     float hv[T];
 #pragma unroll
-                    for (int m = 0; m < T; ++m) hv[m] = hb[m * TX * TY + tc];
-                    const float4* fp = formed(cz);
-                    float nb[4][K];
-                    unpack4<K>(fp[bc - 1], nb[0]);
-                    unpack4<K>(fp[bc + 1], nb[1]);
-                    unpack4<K>(fp[bc - L::BX], nb[2]);
-                    unpack4<K>(fp[bc + L::BX], nb[3]);
+                    for (int m = 0; m < T; ++m) hv[m] = hp[m * TX * TY];
                     const float c6[6] = {cxy[0], cxy[1], cxy[2], cxy[3],
                                          z > 0 ? (wc + wm) * P.ihz2 : 0.f,
                                          z + 1 < nz ? (wc + wup) * P.ihz2 : 0.f};
-                    auto nbf = [&](int m, int a) -> float {
-                        return m < 4 ? nb[m][a] : (m == 4 ? pm[a] : up[a]);
+                    auto nb = [&](int m) -> Maps {
+                        return m == 0 ? Maps(fp[bc - 1]) : m == 1 ? Maps(fp[bc + 1])
+                             : m == 2 ? Maps(fp[bc - L::BX]) : m == 3 ? Maps(fp[bc + L::BX])
+                             : m == 4 ? pm : up;
                     };
-                    float v[K], sums[kStepSums];
-                    step_voxel<K>(P, c6, zc, pc, nbf, hv, want_rr, v, sums);
-                    vout[col + sxy * z] = pack4<K>(v);
-#pragma unroll
-                    for (int s = 0; s < kStepSums; ++s) part[s] += sums[s];
+                    Maps v;
+                    step_voxel<K>(P, c6, zc, pc, nb, hv, want_rr, v, part);
+                    vout[nz_] = v.vec();
                 }
                 __syncwarp();
-                if (lane == 0) mbar_arrive(smem_u32(&h_empty[h_stage(e)]));
+                if (lane == 0) mbar_arrive(he0 + 8 * hs);
+                if (++hs == (unsigned)kStepH) {
+                    hs = 0;
+                    hph ^= 1u;
+                }
             };
 
             for (int jj = ja; jj <= jb; ++jj) {
-                const int c = cb + (jj - ja);
                 const bool inner = jj >= za && jj < zb;
-                const bool ok = !s_fail && mbar_wait(smem_u32(&raw_full[r_stage(c)]), r_phase(c), wait_cycles);
-                if (!ok) s_fail = 1;
-                if (ok) {
+                wait(rf0 + 8 * rs, rph);
+                float4* fp = reinterpret_cast<float4*>(smem + L::S_BASE + fs * L::SLOT);
+                fpm = fpc;
+                fpc = fp;
+                if (!bad) {
                     // Phase A: z_j and p_j of this plane
-                    const unsigned char* st = smem + r_stage(c) * L::RAW;
+                    const unsigned char* st = smem + rs * L::RAW;
                     const float4* bp = reinterpret_cast<const float4*>(st + L::P_OFF);
                     const float4* bv = reinterpret_cast<const float4*>(st + L::V_OFF);
                     const float4* b2 = reinterpret_cast<const float4*>(st + L::P2_OFF);
-                    const float* bw = reinterpret_cast<const float*>(st + L::W_OFF);
-                    const float4 p4 = bp[bc], p24 = third ? b2[bc] : zero4;
-                    step_point<K, MODE>(sc, p4, first ? zero4 : bv[bc], p24, zn, pn);
-                    wn = bw[wcc];
-                    cxyn[0] = okxm ? (wn + bw[wcc - 1]) * P.ihx2 : 0.f;
-                    cxyn[1] = okxp ? (wn + bw[wcc + 1]) * P.ihx2 : 0.f;
-                    cxyn[2] = okym ? (wn + bw[wcc - L::WX]) * P.ihy2 : 0.f;
-                    cxyn[3] = okyp ? (wn + bw[wcc + L::WX]) * P.ihy2 : 0.f;
+                    const float* bw = reinterpret_cast<const float*>(st + L::W_OFF) + wcc;
+                    const Maps p1 = bp[bc], p2 = third ? Maps(b2[bc]) : zero;
+                    step_point<MODE>(sc, p1, first ? zero : Maps(bv[bc]), p2, zn, pn);
+                    wn = bw[0];
+                    cxyn[0] = okxm ? (wn + bw[-1]) * P.ihx2 : 0.f;
+                    cxyn[1] = okxp ? (wn + bw[1]) * P.ihx2 : 0.f;
+                    cxyn[2] = okym ? (wn + bw[-L::WX]) * P.ihy2 : 0.f;
+                    cxyn[3] = okyp ? (wn + bw[L::WX]) * P.ihy2 : 0.f;
                     if (inner) {
-                        float4* fp = formed(c);
-                        fp[bc] = pack4<K>(pn);
+                        fp[bc] = pn.vec();
                         if (tid < L::NH) {
-                            // halo point: y - 1 row, y + TY row, x - 1 column, x + TX column
-                            int hb;
-                            if (tid < TX) hb = tid + 1;
-                            else if (tid < 2 * TX) hb = (TY + 1) * L::BX + tid - TX + 1;
-                            else if (tid < 2 * TX + TY) hb = (tid - 2 * TX + 1) * L::BX;
-                            else hb = (tid - 2 * TX - TY + 1) * L::BX + TX + 1;
-                            float hzj[K], hpj[K];
-                            step_point<K, MODE>(sc, bp[hb], first ? zero4 : bv[hb], third ? b2[hb] : zero4,
-                                                hzj, hpj);
-                            fp[hb] = pack4<K>(hpj);
+                            Maps hz, hpj;
+                            step_point<MODE>(sc, bp[hb], first ? zero : Maps(bv[hb]),
+                                             third ? Maps(b2[hb]) : zero, hz, hpj);
+                            fp[hb] = hpj.vec();
                         }
                         if (inside) {
-                            const long long n = col + sxy * jj;
-                            if (!first) pout[n] = pack4<K>(pn);
+                            if (!first) pout[n] = pn.vec();
                             if (fold) {
                                 const float4* bx = reinterpret_cast<const float4*>(st + L::X_OFF);
-                                xacc[n] = fold_x(readx ? bx[tc] : zero4, sc.alpha_prev, p24, sc.alpha, p4);
+                                xacc[n] = fold_x(readx ? Maps(bx[tc]) : zero, sc, p2, p1).vec();
                             }
                         }
                     }
                 }
                 __syncwarp();
-                if (lane == 0) mbar_arrive(smem_u32(&raw_empty[r_stage(c)]));
-                compute_warps_sync<L::VOX>();
-                if (jj - 1 >= za) phase_b(jj - 1, c - 1, eb + (jj - 1 - za), pn, wn);
-                // the plane above becomes current
-#pragma unroll
-                for (int a = 0; a < K; ++a) {
-                    pm[a] = pc[a];
-                    pc[a] = pn[a];
-                    zc[a] = zn[a];
+                if (lane == 0) mbar_arrive(re0 + 8 * rs);
+                if (++rs == (unsigned)kStepRaw) {
+                    rs = 0;
+                    rph ^= 1u;
                 }
+                if (++fs == 3u) fs = 0;
+                compute_warps_sync<L::VOX>();
+                if (jj - 1 >= za) phase_b(jj - 1, n - sxy, fpm, pn, wn);
+                // the plane above becomes current
+                pm = pc;
+                pc = pn;
+                zc = zn;
 #pragma unroll
                 for (int m = 0; m < 4; ++m) cxy[m] = cxyn[m];
                 wm = wc;
                 wc = wn;
+                n += sxy;
             }
-            if (jb == zb - 1) {
-                // the item reaches the top face: its last plane has no plane above
-                phase_b(jb, cb + (jb - ja), eb + (jb - za), pc, wc);
-            }
-            cb += jb - ja + 1;
-            eb += zb - za;
+            // an item that reaches the top face: its last plane has no plane above
+            if (jb == zb - 1) phase_b(jb, n - sxy, fpc, pc, wc);
+            // the item's sums: the warp's lanes as compensated pairs
+            Acc a[kStepSums];
 #pragma unroll
-            for (int s = 0; s < kStepSums; ++s) {
-                acc[s].add(part[s]);
-                part[s] = 0.f;
-            }
+            for (int s = 0; s < kStepSums; ++s) a[s].hi = part[s];
+            warp_combine<kStepSums>(a, sums);
+            if (lane == 0)
+                for (int s = 0; s < sums; ++s) s_acc[warp][s].add(a[s]);
         }
     }
     __syncthreads();
@@ -384,7 +398,9 @@ __device__ __forceinline__ void step_body(
         __syncthreads();
     }
     double out[kStepSums];
-    if (grid_reduce<kStepSums>(acc, red, out, vg, want_rr ? kStepSums : kSumRR) && tid == 0)
+    if (grid_reduce_warps<kStepSums>(
+            [&](int s, int w) { return s_acc[w][s]; }, kStepWarps, red, out, vg, sums) &&
+        tid == 0)
         step_scalars(out, j, want_rr, hdr, resid);
 }
 

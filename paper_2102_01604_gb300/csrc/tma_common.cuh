@@ -49,6 +49,7 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity)
 // Bounded wait: false after about `cycles` clock cycles.
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, long long cycles)
 {
+    if (mbar_try_wait(bar, parity)) return true;      // no clock read when the phase is complete
     const long long t0 = clock64();
     while (!mbar_try_wait(bar, parity))
         if (clock64() - t0 > cycles) return false;
