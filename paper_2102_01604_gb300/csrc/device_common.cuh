@@ -326,6 +326,18 @@ __device__ __forceinline__ void prefetch_l2(const void* p)
     asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
 }
 
+// Programmatic dependent launch: a kernel launched with launch_dependent may
+// start while its predecessor on the stream still runs, and must call
+// wait_predecessor before it reads or writes anything the predecessor touches
+// (it returns when that grid has completed and its memory is visible; a no-op
+// after an ordinary launch).  release_dependents lets the successor start as
+// soon as every block of this grid has called it or exited.
+__device__ __forceinline__ void wait_predecessor() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void release_dependents()
+{
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 template <typename T>
 __device__ __forceinline__ float load_echo(const T* p, long long i);
 

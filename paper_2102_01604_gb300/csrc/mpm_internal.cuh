@@ -5,6 +5,7 @@
 #pragma once
 
 #include <string>
+#include <utility>
 
 #include "device_common.cuh"
 #include "host_logic.h"
@@ -39,6 +40,24 @@ struct LaunchScope {
     cudaStream_t st;
     void* rec;
 };
+
+// Launches f so that it may start before its predecessor on the stream has
+// finished (programmatic dependent launch): f must call wait_predecessor.
+template <class... P, class... A>
+cudaError_t launch_dependent(void (*f)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args)
+{
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, f, std::forward<A>(args)...);
+}
 
 // ------------------------------------------------------- kernel launchers
 // (defined in voxel_kernels.cu and stencil_kernels.cu; return cudaError_t of

@@ -257,6 +257,31 @@ __device__ __forceinline__ void step_voxel(const DevProblem& P, const float (&c)
     }
 }
 
+// Float64 division in a serial chain: GB300's float64 operations have about a
+// hundred cycles of latency each, and two IEEE divisions with their NaN tests
+// made the one thread that derives the scalars take 4000 cycles (2 us of a
+// 12 us iteration of a small volume).  recip: the float32 reciprocal and one
+// Newton-Raphson step y <- y + y (1 - b y) (relative error about 2^-45; b
+// outside float32's range divides); quot: a / b from it with one residual
+// correction (about 2^-53).
+__device__ __forceinline__ double recip(double b)
+{
+    if (!(b > 1e-30 && b < 1e30)) return 1.0 / b;
+    const double y = (double)(1.0f / (float)b);
+    return fma(y, fma(-b, y, 1.0), y);
+}
+
+__device__ __forceinline__ double quot(double a, double b, double y)
+{
+    const double q = a * y;
+    return fma(fma(-b, q, a), y, q);
+}
+
+__device__ __forceinline__ bool is_nan(double v)
+{
+    return ((unsigned long long)__double_as_longlong(v) << 1) > 0xffe0000000000000ull;
+}
+
 // Scalars of iteration j from its reduced sums (the last block of the launch):
 // alpha_j = r_j.z_j / p_j.q_j, the expanded r_{j+1}.z_{j+1} and |r_{j+1}|^2,
 // beta_j and the stopping tests.  A breakdown (p.q or r.z not positive, or a
@@ -265,21 +290,23 @@ __device__ __forceinline__ void step_scalars(const double (&s)[kStepSums], int j
                                              WsHeader* hdr, double* resid)
 {
     SolveScalars& sc = hdr->sc;
+    const double alpha_old = sc.alpha, beta_old = sc.beta;
     bool bad = false;
 #pragma unroll
-    for (int i = 0; i < kStepSums; ++i) bad |= !(s[i] == s[i]);
+    for (int i = 0; i < kStepSums; ++i) bad |= is_nan(s[i]);
     if (bad) atomicOr(&hdr->status, kStatusNaN);
     const double pq = s[kSumPQ], rz = s[kSumZR];
     if (bad || !(pq > 0.0) || !(rz > 0.0)) {
         sc.done = 1;                       // no further step; the alphas keep their values
         return;
     }
-    const double alpha = rz / pq;
-    const double rz_next = rz - 2.0 * alpha * s[kSumZQ] + alpha * alpha * s[kSumVQ];
-    sc.alpha_prev = sc.alpha;
+    const double ipq = recip(pq), irz = recip(rz);
+    const double alpha = quot(rz, pq, ipq);
+    const double rz_next = fma(alpha, fma(alpha, s[kSumVQ], -2.0 * s[kSumZQ]), rz);
+    sc.alpha_prev = alpha_old;
     sc.alpha = alpha;
-    sc.beta_prev = sc.beta;
-    sc.beta = rz_next / rz;
+    sc.beta_prev = beta_old;
+    sc.beta = quot(rz_next, rz, irz);
     sc.rz = rz_next;
     sc.it = j + 1;
     if (resid_sums) {

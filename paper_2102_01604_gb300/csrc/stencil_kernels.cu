@@ -279,6 +279,7 @@ __device__ __forceinline__ void pcg_init_body(const DevProblem& P, int zc, const
         }
     }
     if (!pd) atomicOr(&hdr->status, kStatusNotPD);
+    release_dependents();
     Acc v[2] = {rz, rr};
     double out[2];
     if (grid_reduce<2>(v, red, out, vg) && threadIdx.x == 0 && threadIdx.y == 0) {
@@ -342,6 +343,7 @@ __global__ void __launch_bounds__(kBlock) k_pcg_step(DevProblem P, int zc, int j
     __shared__ StepScalars s_sc;
     __shared__ int s_done;
     const int tid = threadIdx.x + threadIdx.y * blockDim.x;
+    wait_predecessor();
     if (tid == 0) {
         s_done = hdr->sc.done;
         s_sc = StepScalars{(float)hdr->sc.alpha, (float)hdr->sc.alpha_prev, (float)hdr->sc.beta,
@@ -386,6 +388,7 @@ __global__ void __launch_bounds__(kBlock) k_pcg_step(DevProblem P, int zc, int j
             if (MODE >= kModeFold) xacc[n] = fold_x(MODE == kModeFoldX ? xacc[n] : zero, sc, p2[n], pin[n]).vec();
         }
     }
+    release_dependents();
     Acc acc[kStepSums];
 #pragma unroll
     for (int i = 0; i < kStepSums; ++i) acc[i].add(part[i]);
@@ -411,6 +414,7 @@ __device__ __forceinline__ void pcg_final_body(long long N, const SolveBufs& B, 
                                                float* __restrict__ y_update, const WsHeader* hdr,
                                                double* report_rel, int* report_it, const VGrid& vg)
 {
+    wait_predecessor();
     const SolveScalars sc = hdr->sc;
     const bool have_x = sc.xcount > 0;
     const int pend = sc.it - sc.xcount;        // directions not yet in x: 0, 1 or 2
@@ -535,16 +539,17 @@ int step_mode(int j)
 }
 
 template <int K>
-static void launch_step_plain(const DevProblem& P, const StencilGrid& sg, int j, int want_rr,
+static cudaError_t launch_step_plain(const DevProblem& P, const StencilGrid& sg, int j, int want_rr,
                               const float* h, const float* w, const SolveBufs& B, WsHeader* hdr,
                               double* resid, Reduce red, cudaStream_t st)
 {
     const int jm = j > 0 ? j - 1 : 0;
     const float4 *pin = B.p[jm % 3], *vin = B.v[jm & 1], *p2 = B.p[(j + 1) % 3];
     float4 *vout = B.v[j & 1], *pout = B.p[j % 3];
+    cudaError_t e;
 #define MPM_STEP_PLAIN(M)                                                                          \
-    k_pcg_step<K, M><<<sg.grid, sg.block, 0, st>>>(P, sg.zc, j, want_rr, h, w, pin, vin, p2, vout, pout, \
-                                                   B.x, hdr, resid, red)
+    e = launch_dependent(k_pcg_step<K, M>, sg.grid, sg.block, 0, st, P, sg.zc, j, want_rr, h, w, pin, vin, p2, \
+                         vout, pout, B.x, hdr, resid, red)
     switch (step_mode(j)) {
     case kModeFirst: MPM_STEP_PLAIN(kModeFirst); break;
     case kModeSecond: MPM_STEP_PLAIN(kModeSecond); break;
@@ -553,6 +558,7 @@ static void launch_step_plain(const DevProblem& P, const StencilGrid& sg, int j,
     default: MPM_STEP_PLAIN(kModeFoldX); break;
     }
 #undef MPM_STEP_PLAIN
+    return e;
 }
 
 template <int K>
@@ -577,17 +583,13 @@ static cudaError_t solve_k(const DevProblem& P, int cg_iters, double tol_cg, con
     for (int j = 0; j < cg_iters; ++j) {
         const int rr = (want_resid || j == cg_iters - 1) ? 1 : 0;
         LaunchScope ls(MPM_KERNEL_PCG_STEP, st);
-        if (tma) {
-            cudaError_t e = launch_step_tma(P, tg, maps, j, step_mode(j), rr, hdr, resid, red, st);
-            if (e != cudaSuccess) return e;
-        } else {
-            launch_step_plain<K>(P, sg, j, rr, h, w, B, hdr, resid, red, st);
-        }
+        const cudaError_t e = tma ? launch_step_tma(P, tg, maps, j, step_mode(j), rr, hdr, resid, red, st)
+                                  : launch_step_plain<K>(P, sg, j, rr, h, w, B, hdr, resid, red, st);
+        if (e != cudaSuccess) return e;
     }
     LaunchScope ls(MPM_KERNEL_PCG_FINAL, st);
-    k_pcg_final<K><<<voxel_grid(P.N), kBlock, 0, st>>>(P.N, B, delta, y_update, hdr, report_rel,
-                                                       report_it);
-    return cudaGetLastError();
+    return launch_dependent(k_pcg_final<K>, dim3(voxel_grid(P.N)), dim3(kBlock), 0, st, P.N, B, delta, y_update,
+                            hdr, report_rel, report_it);
 }
 
 cudaError_t tma_autotune(const DevProblem& P, void* solve_ws, WsHeader* hdr, Reduce red,
@@ -687,10 +689,8 @@ cudaError_t launch_pcg_final_batch(int K, const FinalArgs* a, const unsigned* bl
     fill_batch(b, a, blocks, n);
     LaunchScope ls(MPM_KERNEL_PCG_FINAL, st);
     if (K == 4)
-        k_pcg_final_batch<4><<<b.start[n], kBlock, 0, st>>>(b);
-    else
-        k_pcg_final_batch<3><<<b.start[n], kBlock, 0, st>>>(b);
-    return cudaGetLastError();
+        return launch_dependent(k_pcg_final_batch<4>, dim3(b.start[n]), dim3(kBlock), 0, st, b);
+    return launch_dependent(k_pcg_final_batch<3>, dim3(b.start[n]), dim3(kBlock), 0, st, b);
 }
 
 cudaError_t launch_solve(const DevProblem& P, const SolveOpts& so, const float* h,

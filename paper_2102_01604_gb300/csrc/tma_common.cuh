@@ -69,6 +69,12 @@ __device__ __forceinline__ bool mbar_wait_nap(uint32_t bar, uint32_t parity, lon
     return true;
 }
 
+// Fetch a tensor map ahead of the first copy that uses it.
+__device__ __forceinline__ void prefetch_map(const CUtensorMap* map)
+{
+    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
+}
+
 __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, int c0, int c1,
                                             int c2, uint32_t bar)
 {
