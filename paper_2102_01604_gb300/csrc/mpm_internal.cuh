@@ -41,14 +41,16 @@ struct LaunchScope {
     void* rec;
 };
 
-// Launches f so that it may start before its predecessor on the stream has
-// finished (programmatic dependent launch): f must call wait_predecessor.
+// Launches f; with `overlap`, so that it may start before its predecessor on
+// the stream has finished (programmatic dependent launch): f must call
+// wait_predecessor.
 template <class... P, class... A>
-cudaError_t launch_dependent(void (*f)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args)
+cudaError_t launch_dependent(bool overlap, void (*f)(P...), dim3 grid, dim3 block, size_t smem,
+                             cudaStream_t st, A&&... args)
 {
     cudaLaunchAttribute attr;
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
+    attr.val.programmaticStreamSerializationAllowed = overlap ? 1 : 0;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
@@ -99,8 +101,11 @@ struct SolveOpts {
     int mg_nu;
     float mg_omega;
     int mg_coarse_sweeps;
+    bool overlap;           // an iteration's launch may start before the one before it has ended
 };
-SolveOpts solve_opts(const mpm_opts& o);
+// overlap: false for fits that share the GPU with others (the server's), whose
+// blocks an early launch's waiting blocks would keep out
+SolveOpts solve_opts(const mpm_opts& o, bool overlap = true);
 cudaError_t launch_solve(const DevProblem& P, const SolveOpts& so, const float* h,
                          const float* w, const float* g, const float* y, float* delta,
                          float* y_update, double* resid, double* report_rel,
@@ -139,7 +144,7 @@ cudaError_t tma_autotune(const DevProblem& P, void* solve_ws, WsHeader* hdr, Red
                          cudaStream_t st, int* best, float* ms);
 // Iteration j (mode kMode*) of a solve; want_rr also reduces the |r|^2 sums.
 cudaError_t launch_step_tma(const DevProblem& P, const StencilGrid& g, const StepMaps& m, int j,
-                            int mode, int want_rr, WsHeader* hdr, double* resid, Reduce red,
+                            int mode, int want_rr, WsHeader* hdr, double* resid, Reduce red, bool overlap,
                             cudaStream_t st);
 // Launches serving several subjects (batch.cuh): blocks[s] hardware blocks
 // for subject s, n <= kBatchMax.

@@ -190,7 +190,7 @@ size_t solve_ws_bytes(const DevProblem& P)
     return pcg > mg ? pcg : mg;
 }
 
-SolveOpts solve_opts(const mpm_opts& o)
+SolveOpts solve_opts(const mpm_opts& o, bool overlap)
 {
     SolveOpts s;
     s.cg_iters = o.cg_iters;
@@ -199,6 +199,7 @@ SolveOpts solve_opts(const mpm_opts& o)
     s.mg_nu = o.mg_nu > 0 ? o.mg_nu : 1;
     s.mg_omega = o.mg_omega > 0.0 ? (float)o.mg_omega : 0.7f;
     s.mg_coarse_sweeps = o.mg_coarse_sweeps > 0 ? o.mg_coarse_sweeps : 20;
+    s.overlap = overlap;
     return s;
 }
 
@@ -541,14 +542,14 @@ int step_mode(int j)
 template <int K>
 static cudaError_t launch_step_plain(const DevProblem& P, const StencilGrid& sg, int j, int want_rr,
                               const float* h, const float* w, const SolveBufs& B, WsHeader* hdr,
-                              double* resid, Reduce red, cudaStream_t st)
+                              double* resid, Reduce red, bool overlap, cudaStream_t st)
 {
     const int jm = j > 0 ? j - 1 : 0;
     const float4 *pin = B.p[jm % 3], *vin = B.v[jm & 1], *p2 = B.p[(j + 1) % 3];
     float4 *vout = B.v[j & 1], *pout = B.p[j % 3];
     cudaError_t e;
 #define MPM_STEP_PLAIN(M)                                                                          \
-    e = launch_dependent(k_pcg_step<K, M>, sg.grid, sg.block, 0, st, P, sg.zc, j, want_rr, h, w, pin, vin, p2, \
+    e = launch_dependent(overlap, k_pcg_step<K, M>, sg.grid, sg.block, 0, st, P, sg.zc, j, want_rr, h, w, pin, vin, p2, \
                          vout, pout, B.x, hdr, resid, red)
     switch (step_mode(j)) {
     case kModeFirst: MPM_STEP_PLAIN(kModeFirst); break;
@@ -562,7 +563,7 @@ static cudaError_t launch_step_plain(const DevProblem& P, const StencilGrid& sg,
 }
 
 template <int K>
-static cudaError_t solve_k(const DevProblem& P, int cg_iters, double tol_cg, const float* h,
+static cudaError_t solve_k(const DevProblem& P, const SolveOpts& so, const float* h,
                            const float* w, const float* g, const float* y, float* delta,
                            float* y_update, double* resid, double* report_rel, int* report_it,
                            void* solve_ws, WsHeader* hdr, Reduce red, cudaStream_t st)
@@ -570,7 +571,8 @@ static cudaError_t solve_k(const DevProblem& P, int cg_iters, double tol_cg, con
     const StencilGrid sg = stencil_grid(P, kTileX, kTileY);
     const StencilGrid ig = stencil_grid(P, kTileX, kTileY, kInitWaves);
     SolveBufs B = carve(P, solve_ws);
-    const double tol2 = tol_cg > 0.0 ? tol_cg * tol_cg : 0.0;
+    const int cg_iters = so.cg_iters;
+    const double tol2 = so.tol_cg > 0.0 ? so.tol_cg * so.tol_cg : 0.0;
     {
         LaunchScope ls(MPM_KERNEL_PCG_INIT, st);
         k_pcg_init<K><<<ig.grid, ig.block, 0, st>>>(P, ig.zc, h, w, g, y, B.p[0], tol2, hdr, resid, red);
@@ -583,12 +585,12 @@ static cudaError_t solve_k(const DevProblem& P, int cg_iters, double tol_cg, con
     for (int j = 0; j < cg_iters; ++j) {
         const int rr = (want_resid || j == cg_iters - 1) ? 1 : 0;
         LaunchScope ls(MPM_KERNEL_PCG_STEP, st);
-        const cudaError_t e = tma ? launch_step_tma(P, tg, maps, j, step_mode(j), rr, hdr, resid, red, st)
-                                  : launch_step_plain<K>(P, sg, j, rr, h, w, B, hdr, resid, red, st);
+        const cudaError_t e = tma ? launch_step_tma(P, tg, maps, j, step_mode(j), rr, hdr, resid, red, so.overlap, st)
+                                  : launch_step_plain<K>(P, sg, j, rr, h, w, B, hdr, resid, red, so.overlap, st);
         if (e != cudaSuccess) return e;
     }
     LaunchScope ls(MPM_KERNEL_PCG_FINAL, st);
-    return launch_dependent(k_pcg_final<K>, dim3(voxel_grid(P.N)), dim3(kBlock), 0, st, P.N, B, delta, y_update,
+    return launch_dependent(so.overlap, k_pcg_final<K>, dim3(voxel_grid(P.N)), dim3(kBlock), 0, st, P.N, B, delta, y_update,
                             hdr, report_rel, report_it);
 }
 
@@ -627,7 +629,7 @@ cudaError_t tma_autotune(const DevProblem& P, void* solve_ws, WsHeader* hdr, Red
         for (int i = 0; i <= reps && e == cudaSuccess; ++i) {
             if (i == 1) e = cudaEventRecord(a, st);
             if (e == cudaSuccess) e = cudaMemsetAsync(hdr, 0, sizeof(WsHeader), st);
-            if (e == cudaSuccess) e = launch_step_tma(P, g, m, 3, kModeStep, 0, hdr, nullptr, red, st);
+            if (e == cudaSuccess) e = launch_step_tma(P, g, m, 3, kModeStep, 0, hdr, nullptr, red, true, st);
         }
         if (e == cudaSuccess) e = cudaEventRecord(b, st);
         if (e == cudaSuccess) e = cudaEventSynchronize(b);
@@ -689,8 +691,8 @@ cudaError_t launch_pcg_final_batch(int K, const FinalArgs* a, const unsigned* bl
     fill_batch(b, a, blocks, n);
     LaunchScope ls(MPM_KERNEL_PCG_FINAL, st);
     if (K == 4)
-        return launch_dependent(k_pcg_final_batch<4>, dim3(b.start[n]), dim3(kBlock), 0, st, b);
-    return launch_dependent(k_pcg_final_batch<3>, dim3(b.start[n]), dim3(kBlock), 0, st, b);
+        return launch_dependent(true, k_pcg_final_batch<4>, dim3(b.start[n]), dim3(kBlock), 0, st, b);
+    return launch_dependent(true, k_pcg_final_batch<3>, dim3(b.start[n]), dim3(kBlock), 0, st, b);
 }
 
 cudaError_t launch_solve(const DevProblem& P, const SolveOpts& so, const float* h,
@@ -702,9 +704,9 @@ cudaError_t launch_solve(const DevProblem& P, const SolveOpts& so, const float* 
         return launch_solve_mg(P, so, h, w, g, y, delta, y_update, resid, report_rel, report_it,
                                solve_ws, hdr, red, st);
     if (P.K == 4)
-        return solve_k<4>(P, so.cg_iters, so.tol_cg, h, w, g, y, delta, y_update, resid, report_rel,
+        return solve_k<4>(P, so, h, w, g, y, delta, y_update, resid, report_rel,
                           report_it, solve_ws, hdr, red, st);
-    return solve_k<3>(P, so.cg_iters, so.tol_cg, h, w, g, y, delta, y_update, resid, report_rel,
+    return solve_k<3>(P, so, h, w, g, y, delta, y_update, resid, report_rel,
                       report_it, solve_ws, hdr, red, st);
 }
 

@@ -544,7 +544,8 @@ bool make_step_maps(const DevProblem& P, const float* h, const float* w, const S
 
 template <int K, int TX, int TY, int MODE>
 static cudaError_t launch_step_m(const DevProblem& P, int nchunk, dim3 grid, const StepMaps& m, int j,
-                                 int want_rr, WsHeader* hdr, double* resid, Reduce red, cudaStream_t st)
+                                 int want_rr, WsHeader* hdr, double* resid, Reduce red, bool overlap,
+                                 cudaStream_t st)
 {
     using L = StepLayout<K, TX, TY, (MODE >= kModeFold)>;
     static bool attr = false;
@@ -557,7 +558,7 @@ static cudaError_t launch_step_m(const DevProblem& P, int nchunk, dim3 grid, con
     }
     const int jm = j > 0 ? j - 1 : 0;
     return launch_dependent(
-        k_pcg_step_tma<K, TX, TY, MODE>, grid, dim3(L::THREADS, 1, 1), L::SMEM, st, P, nchunk, j, want_rr, m.p[jm % 3], m.v[jm & 1], m.p[(j + 1) % 3], m.w, m.h, m.x,
+        overlap, k_pcg_step_tma<K, TX, TY, MODE>, grid, dim3(L::THREADS, 1, 1), L::SMEM, st, P, nchunk, j, want_rr, m.p[jm % 3], m.v[jm & 1], m.p[(j + 1) % 3], m.w, m.h, m.x,
         m.B.v[j & 1], m.B.p[j % 3], m.B.x, hdr, resid, red,
         g_wait_cycles.load(std::memory_order_relaxed), g_withhold.load(std::memory_order_relaxed));
 }
@@ -565,14 +566,14 @@ static cudaError_t launch_step_m(const DevProblem& P, int nchunk, dim3 grid, con
 template <int K, int TX, int TY>
 static cudaError_t launch_step_k(const DevProblem& P, int nchunk, dim3 grid, const StepMaps& m, int j,
                                  int mode, int want_rr, WsHeader* hdr, double* resid, Reduce red,
-                                 cudaStream_t st)
+                                 bool overlap, cudaStream_t st)
 {
     switch (mode) {
-    case kModeFirst: return launch_step_m<K, TX, TY, kModeFirst>(P, nchunk, grid, m, j, want_rr, hdr, resid, red, st);
-    case kModeSecond: return launch_step_m<K, TX, TY, kModeSecond>(P, nchunk, grid, m, j, want_rr, hdr, resid, red, st);
-    case kModeStep: return launch_step_m<K, TX, TY, kModeStep>(P, nchunk, grid, m, j, want_rr, hdr, resid, red, st);
-    case kModeFold: return launch_step_m<K, TX, TY, kModeFold>(P, nchunk, grid, m, j, want_rr, hdr, resid, red, st);
-    default: return launch_step_m<K, TX, TY, kModeFoldX>(P, nchunk, grid, m, j, want_rr, hdr, resid, red, st);
+    case kModeFirst: return launch_step_m<K, TX, TY, kModeFirst>(P, nchunk, grid, m, j, want_rr, hdr, resid, red, overlap, st);
+    case kModeSecond: return launch_step_m<K, TX, TY, kModeSecond>(P, nchunk, grid, m, j, want_rr, hdr, resid, red, overlap, st);
+    case kModeStep: return launch_step_m<K, TX, TY, kModeStep>(P, nchunk, grid, m, j, want_rr, hdr, resid, red, overlap, st);
+    case kModeFold: return launch_step_m<K, TX, TY, kModeFold>(P, nchunk, grid, m, j, want_rr, hdr, resid, red, overlap, st);
+    default: return launch_step_m<K, TX, TY, kModeFoldX>(P, nchunk, grid, m, j, want_rr, hdr, resid, red, overlap, st);
     }
 }
 
@@ -614,7 +615,7 @@ static cudaError_t launch_step_batch_m(const Batch<StepArgs>& b, cudaStream_t st
         if (e != cudaSuccess) return e;
         attr = true;
     }
-    return launch_dependent(k_pcg_step_tma_batch<K, TX, TY, MODE>, dim3(b.start[b.n]), dim3(L::THREADS, 1, 1),
+    return launch_dependent(true, k_pcg_step_tma_batch<K, TX, TY, MODE>, dim3(b.start[b.n]), dim3(L::THREADS, 1, 1),
                             L::SMEM, st, b);
 }
 
@@ -750,17 +751,17 @@ cudaError_t prime_tma_kernels()
 }
 
 cudaError_t launch_step_tma(const DevProblem& P, const StencilGrid& g, const StepMaps& m, int j,
-                            int mode, int want_rr, WsHeader* hdr, double* resid, Reduce red,
+                            int mode, int want_rr, WsHeader* hdr, double* resid, Reduce red, bool overlap,
                             cudaStream_t st)
 {
     if (P.K == 4) {
-        if (m.tile == 2) return launch_step_k<4, 32, 16>(P, g.zc, g.grid, m, j, mode, want_rr, hdr, resid, red, st);
-        if (m.tile == 1) return launch_step_k<4, 32, 8>(P, g.zc, g.grid, m, j, mode, want_rr, hdr, resid, red, st);
-        return launch_step_k<4, 16, 16>(P, g.zc, g.grid, m, j, mode, want_rr, hdr, resid, red, st);
+        if (m.tile == 2) return launch_step_k<4, 32, 16>(P, g.zc, g.grid, m, j, mode, want_rr, hdr, resid, red, overlap, st);
+        if (m.tile == 1) return launch_step_k<4, 32, 8>(P, g.zc, g.grid, m, j, mode, want_rr, hdr, resid, red, overlap, st);
+        return launch_step_k<4, 16, 16>(P, g.zc, g.grid, m, j, mode, want_rr, hdr, resid, red, overlap, st);
     }
-    if (m.tile == 2) return launch_step_k<3, 32, 16>(P, g.zc, g.grid, m, j, mode, want_rr, hdr, resid, red, st);
-    if (m.tile == 1) return launch_step_k<3, 32, 8>(P, g.zc, g.grid, m, j, mode, want_rr, hdr, resid, red, st);
-    return launch_step_k<3, 16, 16>(P, g.zc, g.grid, m, j, mode, want_rr, hdr, resid, red, st);
+    if (m.tile == 2) return launch_step_k<3, 32, 16>(P, g.zc, g.grid, m, j, mode, want_rr, hdr, resid, red, overlap, st);
+    if (m.tile == 1) return launch_step_k<3, 32, 8>(P, g.zc, g.grid, m, j, mode, want_rr, hdr, resid, red, overlap, st);
+    return launch_step_k<3, 16, 16>(P, g.zc, g.grid, m, j, mode, want_rr, hdr, resid, red, overlap, st);
 }
 
 }  // namespace mpm
