@@ -23,12 +23,13 @@ struct Batch {
 
 struct JtvArgs {
     DevProblem P;
-    int zc;
+    int zc, stages;       // z planes per block; ring of the staged kernel (0: the plain one)
     unsigned gx, gy, gz;
     const float* y;
     float* w;
     double* jtv;
     Reduce red;
+    unsigned* status;     // kStatusTimeout of the staged kernel
 };
 
 struct GradArgs {

@@ -374,7 +374,7 @@ static cudaError_t fit_enqueue_updates(const FitJob& j, cudaStream_t st, int* it
     for (;; ++it) {
         NvtxUpdate range(it);
         w_fresh = (it % npi == 0);
-        if ((e = launch_jtv(P, j.y, w_fresh ? L.w : nullptr, L.jtv + it, L.red, st))) return e;
+        if ((e = launch_jtv(P, j.y, w_fresh ? L.w : nullptr, L.jtv + it, L.red, &L.hdr->status, st))) return e;
         if ((e = launch_lik(j, it, st))) return e;
         if (it >= j.opts.gn_iters) break;
         if ((e = launch_solve(P, solve_opts(j.opts), L.h, L.w, L.g, j.y, nullptr, j.y,
@@ -382,7 +382,7 @@ static cudaError_t fit_enqueue_updates(const FitJob& j, cudaStream_t st, int* it
             return e;
     }
     if (j.var) {
-        if (!w_fresh && (e = launch_jtv(P, j.y, L.w, L.jtv + MPM_MAX_REPORT + 1, L.red, st))) return e;
+        if (!w_fresh && (e = launch_jtv(P, j.y, L.w, L.jtv + MPM_MAX_REPORT + 1, L.red, &L.hdr->status, st))) return e;
         if ((e = launch_uncertainty(P, L.h, L.w, j.y, j.var, nullptr, nullptr, &L.hdr->status, st)))
             return e;
     }
@@ -403,7 +403,7 @@ static mpm_status fit_run_adaptive(const FitJob& j, cudaStream_t st, int* iters_
     for (;; ++it) {
         NvtxUpdate range(it);
         w_fresh = (it % npi == 0);
-        MPM_CUDA(launch_jtv(P, j.y, w_fresh ? L.w : nullptr, L.jtv + it, L.red, st));
+        MPM_CUDA(launch_jtv(P, j.y, w_fresh ? L.w : nullptr, L.jtv + it, L.red, &L.hdr->status, st));
         MPM_CUDA(launch_lik(j, it, st));
         if (it >= j.opts.gn_iters) break;
         double v[2];
@@ -420,7 +420,7 @@ static mpm_status fit_run_adaptive(const FitJob& j, cudaStream_t st, int* iters_
                               nullptr, L.cg_rel + it, L.cg_it + it, L.solve, L.hdr, L.red, st));
     }
     if (j.var) {
-        if (!w_fresh) MPM_CUDA(launch_jtv(P, j.y, L.w, L.jtv + MPM_MAX_REPORT + 1, L.red, st));
+        if (!w_fresh) MPM_CUDA(launch_jtv(P, j.y, L.w, L.jtv + MPM_MAX_REPORT + 1, L.red, &L.hdr->status, st));
         MPM_CUDA(launch_uncertainty(P, L.h, L.w, j.y, j.var, nullptr, nullptr, &L.hdr->status, st));
     }
     *iters_out = it;
@@ -561,8 +561,8 @@ static mpm_status capture_updates(FitJob* jobs, int n, GraphEntry& out)
 // One subject of a phase-batched fit: its grids and the TMA maps of its solve.
 struct PhasedSubject {
     FitJob* j;
-    StencilGrid sg;          // 32 x 8 stencil grid of the JTV kernel
-    StencilGrid ig;          // and of the PCG start
+    double share;            // its part of the group's voxels
+    StencilGrid ig;          // 32 x 8 stencil grid of the PCG start
     SolveBufs B;
     StepMaps maps;
     int nchunk;              // z ranges of its share of the iteration's wave
@@ -595,10 +595,10 @@ static cudaError_t enqueue_phased(std::vector<PhasedSubject>& subj, int tile, cu
     std::vector<StepArgs> sa(n);
     std::vector<FinalArgs> fa(n);
     std::vector<UncArgs> ua;
-    std::vector<unsigned> bst(n), bini(n), bvox(n), bstep(n);
+    std::vector<double> share(n);
+    std::vector<unsigned> bini(n), bvox(n), bstep(n);
     for (int s = 0; s < n; ++s) {
-        const StencilGrid& g = subj[s].sg;
-        bst[s] = g.grid.x * g.grid.y * g.grid.z;
+        share[s] = subj[s].share;
         const StencilGrid& gi = subj[s].ig;
         bini[s] = gi.grid.x * gi.grid.y * gi.grid.z;
         bvox[s] = subj[s].vox_blocks;
@@ -607,11 +607,10 @@ static cudaError_t enqueue_phased(std::vector<PhasedSubject>& subj, int tile, cu
     auto jtv = [&](bool fresh, int slot) {
         for (int s = 0; s < n; ++s) {
             const FitJob& j = *subj[s].j;
-            const StencilGrid& g = subj[s].sg;
-            ja[s] = JtvArgs{j.P, g.zc, g.grid.x, g.grid.y, g.grid.z, j.y, fresh ? j.L.w : nullptr,
-                            j.L.jtv + slot, j.L.red};
+            ja[s] = JtvArgs{j.P, 0, 0, 0, 0, 0, j.y, fresh ? j.L.w : nullptr, j.L.jtv + slot, j.L.red,
+                            &j.L.hdr->status};
         }
-        return launch_jtv_batch(K, ja.data(), bst.data(), n, st);
+        return launch_jtv_batch(K, ja.data(), share.data(), n, st);
     };
     cudaError_t e = cudaSuccess;
     bool w_fresh = false;
@@ -650,21 +649,21 @@ static cudaError_t enqueue_phased(std::vector<PhasedSubject>& subj, int tile, cu
     }
     // the posterior variance of the subjects that ask for it
     std::vector<JtvArgs> jv;
-    std::vector<unsigned> bjv, buv;
+    std::vector<double> sjv;
+    std::vector<unsigned> buv;
     ua.clear();
     for (int s = 0; s < n; ++s) {
         const FitJob& j = *subj[s].j;
         if (!j.var) continue;
-        const StencilGrid& g = subj[s].sg;
-        jv.push_back(JtvArgs{j.P, g.zc, g.grid.x, g.grid.y, g.grid.z, j.y, j.L.w,
-                             j.L.jtv + MPM_MAX_REPORT + 1, j.L.red});
-        bjv.push_back(bst[s]);
+        jv.push_back(JtvArgs{j.P, 0, 0, 0, 0, 0, j.y, j.L.w, j.L.jtv + MPM_MAX_REPORT + 1, j.L.red,
+                             &j.L.hdr->status});
+        sjv.push_back(share[s]);
         ua.push_back(UncArgs{j.P, j.L.h, j.L.w, j.y, j.var, nullptr, nullptr, &j.L.hdr->status});
         buv.push_back(bvox[s]);
     }
     if (!ua.empty()) {
         const int m = (int)ua.size();
-        if (!w_fresh && (e = launch_jtv_batch(K, jv.data(), bjv.data(), m, st))) return e;
+        if (!w_fresh && (e = launch_jtv_batch(K, jv.data(), sjv.data(), m, st))) return e;
         if ((e = launch_uncertainty_batch(K, ua.data(), buv.data(), m, st))) return e;
     }
     for (int s = 0; s < n; ++s) iters[index[s]] = it;
@@ -711,10 +710,9 @@ static void plan_phased(FitJob* jobs, int n, std::vector<std::vector<PhasedSubje
             long long vox = 0;
             for (const PhasedSubject& ps : grp) vox += ps.j->P.N;
             for (PhasedSubject& ps : grp) {
-                const double share = (double)ps.j->P.N / (double)vox;
-                ps.sg = stencil_grid(ps.j->P, kTileX, kTileY, 2, share);
-                ps.ig = stencil_grid(ps.j->P, kTileX, kTileY, kInitWaves, share);
-                const long long cap = std::max(1LL, std::llround(share * voxel_grid(1LL << 40)));
+                ps.share = (double)ps.j->P.N / (double)vox;
+                ps.ig = stencil_grid(ps.j->P, kTileX, kTileY, kInitWaves, ps.share);
+                const long long cap = std::max(1LL, std::llround(ps.share * voxel_grid(1LL << 40)));
                 ps.vox_blocks = (unsigned)std::min<long long>(voxel_grid(ps.j->P.N), cap);
             }
             std::vector<long long> t, blocks;
@@ -1045,7 +1043,7 @@ mpm_status mpm_jtv_weights(const mpm_problem* problem, const float* y, float* w,
     FitWs L;
     MPM_TRY(check_ws(P, MPM_CALL_JTV, ws, ws_bytes, L));
     MPM_CUDA(cudaMemsetAsync(L.hdr, 0, sizeof(WsHeader), st));
-    MPM_CUDA(launch_jtv(P, y, w, jtv, L.red, st));
+    MPM_CUDA(launch_jtv(P, y, w, jtv, L.red, &L.hdr->status, st));
     return MPM_OK;
 }
 

@@ -90,8 +90,10 @@ cudaError_t launch_image_means(const DevProblem& P, int echo_dtype, const void* 
 // (init_maps.cuh), written to y.
 cudaError_t launch_init_maps(const DevProblem& P, const double* means, float* y, cudaStream_t st);
 
+// `status` receives kStatusTimeout if a staged copy never lands.
 cudaError_t launch_jtv(const DevProblem& P, const float* y, float* w, double* jtv,
-                       Reduce red, cudaStream_t st);
+                       Reduce red, unsigned* status, cudaStream_t st);
+cudaError_t prime_jtv_kernels();   // shared-memory opt-ins, done before any graph capture
 // Schedule of one solve (from mpm_opts; the multigrid fields resolved to
 // their defaults).
 struct SolveOpts {
@@ -149,7 +151,8 @@ cudaError_t launch_step_tma(const DevProblem& P, const StencilGrid& g, const Ste
 // Launches serving several subjects (batch.cuh): blocks[s] hardware blocks
 // for subject s, n <= kBatchMax.
 SolveBufs solve_bufs(const DevProblem& P, void* solve_ws);
-cudaError_t launch_jtv_batch(int K, const JtvArgs* a, const unsigned* blocks, int n, cudaStream_t st);
+// share[s]: subject s's part of the group's voxels (the launch sets the grids).
+cudaError_t launch_jtv_batch(int K, const JtvArgs* a, const double* share, int n, cudaStream_t st);
 cudaError_t launch_grad_hess_batch(int K, int precond, int echo_dtype, const GradArgs* a,
                                    const unsigned* blocks, int n, cudaStream_t st);
 cudaError_t launch_pcg_init_batch(int K, const InitArgs* a, const unsigned* blocks, int n,

@@ -95,7 +95,7 @@ static mpm_status srv_eval(mpm_server* s, Request& r)
     cudaStream_t st = r.stream;
     const FitWs& L = r.L;
     r.w_fresh = (r.it % r.opts.newton_per_irls == 0);
-    SRV_CUDA(launch_jtv(r.P, r.y, r.w_fresh ? L.w : nullptr, L.jtv + r.it, L.red, st));
+    SRV_CUDA(launch_jtv(r.P, r.y, r.w_fresh ? L.w : nullptr, L.jtv + r.it, L.red, &L.hdr->status, st));
     SRV_CUDA(launch_grad_hess(r.P, r.problem.echo_dtype, r.x, r.y, r.b1p, r.b1m, L.g, L.h,
                               L.nll + r.it, L.red, &L.hdr->status, st));
     SlotHost& h = s->host[r.slot];
@@ -113,7 +113,7 @@ static mpm_status srv_finish(mpm_server* s, Request& r)
     const FitWs& L = r.L;
     const int it = r.it;
     if (r.var) {
-        if (!r.w_fresh) SRV_CUDA(launch_jtv(r.P, r.y, L.w, L.jtv + MPM_MAX_REPORT + 1, L.red, st));
+        if (!r.w_fresh) SRV_CUDA(launch_jtv(r.P, r.y, L.w, L.jtv + MPM_MAX_REPORT + 1, L.red, &L.hdr->status, st));
         SRV_CUDA(launch_uncertainty(r.P, L.h, L.w, r.y, r.var, nullptr, nullptr, &L.hdr->status, st));
     }
     SlotHost& h = s->host[r.slot];

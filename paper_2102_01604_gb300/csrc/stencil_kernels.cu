@@ -14,9 +14,11 @@
 // device memory and are produced by the last block of each reducing launch,
 // so the whole PCG runs without a host round trip.
 #include <algorithm>
+#include <type_traits>
 
 #include "mpm_internal.cuh"
 #include "pcg_step.cuh"
+#include "tma_common.cuh"
 
 namespace mpm {
 
@@ -57,6 +59,350 @@ static bool index32(const DevProblem& P)
 
 constexpr int kInitAhead = 2;     // planes between the PCG start's L2 hint and the use
 
+// (b - a)^2 of one voxel or of two at once (paired instructions, each lane
+// rounded as the single form), and s + q h of two.
+__device__ __forceinline__ float sqdiff(float b, float a)
+{
+    const float d = __fsub_rn(b, a);
+    return __fmul_rn(d, d);
+}
+__device__ __forceinline__ float2 sqdiff(float2 b, float2 a)
+{
+    const float2 d = __ffma2_rn(a, make_float2(-1.0f, -1.0f), b);   // b - a, one rounding
+    return __fmul2_rn(d, d);
+}
+__device__ __forceinline__ float2 addmul(float2 q, float h, float2 s)
+{
+    return __ffma2_rn(q, make_float2(h, h), s);
+}
+// Square roots s of x and their reciprocals r, two at once and without a
+// branch: Newton-Raphson from the hardware's 1/sqrt estimate y, s = x y + (x -
+// (x y)^2) y / 2 and r = y + y (1 - s y), each within about half an ulp (the
+// residuals are exact in the fused multiply-adds).  For x in [1e-30, 1e30].
+__device__ __forceinline__ void sqrt_recip(float2 x, float2& s, float2& r)
+{
+    const float2 y = make_float2(rsqrtf(x.x), rsqrtf(x.y));
+    const float2 s0 = __fmul2_rn(x, y), ns0 = make_float2(-s0.x, -s0.y);
+    s = __ffma2_rn(__ffma2_rn(ns0, s0, x), __fmul2_rn(y, make_float2(0.5f, 0.5f)), s0);
+    const float2 ns = make_float2(-s.x, -s.y);
+    r = __ffma2_rn(y, __ffma2_rn(ns, y, make_float2(1.0f, 1.0f)), y);
+}
+
+// Two compensated accumulators side by side (Acc::add in paired instructions).
+struct Acc2 {
+    float2 hi = {0.f, 0.f}, lo = {0.f, 0.f};
+    __device__ __forceinline__ static float2 neg(float2 v) { return make_float2(-v.x, -v.y); }
+    __device__ __forceinline__ void add(float2 x)
+    {
+        const float2 s = __fadd2_rn(hi, x);
+        const float2 bp = __fadd2_rn(s, neg(hi));
+        const float2 e = __fadd2_rn(__fadd2_rn(hi, neg(__fadd2_rn(s, neg(bp)))), __fadd2_rn(x, neg(bp)));
+        hi = s;
+        lo = __fadd2_rn(lo, e);
+    }
+    __device__ __forceinline__ Acc sum() const
+    {
+        Acc a, b;
+        a.hi = hi.x, a.lo = lo.x;
+        b.hi = hi.y, b.lo = lo.y;
+        a.add(b);
+        return a;
+    }
+};
+
+constexpr int kJtvThreads = 256;
+constexpr int kJtvRun = 4 * kJtvThreads;   // voxels of a plane per block of the staged kernel
+constexpr int kJtvStagesMax = 4;
+
+// Floats of one map in a stage: the block's voxels, a row on either side and
+// the rest of the 16-byte granules at both ends.
+__host__ __device__ constexpr int jtv_slot(int nx) { return (kJtvRun + 2 * nx + 6 + 3) / 4 * 4; }
+
+// The staged kernel.  A block takes 1024 consecutive voxels of a plane and
+// marches up a z range.  What it needs of a plane -- its voxels and one row
+// below and above them -- is one contiguous range of each map, so K lanes bring
+// each plane into a ring of `stages` shared-memory stages with one bulk copy
+// each, planes ahead of their use, whatever the alignment: a copy takes the
+// 16-byte granules that hold the range, and the range starts `shift` floats
+// into its slot.  (Granules that would reach out of y are left out and their
+// floats copied one by one.)  Plane z and the squared differences to plane
+// z - 1 stay in registers; the y neighbours and plane z + 1 come from the
+// stages.  RUNS (rows and arrays on 16-byte boundaries): a thread takes four
+// neighbouring voxels along x, shared accesses are 16 bytes, the x neighbours
+// come from the neighbouring lanes and every squared difference along x serves
+// both its voxels.  Otherwise a thread takes four voxels 256 apart, so that a
+// warp's shared accesses are 32 consecutive floats.  The six terms of a voxel
+// are summed in the order x-, x+, y-, y+, z-, z+ (a missing neighbour's term
+// left out).
+//
+// 20 B per voxel: HBM-bound once the loads are in flight and the instructions
+// few.  The 32 x 8 tile kernel below takes about 350 thread instructions per
+// voxel, 108.7 us at 176x240x256 (0.29 of the copy bandwidth) and 78 us at
+// 181x217x181.  Runs of four with their loads through L1: 80.2 us, bound by the
+// latency of 16 warps' loads; staged, 77.7; with the paired square roots and
+// sums and one wave of z ranges 63.5 us (90 us without RUNS), 181x217x181 58 us.
+// One thread filling all maps' stages was 16 us slower: it is on the path from
+// one plane's barrier to the next.
+template <int K, bool RUNS, typename IT>
+__device__ __forceinline__ void jtv_staged_body(const DevProblem& P, int zc, int stages,
+                                                const float* __restrict__ y, float* __restrict__ w,
+                                                double* jtv, Reduce red, unsigned* status,
+                                                long long wait_cycles, int withhold, const VGrid& vg)
+{
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    __shared__ __align__(8) uint64_t full[kJtvStagesMax];
+    __shared__ volatile int s_fail;
+    float* smem = reinterpret_cast<float*>(smem_raw);
+    const IT N = (IT)P.N;
+    const int nx = P.nx, ny = P.ny, nz = P.nz;
+    const int sxy = nx * ny;                                 // at most 2^23 (check_problem)
+    const int tid = threadIdx.x;
+    const int z0 = (int)vg.bz * zc, z1 = min(nz, z0 + zc), zlast = min(z1, nz - 1);
+    const int n0 = (int)vg.bx * kJtvRun;                     // this block's first voxel of a plane
+    const int lo = max(n0 - nx, 0), hi = min(n0 + kJtvRun + nx, sxy);
+    const int slot = jtv_slot(nx);
+    const uint32_t bar0 = smem_u32(&full[0]);
+    // floats by which the range of (map k, plane z) starts into its slot
+    const unsigned ymod = (unsigned)(reinterpret_cast<uintptr_t>(y) >> 2);
+    auto shift = [&](int k, int z) {
+        return (int)((ymod + (unsigned)k * (unsigned)P.N + (unsigned)z * (unsigned)sxy + (unsigned)lo) & 3u);
+    };
+    // Lane k of the first warp brings plane z of map k into stage st (the K
+    // copies of a stage complete its barrier together).
+    auto fill = [&](int z, int st) {
+        const int k = tid;
+        const uint32_t bar = bar0 + 8 * st;
+        const float* r = y + k * N + (IT)sxy * z + lo;                  // the range's first float
+        const int len = hi - lo;
+        if (RUNS) {                                                     // whole granules, inside y
+            mbar_expect_tx(bar, (uint32_t)len * 4u);
+            bulk_load(smem_u32(smem + (st * K + k) * slot), r, (uint32_t)len * 4u, bar);
+            return;
+        }
+        const int sh = shift(k, z);
+        float* d = smem + (st * K + k) * slot + sh;                     // its place
+        int b = -sh, e = (sh + len + 3) / 4 * 4 - sh;                   // the granules, from r
+        if (r + b < y) b += 4;
+        if (r + e > y + K * N) e -= 4;
+        const uint32_t bytes = e > b ? (uint32_t)(e - b) * 4u : 0u;
+        mbar_expect_tx(bar, bytes);
+        if (bytes) bulk_load(smem_u32(d + b), r + b, bytes, bar);
+        for (int q = 0; q < b && q < len; ++q) d[q] = __ldg(r + q);
+        for (int q = bytes ? e : max(b, 0); q < len; ++q) d[q] = __ldg(r + q);
+    };
+    if (tid == 0) {
+        s_fail = 0;
+        for (int st = 0; st < kJtvStagesMax; ++st) mbar_init(bar0 + 8 * st, K);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncthreads();
+    const bool feeds = tid < K && !withhold;
+    int issued = 0;                                          // planes brought in (the feeding lanes)
+    if (feeds)
+        for (; issued < stages && z0 + issued <= zlast; ++issued) fill(z0 + issued, issued);
+    if (!RUNS) __syncthreads();                              // the floats copied one by one
+    bool bad = false;
+    auto wait = [&](int st, uint32_t ph) {
+        if (bad || mbar_try_wait(bar0 + 8 * st, ph)) return;
+        if (s_fail || !mbar_wait(bar0 + 8 * st, ph, wait_cycles)) {
+            bad = true;
+            s_fail = 1;
+        }
+    };
+    // The thread's four voxels, as two pairs: their places in the range
+    // (clamped to it) and, in `ok`, five bits each: inside, x-, x+, y-, y+.
+    const int lane = tid & 31;
+    int o[4];
+    unsigned ok = 0;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int v = n0 + (RUNS ? 4 * tid + i : i * kJtvThreads + tid);
+        const int yy = v / nx, x = v - yy * nx;
+        const bool in = v < sxy;
+        o[i] = in ? v - lo : (RUNS ? i : 0);
+        if (in)
+            ok |= (1u | (x > 0 ? 2u : 0u) | (x < nx - 1 ? 4u : 0u) | (yy > 0 ? 8u : 0u) | (yy < ny - 1 ? 16u : 0u))
+                  << (5 * i);
+    }
+    // RUNS: no lane's run lies at a y face
+    const bool ymid = RUNS && __all_sync(0xffffffffu, !(ok & 1u) || (ok & 24u) == 24u);
+    auto has = [&](int i, unsigned bit) { return (ok & (bit << (5 * i))) != 0; };
+    auto only = [&](float2 q, int h, unsigned bit) {       // the terms of the neighbours that exist
+        return make_float2(has(2 * h, bit) ? q.x : 0.0f, has(2 * h + 1, bit) ? q.y : 0.0f);
+    };
+    auto pair_at = [&](const float* p, int h, int d) {      // RUNS: both at once
+        if constexpr (RUNS) return *reinterpret_cast<const float2*>(p + o[2 * h] + d);
+        else return make_float2(p[o[2 * h] + d], p[o[2 * h + 1] + d]);
+    };
+    auto four_at = [&](const float* p, int d, float2 (&q)[2]) {
+        if constexpr (RUNS) {
+            const float4 v = *reinterpret_cast<const float4*>(p + o[0] + d);
+            q[0] = make_float2(v.x, v.y);
+            q[1] = make_float2(v.z, v.w);
+        } else {
+            q[0] = pair_at(p, 0, d);
+            q[1] = pair_at(p, 1, d);
+        }
+    };
+    // neighbour offset d of one voxel, 0 (the voxel itself) where it has none
+    auto off = [&](int i, int d, unsigned bit) { return has(i, bit) ? d : 0; };
+    float2 cu[K][2], zl[K][2];                               // plane z; squared differences to plane z - 1
+    Acc2 acc;
+    int st = 0;                                              // stage of plane z
+    uint32_t ph = 0;                                         // phase of the ring's current turn
+    wait(0, 0);
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        four_at(smem + k * slot + shift(k, z0), 0, cu[k]);
+        zl[k][0] = zl[k][1] = make_float2(0.f, 0.f);
+        if (z0 > 0 && (ok & 1u)) {
+            float2 dn[2];
+            const float* q = y + k * N + (IT)sxy * (z0 - 1) + lo;
+            if constexpr (RUNS) {
+                four_at(q, 0, dn);
+            } else {
+                dn[0] = make_float2(__ldg(q + o[0]), __ldg(q + o[1]));
+                dn[1] = make_float2(__ldg(q + o[2]), __ldg(q + o[3]));
+            }
+            zl[k][0] = sqdiff(dn[0], cu[k][0]);
+            zl[k][1] = sqdiff(dn[1], cu[k][1]);
+        }
+    }
+    for (int z = z0; z < z1; ++z) {
+        const bool above = z + 1 < nz;
+        const int su = st + 1 == stages ? 0 : st + 1;        // stage of plane z + 1
+        const uint32_t pu = su == 0 ? ph ^ 1u : ph;
+        if (above) wait(su, pu);
+        float2 uu[2];
+        // MID: every voxel of the warp has its y neighbours and plane z + 1 exists
+        auto plane = [&](auto mid) {
+            constexpr bool MID = decltype(mid)::value;
+#pragma unroll
+            for (int k = 0; k < K; ++k) {
+                const float* p = smem + (st * K + k) * slot + (RUNS ? 0 : shift(k, z));
+                const float* u = above ? smem + (su * K + k) * slot + (RUNS ? 0 : shift(k, z + 1)) : p;
+                const float2 a = cu[k][0], b = cu[k][1];
+                float2 up[2], ym[2], yp[2], s[2];
+                four_at(u, 0, up);
+                if constexpr (RUNS) {
+                    four_at(p, off(0, -nx, 8u), ym);
+                    four_at(p, off(0, nx, 16u), yp);
+                    float vl = __shfl_up_sync(0xffffffffu, b.y, 1);
+                    float vr = __shfl_down_sync(0xffffffffu, a.x, 1);
+                    if (lane == 0) vl = p[o[0] + off(0, -1, 2u)];
+                    if (lane == 31) vr = p[o[3] + off(3, 1, 4u)];
+                    const float ql = has(0, 2u) ? sqdiff(vl, a.x) : 0.0f, qr = has(3, 4u) ? sqdiff(vr, b.y) : 0.0f;
+                    const float q01 = sqdiff(a.y, a.x), q12 = sqdiff(b.x, a.y), q23 = sqdiff(b.y, b.x);
+                    const float2 h2 = make_float2(P.ihx2, P.ihx2);
+                    s[0] = __ffma2_rn(make_float2(q01, q12), h2, __fmul2_rn(make_float2(ql, q01), h2));
+                    s[1] = __ffma2_rn(make_float2(q23, qr), h2, __fmul2_rn(make_float2(q12, q23), h2));
+                } else {
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const int i = 2 * h, j = i + 1;
+                        const float2 xm = make_float2(p[o[i] + off(i, -1, 2u)], p[o[j] + off(j, -1, 2u)]);
+                        const float2 xp = make_float2(p[o[i] + off(i, 1, 4u)], p[o[j] + off(j, 1, 4u)]);
+                        ym[h] = make_float2(p[o[i] + off(i, -nx, 8u)], p[o[j] + off(j, -nx, 8u)]);
+                        yp[h] = make_float2(p[o[i] + off(i, nx, 16u)], p[o[j] + off(j, nx, 16u)]);
+                        s[h] = __fmul2_rn(only(sqdiff(xm, cu[k][h]), h, 2u), make_float2(P.ihx2, P.ihx2));
+                        s[h] = addmul(only(sqdiff(xp, cu[k][h]), h, 4u), P.ihx2, s[h]);
+                    }
+                }
+                const float2 l2 = make_float2(P.lambda[k], P.lambda[k]);
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    float2 ya = sqdiff(ym[h], cu[k][h]), yb = sqdiff(yp[h], cu[k][h]);
+                    float2 zu = sqdiff(up[h], cu[k][h]);
+                    if (!MID) {
+                        ya = only(ya, h, 8u);
+                        yb = only(yb, h, 16u);
+                        if (!above) zu = make_float2(0.f, 0.f);
+                    }
+                    s[h] = addmul(ya, P.ihy2, s[h]);
+                    s[h] = addmul(yb, P.ihy2, s[h]);
+                    s[h] = addmul(zl[k][h], P.ihz2, s[h]);
+                    s[h] = addmul(zu, P.ihz2, s[h]);
+                    zl[k][h] = zu;
+                    cu[k][h] = up[h];
+                    uu[h] = k == 0 ? __fmul2_rn(l2, s[h]) : __ffma2_rn(l2, s[h], uu[h]);
+                }
+            }
+        };
+        if (RUNS && ymid && above) plane(std::true_type());
+        else plane(std::false_type());
+        if (!bad) {
+            const float2 e2 = make_float2(P.eps2, P.eps2);
+            const float2 va = __fadd2_rn(uu[0], e2), vb = __fadd2_rn(uu[1], e2);
+            float2 sa, sb, ra, rb;
+            const float vmin = fminf(fminf(va.x, va.y), fminf(vb.x, vb.y));
+            const float vmax = fmaxf(fmaxf(va.x, va.y), fmaxf(vb.x, vb.y));
+            const float vsum = (va.x + va.y) + (vb.x + vb.y);        // NaN if any value is
+            if (vmin >= 1e-30f && vmax <= 1e30f && vsum == vsum) {
+                sqrt_recip(va, sa, ra);
+                sqrt_recip(vb, sb, rb);
+            } else {
+                sa = make_float2(sqrtf(va.x), sqrtf(va.y));
+                sb = make_float2(sqrtf(vb.x), sqrtf(vb.y));
+                ra = make_float2(1.0f / sa.x, 1.0f / sa.y);
+                rb = make_float2(1.0f / sb.x, 1.0f / sb.y);
+            }
+            acc.add(only(sa, 0, 1u));
+            acc.add(only(sb, 1, 1u));
+            if (w) {
+                float* wz = w + (IT)sxy * z + lo;
+                if (RUNS) {
+                    if (ok & 1u) *reinterpret_cast<float4*>(wz + o[0]) = make_float4(ra.x, ra.y, rb.x, rb.y);
+                } else {
+                    if (has(0, 1u)) wz[o[0]] = ra.x;
+                    if (has(1, 1u)) wz[o[1]] = ra.y;
+                    if (has(2, 1u)) wz[o[2]] = rb.x;
+                    if (has(3, 1u)) wz[o[3]] = rb.y;
+                }
+            }
+        }
+        __syncthreads();
+        // every thread has read plane z: its stage takes the next plane
+        // (unless a wait gave up: no second copy in flight to a stage)
+        if (feeds && !s_fail && z0 + issued <= zlast) {
+            fill(z0 + issued, st);
+            ++issued;
+        }
+        st = su;
+        ph = pu;
+    }
+    if (s_fail) {
+        // drain: the last copies into each stage (earlier ones were waited for)
+        if (tid == 0) {
+            for (int i = max(0, issued - stages); i < issued; ++i)
+                mbar_wait(bar0 + 8 * (i % stages), (uint32_t)(i / stages) & 1u, wait_cycles);
+            if (status) atomicOr(status, kStatusTimeout);
+        }
+        __syncthreads();
+    }
+    Acc v[1] = {acc.sum()};
+    double out[1];
+    if (grid_reduce<1>(v, red, out, vg) && threadIdx.x == 0) *jtv = out[0];
+}
+
+template <int K, bool RUNS, typename IT>
+__global__ void __launch_bounds__(kJtvThreads, 2)
+    k_jtv_staged(DevProblem P, int zc, int stages, const float* __restrict__ y, float* __restrict__ w,
+                 double* jtv, Reduce red, unsigned* status, long long wait_cycles, int withhold)
+{
+    jtv_staged_body<K, RUNS, IT>(P, zc, stages, y, w, jtv, red, status, wait_cycles, withhold, hw_grid());
+}
+
+template <int K, bool RUNS, typename IT>
+__global__ void __launch_bounds__(kJtvThreads, 2)
+    k_jtv_staged_batch(const __grid_constant__ Batch<JtvArgs> b, long long wait_cycles, int withhold)
+{
+    const int s = batch_subject(b.start, b.n);
+    const JtvArgs& a = b.a[s];
+    jtv_staged_body<K, RUNS, IT>(a.P, a.zc, a.stages, a.y, a.w, a.jtv, a.red, a.status, wait_cycles, withhold,
+                           batch_grid(b.start[s], a.gx, a.gy, a.gz));
+}
+
+// The tile kernel, for rows too wide for three stages.
 // Each thread marches up its z range with the centre values of planes z - 1,
 // z and z + 1 in registers; the centre of plane z + 2 is loaded one plane
 // ahead.  The x / y neighbours come from the plane's tile in shared memory
@@ -514,20 +860,112 @@ StencilGrid stencil_grid(const DevProblem& P, int tx, int ty, int waves, double 
     return sg;
 }
 
-cudaError_t launch_jtv(const DevProblem& P, const float* y, float* w, double* jtv, Reduce red,
-                       cudaStream_t st)
+// Stages of the staged JTV kernel for this volume: as many as leave two blocks
+// per SM, at least three (plane z, plane z + 1 and one in flight) within a
+// block's shared memory; 0 (the tile kernel) where those do not fit, rows of
+// more than about 1900 voxels at K = 4, and for small volumes, where the staged
+// kernel's longer start-up costs what it gives (64^3: 14.3 us staged, 14.6 not;
+// without runs of four, 61^3: 15.4 and 12.9; 181x217x181: 58 and 78).
+constexpr long long kJtvStagedMinRuns = 1LL << 17, kJtvStagedMin = 1LL << 20;
+constexpr int kJtvSmemHalf = 110 * 1024, kJtvSmemMax = 220 * 1024;
+
+static int jtv_smem(const DevProblem& P, int stages) { return 4 * P.K * jtv_slot(P.nx) * stages; }
+
+static bool jtv_runs(const DevProblem& P, const float* y, const float* w)
 {
-    const StencilGrid sg = stencil_grid(P, kTileX, kTileY);
-    LaunchScope ls(MPM_KERNEL_JTV, st);
-    const bool i32 = index32(P);
-    if (P.K == 4) {
-        if (i32) k_jtv<4, int><<<sg.grid, sg.block, 0, st>>>(P, sg.zc, y, w, jtv, red);
-        else k_jtv<4, long long><<<sg.grid, sg.block, 0, st>>>(P, sg.zc, y, w, jtv, red);
-    } else {
-        if (i32) k_jtv<3, int><<<sg.grid, sg.block, 0, st>>>(P, sg.zc, y, w, jtv, red);
-        else k_jtv<3, long long><<<sg.grid, sg.block, 0, st>>>(P, sg.zc, y, w, jtv, red);
+    return P.nx % 4 == 0 && (reinterpret_cast<uintptr_t>(y) | reinterpret_cast<uintptr_t>(w)) % 16 == 0;
+}
+
+static int jtv_stages(const DevProblem& P, const float* y, const float* w)
+{
+    if (P.N < (jtv_runs(P, y, w) ? kJtvStagedMinRuns : kJtvStagedMin)) return 0;
+    for (int n = kJtvStagesMax; n >= 3; --n)
+        if (jtv_smem(P, n) <= (n > 3 ? kJtvSmemHalf : kJtvSmemMax)) return n;
+    return 0;
+}
+
+// Grid of the JTV kernel.  Staged: blocks over the voxels of a plane times z
+// ranges, the split of tma_chunks over the resident blocks (a range also reads
+// the planes below and above it, as an item of the PCG iteration does); a
+// subject that shares a launch takes `share` of the blocks.
+static void jtv_grid(const DevProblem& P, int stages, double share, JtvArgs& a)
+{
+    a.stages = stages;
+    if (!stages) {
+        const StencilGrid sg = stencil_grid(P, kTileX, kTileY, 2, share);
+        a.zc = sg.zc;
+        a.gx = sg.grid.x;
+        a.gy = sg.grid.y;
+        a.gz = sg.grid.z;
+        return;
     }
+    const long long bx = ((long long)P.nx * P.ny + kJtvRun - 1) / kJtvRun;
+    const int per_sm = jtv_smem(P, stages) <= kJtvSmemHalf ? 2 : 1;
+    const int gz = tma_chunks(bx, P.nz, std::max(1LL, (long long)(share * per_sm * kNumSm)));
+    a.zc = (P.nz + gz - 1) / gz;
+    a.gx = (unsigned)bx;
+    a.gy = 1;
+    a.gz = (unsigned)((P.nz + a.zc - 1) / a.zc);
+}
+
+template <int K, bool RUNS, typename IT>
+static cudaError_t jtv_smem_opt_in()
+{
+    static bool done = false;
+    if (done) return cudaSuccess;
+    cudaError_t e = cudaFuncSetAttribute(k_jtv_staged<K, RUNS, IT>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, kJtvSmemMax);
+    if (!e)
+        e = cudaFuncSetAttribute(k_jtv_staged_batch<K, RUNS, IT>,
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, kJtvSmemMax);
+    done = e == cudaSuccess;
+    return e;
+}
+
+template <int K>
+static cudaError_t prime_jtv_k()
+{
+    cudaError_t e = jtv_smem_opt_in<K, true, int>();
+    if (!e) e = jtv_smem_opt_in<K, true, long long>();
+    if (!e) e = jtv_smem_opt_in<K, false, int>();
+    if (!e) e = jtv_smem_opt_in<K, false, long long>();
+    return e;
+}
+
+cudaError_t prime_jtv_kernels()
+{
+    const cudaError_t e = prime_jtv_k<4>();
+    return e ? e : prime_jtv_k<3>();
+}
+
+template <int K, bool RUNS, typename IT>
+static cudaError_t launch_jtv_staged(const JtvArgs& a, cudaStream_t st)
+{
+    const cudaError_t e = jtv_smem_opt_in<K, RUNS, IT>();
+    if (e) return e;
+    k_jtv_staged<K, RUNS, IT><<<dim3(a.gx, a.gy, a.gz), kJtvThreads, jtv_smem(a.P, a.stages), st>>>(
+        a.P, a.zc, a.stages, a.y, a.w, a.jtv, a.red, a.status, copy_wait_cycles(), copy_withhold());
     return cudaGetLastError();
+}
+
+template <int K, typename IT>
+static cudaError_t launch_jtv_k(const JtvArgs& a, cudaStream_t st)
+{
+    if (a.stages)
+        return jtv_runs(a.P, a.y, a.w) ? launch_jtv_staged<K, true, IT>(a, st)
+                                       : launch_jtv_staged<K, false, IT>(a, st);
+    k_jtv<K, IT><<<dim3(a.gx, a.gy, a.gz), dim3(kTileX, kTileY, 1), 0, st>>>(a.P, a.zc, a.y, a.w, a.jtv, a.red);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_jtv(const DevProblem& P, const float* y, float* w, double* jtv, Reduce red,
+                       unsigned* status, cudaStream_t st)
+{
+    JtvArgs a{P, 0, 0, 0, 0, 0, y, w, jtv, red, status};
+    jtv_grid(P, jtv_stages(P, y, w), 1.0, a);
+    LaunchScope ls(MPM_KERNEL_JTV, st);
+    if (P.K == 4) return index32(P) ? launch_jtv_k<4, int>(a, st) : launch_jtv_k<4, long long>(a, st);
+    return index32(P) ? launch_jtv_k<3, int>(a, st) : launch_jtv_k<3, long long>(a, st);
 }
 
 // What iteration j of a solve does besides the common work.
@@ -652,22 +1090,54 @@ cudaError_t tma_autotune(const DevProblem& P, void* solve_ws, WsHeader* hdr, Red
 
 SolveBufs solve_bufs(const DevProblem& P, void* solve_ws) { return carve(P, solve_ws); }
 
-cudaError_t launch_jtv_batch(int K, const JtvArgs* a, const unsigned* blocks, int n, cudaStream_t st)
+template <int K, bool RUNS, typename IT>
+static cudaError_t launch_jtv_batch_staged(int smem, const Batch<JtvArgs>& b, cudaStream_t st)
 {
-    Batch<JtvArgs> b;
-    fill_batch(b, a, blocks, n);
-    bool i32 = true;
-    for (int i = 0; i < n; ++i) i32 = i32 && index32(a[i].P);
-    LaunchScope ls(MPM_KERNEL_JTV, st);
-    const dim3 blk(kTileX, kTileY, 1);
-    if (K == 4) {
-        if (i32) k_jtv_batch<4, int><<<b.start[n], blk, 0, st>>>(b);
-        else k_jtv_batch<4, long long><<<b.start[n], blk, 0, st>>>(b);
-    } else {
-        if (i32) k_jtv_batch<3, int><<<b.start[n], blk, 0, st>>>(b);
-        else k_jtv_batch<3, long long><<<b.start[n], blk, 0, st>>>(b);
-    }
+    const cudaError_t e = jtv_smem_opt_in<K, RUNS, IT>();
+    if (e) return e;
+    k_jtv_staged_batch<K, RUNS, IT><<<b.start[b.n], kJtvThreads, smem, st>>>(b, copy_wait_cycles(),
+                                                                             copy_withhold());
     return cudaGetLastError();
+}
+
+template <int K, typename IT>
+static cudaError_t launch_jtv_batch_k(bool staged, bool runs, int smem, const Batch<JtvArgs>& b,
+                                      cudaStream_t st)
+{
+    if (staged)
+        return runs ? launch_jtv_batch_staged<K, true, IT>(smem, b, st)
+                    : launch_jtv_batch_staged<K, false, IT>(smem, b, st);
+    k_jtv_batch<K, IT><<<b.start[b.n], dim3(kTileX, kTileY, 1), 0, st>>>(b);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_jtv_batch(int K, const JtvArgs* a, const double* share, int n, cudaStream_t st)
+{
+    // one kernel for the whole launch: staged if every subject can take it
+    static thread_local Batch<JtvArgs> b;
+    unsigned blocks[kBatchMax];
+    JtvArgs args[kBatchMax];
+    bool i32 = true, staged = true, runs = true;
+    for (int i = 0; i < n; ++i) {
+        i32 = i32 && index32(a[i].P);
+        staged = staged && jtv_stages(a[i].P, a[i].y, a[i].w) > 0;
+        runs = runs && jtv_runs(a[i].P, a[i].y, a[i].w);
+    }
+    int smem = 0;
+    for (int i = 0; i < n; ++i) {
+        args[i] = a[i];
+        const int stages = staged ? jtv_stages(a[i].P, a[i].y, a[i].w) : 0;
+        jtv_grid(a[i].P, stages, share[i], args[i]);
+        blocks[i] = args[i].gx * args[i].gy * args[i].gz;
+        smem = std::max(smem, jtv_smem(a[i].P, stages));
+    }
+    fill_batch(b, args, blocks, n);
+    LaunchScope ls(MPM_KERNEL_JTV, st);
+    if (K == 4)
+        return i32 ? launch_jtv_batch_k<4, int>(staged, runs, smem, b, st)
+                   : launch_jtv_batch_k<4, long long>(staged, runs, smem, b, st);
+    return i32 ? launch_jtv_batch_k<3, int>(staged, runs, smem, b, st)
+               : launch_jtv_batch_k<3, long long>(staged, runs, smem, b, st);
 }
 
 cudaError_t launch_pcg_init_batch(int K, const InitArgs* a, const unsigned* blocks, int n,
