@@ -378,7 +378,7 @@ static cudaError_t fit_enqueue_updates(const FitJob& j, cudaStream_t st, int* it
         if ((e = launch_lik(j, it, st))) return e;
         if (it >= j.opts.gn_iters) break;
         if ((e = launch_solve(P, solve_opts(j.opts), L.h, L.w, L.g, j.y, nullptr, j.y,
-                              nullptr, L.cg_rel + it, L.cg_it + it, L.solve, L.hdr, L.red, st)))
+                              nullptr, L.cg_rel + it, L.cg_it + it, L.solve, solve_ws_bytes(P), L.hdr, L.red, st)))
             return e;
     }
     if (j.var) {
@@ -417,7 +417,7 @@ static mpm_status fit_run_adaptive(const FitJob& j, cudaStream_t st, int* iters_
         }
         F_prev = F;
         MPM_CUDA(launch_solve(P, solve_opts(j.opts), L.h, L.w, L.g, j.y, nullptr, j.y,
-                              nullptr, L.cg_rel + it, L.cg_it + it, L.solve, L.hdr, L.red, st));
+                              nullptr, L.cg_rel + it, L.cg_it + it, L.solve, solve_ws_bytes(P), L.hdr, L.red, st));
     }
     if (j.var) {
         if (!w_fresh) MPM_CUDA(launch_jtv(P, j.y, L.w, L.jtv + MPM_MAX_REPORT + 1, L.red, &L.hdr->status, st));
@@ -692,7 +692,7 @@ static void plan_phased(FitJob* jobs, int n, std::vector<std::vector<PhasedSubje
         PhasedSubject ps;
         ps.j = &j;
         ps.B = solve_bufs(j.P, j.L.solve);
-        if (!make_step_maps(j.P, j.L.h, j.L.w, ps.B, tile, &ps.maps)) continue;
+        if (!make_step_maps(j.P, j.L.h, j.L.w, j.P.nx, ps.B, tile, &ps.maps)) continue;
 
         rest[i] = 0;
         const long long key = phased_class(j, tile);
@@ -1072,7 +1072,7 @@ mpm_status mpm_solve(const mpm_problem* problem, const mpm_opts* opts, const flo
     MPM_TRY(check_ws(P, MPM_CALL_SOLVE, ws, ws_bytes, L));
     MPM_CUDA(cudaMemsetAsync(L.hdr, 0, sizeof(WsHeader), st));
     MPM_CUDA(launch_solve(P, solve_opts(*opts), h, w, g, y, delta, nullptr, resid,
-                          nullptr, nullptr, L.solve, L.hdr, L.red, st));
+                          nullptr, nullptr, L.solve, solve_ws_bytes(P), L.hdr, L.red, st));
     return MPM_OK;
 }
 

@@ -111,9 +111,10 @@ SolveOpts solve_opts(const mpm_opts& o, bool overlap = true);
 cudaError_t launch_solve(const DevProblem& P, const SolveOpts& so, const float* h,
                          const float* w, const float* g, const float* y, float* delta,
                          float* y_update, double* resid, double* report_rel,
-                         int* report_it, void* solve_ws, WsHeader* hdr, Reduce red,
+                         int* report_it, void* solve_ws, size_t ws_bytes, WsHeader* hdr, Reduce red,
                          cudaStream_t st);
-size_t solve_ws_bytes(const DevProblem& P);   // enough for either solver
+size_t solve_ws_bytes(const DevProblem& P);   // enough for either solver, padded rows included
+size_t solve_ws_least(const DevProblem& P);   // without room for padded rows (plain iteration where needed)
 size_t mg_ws_bytes(const DevProblem& P);      // multigrid.cu
 cudaError_t launch_solve_mg(const DevProblem& P, const SolveOpts& o, const float* h, const float* w,
                             const float* g, const float* y, float* delta, float* y_update,
@@ -131,8 +132,10 @@ struct StepMaps {
     int tile;          // index of the tile shape the maps were encoded for
 };
 int tma_tile_count();
-bool make_step_maps(const DevProblem& P, const float* h, const float* w, const SolveBufs& B,
+// h and w have rows of `pitch` floats.
+bool make_step_maps(const DevProblem& P, const float* h, const float* w, int pitch, const SolveBufs& B,
                     int tile, StepMaps* out);
+bool tma_tile_fits(const DevProblem& P, int tile);   // the tile's boxes are no larger than the volume
 StencilGrid tma_grid(const DevProblem& P, int tile);
 cudaError_t prime_tma_kernels();   // shared-memory opt-ins, done before any graph capture
 cudaError_t prime_voxel_kernels(); // those of the staged voxel pass (voxel_tma.cu)

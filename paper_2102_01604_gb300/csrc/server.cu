@@ -254,7 +254,7 @@ mpm_status mpm_server_step(mpm_server* s, int* n_active, int* n_queued, int* n_f
                 r.F_prev = F;
                 const FitWs& L = r.L;
                 SRV_CUDA(launch_solve(r.P, solve_opts(r.opts, false), L.h, L.w, L.g, r.y, nullptr,
-                                      r.y, nullptr, L.cg_rel + r.it, L.cg_it + r.it, L.solve, L.hdr,
+                                      r.y, nullptr, L.cg_rel + r.it, L.cg_it + r.it, L.solve, solve_ws_bytes(r.P), L.hdr,
                                       L.red, r.stream));
                 r.it += 1;
                 st = srv_eval(s, r);

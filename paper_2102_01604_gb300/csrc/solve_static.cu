@@ -65,7 +65,8 @@ extern "C" mpm_status mpm_solve_static(const mpm_problem* problem, const mpm_opt
         }
         return MPM_OK;
     }
-    const size_t need = kHeaderBytes + kPartialBytes + solve_ws_bytes(P);
+    // (padded copies of w and H where there is room for them, see launch_solve)
+    const size_t need = kHeaderBytes + kPartialBytes + solve_ws_least(P);
     if (need > kStaticScratchBytes)
         return fail(MPM_ERR_WORKSPACE_TOO_SMALL,
                     "mpm_solve_static: this problem needs %zu bytes of scratch but the fixed "
@@ -73,7 +74,7 @@ extern "C" mpm_status mpm_solve_static(const mpm_problem* problem, const mpm_opt
                     "caller workspace",
                     need, kStaticScratchBytes,
                     (long long)((kStaticScratchBytes - kHeaderBytes - kPartialBytes) /
-                                (solve_ws_bytes(P) / (P.N > 0 ? P.N : 1))),
+                                (solve_ws_least(P) / (P.N > 0 ? P.N : 1))),
                     P.K);
     if ((s = check_dev(h, "h", false, 4)) != MPM_OK) return s;
     if ((s = check_dev(w, "w", false, 4)) != MPM_OK) return s;
@@ -94,7 +95,7 @@ extern "C" mpm_status mpm_solve_static(const mpm_problem* problem, const mpm_opt
     cudaError_t e = cudaMemsetAsync(hdr, 0, sizeof(WsHeader), st);
     if (e != cudaSuccess) return fail(MPM_ERR_CUDA, "cudaMemsetAsync: %s", cudaGetErrorString(e));
     e = launch_solve(P, solve_opts(*opts), h, w, g, y, delta, nullptr, resid, nullptr,
-                     nullptr, solve, hdr, red, st);
+                     nullptr, solve, kStaticScratchBytes - kHeaderBytes - kPartialBytes, hdr, red, st);
     if (e != cudaSuccess) return fail(MPM_ERR_CUDA, "launch: %s", cudaGetErrorString(e));
     return MPM_OK;
 }

@@ -527,13 +527,44 @@ __global__ void __launch_bounds__(kBlock) k_jtv_batch(const __grid_constant__ Ba
 
 static size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 
-// v[2], p[3] and x, each [N] float4; or the multigrid solver's
-// buffers (multigrid.cu), whichever is larger.
+// v[2], p[3] and x, each [N] float4.
+static size_t pcg_bytes(const DevProblem& P) { return 6 * align256(sizeof(float4) * (size_t)P.N); }
+
+// Copies of w and H with rows padded to a multiple of 4 floats (16 bytes), the
+// row pitch the copy engine needs, for volumes whose x size is not one: the
+// staged iteration then applies to them too.  The PCG start writes them as it
+// reads w and H.  Solve of 181x217x181, 30 iterations: 9.61 ms with the plain
+// iteration, 5.36 ms this way.
+struct PackedRows {
+    int pitch;           // floats per row
+    size_t plane;        // floats per array
+    float *w, *h;        // [plane], [T][plane]
+};
+
+static size_t packed_rows(const DevProblem& P, char* at, PackedRows* out)
+{
+    PackedRows r;
+    r.pitch = (P.nx + 3) / 4 * 4;
+    r.plane = (size_t)r.pitch * P.ny * P.nz;
+    const size_t w = align256(sizeof(float) * r.plane);
+    r.w = reinterpret_cast<float*>(at);
+    r.h = at ? reinterpret_cast<float*>(at + w) : nullptr;
+    if (out) *out = r;
+    return w + align256(sizeof(float) * P.T * r.plane);
+}
+
+static bool wants_packed(const DevProblem& P)
+{
+    return P.nx % 4 != 0 && tma_tile_fits(P, tma_tile_choice(P));
+}
+
+size_t solve_ws_least(const DevProblem& P) { return std::max(pcg_bytes(P), mg_ws_bytes(P)); }
+
+// The larger of the two solvers' needs; with rows to pad, room for their copies.
 size_t solve_ws_bytes(const DevProblem& P)
 {
-    const size_t pcg = 6 * align256(sizeof(float4) * (size_t)P.N);
-    const size_t mg = mg_ws_bytes(P);
-    return pcg > mg ? pcg : mg;
+    const size_t least = solve_ws_least(P);
+    return P.nx % 4 ? std::max(least, pcg_bytes(P) + packed_rows(P, nullptr, nullptr)) : least;
 }
 
 SolveOpts solve_opts(const mpm_opts& o, bool overlap)
@@ -567,7 +598,7 @@ __device__ __forceinline__ void pcg_init_body(const DevProblem& P, int zc, const
                                               const float* __restrict__ w, const float* __restrict__ g,
                                               const float* __restrict__ y, float4* __restrict__ p0,
                                               double tol2, WsHeader* hdr, double* resid, Reduce red,
-                                              const VGrid& vg)
+                                              const PackedRows& rows, const VGrid& vg)
 {
     constexpr int T = K * (K + 1) / 2;
     const long long N = P.N;
@@ -610,6 +641,12 @@ __device__ __forceinline__ void pcg_init_body(const DevProblem& P, int zc, const
             float hv[T], M[K][K];
 #pragma unroll
             for (int t = 0; t < T; ++t) hv[t] = __ldg(h + t * N + n);
+            if (rows.w) {
+                const size_t np = x + (size_t)rows.pitch * (yy + (size_t)P.ny * z);
+                rows.w[np] = wn;
+#pragma unroll
+                for (int t = 0; t < T; ++t) rows.h[t * rows.plane + np] = hv[t];
+            }
             precond_block<K>(P, hv, edge_sum(e.c), M);
             float L[T], zz[K];
             pd &= cholesky_f32<K>(M, L);
@@ -654,9 +691,9 @@ __global__ void __launch_bounds__(kBlock) k_pcg_init(DevProblem P, int zc, const
                                                      const float* __restrict__ g,
                                                      const float* __restrict__ y, float4* __restrict__ p0,
                                                      double tol2, WsHeader* hdr, double* resid,
-                                                     Reduce red)
+                                                     Reduce red, PackedRows rows)
 {
-    pcg_init_body<K>(P, zc, h, w, g, y, p0, tol2, hdr, resid, red, hw_grid());
+    pcg_init_body<K>(P, zc, h, w, g, y, p0, tol2, hdr, resid, red, rows, hw_grid());
 }
 
 template <int K>
@@ -664,7 +701,7 @@ __global__ void __launch_bounds__(kBlock) k_pcg_init_batch(const __grid_constant
 {
     const int s = batch_subject(b.start, b.n);
     const InitArgs& a = b.a[s];
-    pcg_init_body<K>(a.P, a.zc, a.h, a.w, a.g, a.y, a.p0, a.tol2, a.hdr, a.resid, a.red,
+    pcg_init_body<K>(a.P, a.zc, a.h, a.w, a.g, a.y, a.p0, a.tol2, a.hdr, a.resid, a.red, PackedRows{},
                      batch_grid(b.start[s], a.gx, a.gy, a.gz));
 }
 
@@ -673,7 +710,7 @@ __global__ void __launch_bounds__(kBlock) k_pcg_init_batch(const __grid_constant
 // Plain form of one PCG iteration (pcg_step.cuh): a thread per (x, y) column
 // marching a run of z planes; each neighbour's p_j is formed from its own
 // p_{j-1}, v_{j-1} and p_{j-2} read from memory.  Used for volumes or pointers the TMA kernel
-// cannot take (nx not a multiple of 4, a volume smaller than a tile).
+// cannot take (a volume smaller than a tile, unaligned buffers).
 template <int K, int MODE>
 __global__ void __launch_bounds__(kBlock) k_pcg_step(DevProblem P, int zc, int j, int want_rr,
                                                      const float* __restrict__ h,
@@ -1004,20 +1041,28 @@ template <int K>
 static cudaError_t solve_k(const DevProblem& P, const SolveOpts& so, const float* h,
                            const float* w, const float* g, const float* y, float* delta,
                            float* y_update, double* resid, double* report_rel, int* report_it,
-                           void* solve_ws, WsHeader* hdr, Reduce red, cudaStream_t st)
+                           void* solve_ws, size_t ws_bytes, WsHeader* hdr, Reduce red, cudaStream_t st)
 {
     const StencilGrid sg = stencil_grid(P, kTileX, kTileY);
     const StencilGrid ig = stencil_grid(P, kTileX, kTileY, kInitWaves);
     SolveBufs B = carve(P, solve_ws);
     const int cg_iters = so.cg_iters;
     const double tol2 = so.tol_cg > 0.0 ? so.tol_cg * so.tol_cg : 0.0;
-    {
-        LaunchScope ls(MPM_KERNEL_PCG_INIT, st);
-        k_pcg_init<K><<<ig.grid, ig.block, 0, st>>>(P, ig.zc, h, w, g, y, B.p[0], tol2, hdr, resid, red);
-    }
     StepMaps maps;
     const int tile = tma_tile_choice(P);
-    const bool tma = tile >= 0 && make_step_maps(P, h, w, B, tile, &maps);
+    PackedRows rows{};
+    bool tma;
+    if (wants_packed(P) && ws_bytes >= pcg_bytes(P) + packed_rows(P, nullptr, nullptr)) {
+        packed_rows(P, static_cast<char*>(solve_ws) + pcg_bytes(P), &rows);
+        tma = make_step_maps(P, rows.h, rows.w, rows.pitch, B, tile, &maps);
+        if (!tma) rows = PackedRows{};
+    } else {
+        tma = make_step_maps(P, h, w, P.nx, B, tile, &maps);
+    }
+    {
+        LaunchScope ls(MPM_KERNEL_PCG_INIT, st);
+        k_pcg_init<K><<<ig.grid, ig.block, 0, st>>>(P, ig.zc, h, w, g, y, B.p[0], tol2, hdr, resid, red, rows);
+    }
     const StencilGrid tg = tma ? tma_grid(P, tile) : sg;
     const bool want_resid = resid != nullptr || tol2 > 0.0;
     for (int j = 0; j < cg_iters; ++j) {
@@ -1061,7 +1106,7 @@ cudaError_t tma_autotune(const DevProblem& P, void* solve_ws, WsHeader* hdr, Red
     for (int t = 0; t < tma_tile_count(); ++t) {
         ms[t] = -1.0f;
         StepMaps m;
-        if (!make_step_maps(P, h, w, B, t, &m)) continue;
+        if (!make_step_maps(P, h, w, P.nx, B, t, &m)) continue;
         const StencilGrid g = tma_grid(P, t);
         constexpr int reps = 5;
         for (int i = 0; i <= reps && e == cudaSuccess; ++i) {
@@ -1168,16 +1213,16 @@ cudaError_t launch_pcg_final_batch(int K, const FinalArgs* a, const unsigned* bl
 cudaError_t launch_solve(const DevProblem& P, const SolveOpts& so, const float* h,
                          const float* w, const float* g, const float* y, float* delta,
                          float* y_update, double* resid, double* report_rel, int* report_it,
-                         void* solve_ws, WsHeader* hdr, Reduce red, cudaStream_t st)
+                         void* solve_ws, size_t ws_bytes, WsHeader* hdr, Reduce red, cudaStream_t st)
 {
     if (so.mg_levels > 0)
         return launch_solve_mg(P, so, h, w, g, y, delta, y_update, resid, report_rel, report_it,
                                solve_ws, hdr, red, st);
     if (P.K == 4)
         return solve_k<4>(P, so, h, w, g, y, delta, y_update, resid, report_rel,
-                          report_it, solve_ws, hdr, red, st);
+                          report_it, solve_ws, ws_bytes, hdr, red, st);
     return solve_k<3>(P, so, h, w, g, y, delta, y_update, resid, report_rel,
-                      report_it, solve_ws, hdr, red, st);
+                      report_it, solve_ws, ws_bytes, hdr, red, st);
 }
 
 }  // namespace mpm

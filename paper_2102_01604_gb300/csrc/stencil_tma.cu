@@ -503,15 +503,22 @@ int tma_tile_choice(const DevProblem& P)
     return (P.nx >= 40 && P.ny >= 10) ? 1 : 0;    // 32 x 8 when it fits, else 16 x 16
 }
 
-bool make_step_maps(const DevProblem& P, const float* h, const float* w, const SolveBufs& B, int tile,
-                    StepMaps* out)
+bool tma_tile_fits(const DevProblem& P, int tile)
 {
     if (tile < 0 || tile >= tma_tile_count()) return false;
+    return P.nx >= kTileShapes[tile][0] + 8 && P.ny >= kTileShapes[tile][1] + 2;
+}
+
+bool make_step_maps(const DevProblem& P, const float* h, const float* w, int pitch, const SolveBufs& B,
+                    int tile, StepMaps* out)
+{
+    // boxes are kept no larger than the volume
+    if (!tma_tile_fits(P, tile)) return false;
     const int TX = kTileShapes[tile][0], TY = kTileShapes[tile][1];
     const int BX = TX + 2, BY = TY + 2, WX = TX + 8;
-    // The planar maps need 16-byte row strides (nx a multiple of 4); boxes
-    // are kept no larger than the volume; every base must be 16-byte aligned.
-    if (P.nx % 4 != 0 || P.nx < WX || P.ny < BY) return false;
+    // The planar maps need 16-byte row strides (a pitch of a multiple of 4
+    // floats); every base must be 16-byte aligned.
+    if (pitch % 4 != 0) return false;
     uintptr_t any = reinterpret_cast<uintptr_t>(h) | reinterpret_cast<uintptr_t>(w) |
                     reinterpret_cast<uintptr_t>(B.x);
     for (float4* v : B.v) any |= reinterpret_cast<uintptr_t>(v);
@@ -526,9 +533,10 @@ bool make_step_maps(const DevProblem& P, const float* h, const float* w, const S
     const cuuint32_t tilebox[3] = {(cuuint32_t)(4 * TX), (cuuint32_t)TY, 1};
     // planar arrays
     const cuuint64_t d3[3] = {nx, ny, nz};
-    const cuuint64_t s3[2] = {4 * nx, 4 * nx * ny};
+    const cuuint64_t row = 4 * (cuuint64_t)pitch;
+    const cuuint64_t s3[2] = {row, row * ny};
     const cuuint64_t dh[4] = {nx, ny, nz, (cuuint64_t)P.T};
-    const cuuint64_t sh[3] = {4 * nx, 4 * nx * ny, 4 * (cuuint64_t)P.N};
+    const cuuint64_t sh[3] = {row, row * ny, row * ny * nz};
     const cuuint32_t wbox[3] = {(cuuint32_t)WX, (cuuint32_t)BY, 1};
     const cuuint32_t hbox[4] = {(cuuint32_t)TX, (cuuint32_t)TY, 1, (cuuint32_t)P.T};
     auto f = [](const float4* v) { return reinterpret_cast<const float*>(v); };
