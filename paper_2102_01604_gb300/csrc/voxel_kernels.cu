@@ -206,6 +206,8 @@ constexpr float kPivotMin = 1e-2f;   // smallest equilibrated pivot of the float
 // factorization adds about K kappa(A) 2^-24, and kappa(A) is of the order of
 // 1 / (smallest pivot L_jj^2).  False, with nothing written, when a pivot is
 // below kPivotMin (or M_kk is not positive): such blocks take block_var_f64.
+// Every rounding is spelled out, so one voxel per thread and two give the same
+// bits.
 template <int K>
 __device__ __forceinline__ bool block_var_f32(const float (&M)[K][K], bool want_ld, float (&var)[K],
                                               float& ld)
@@ -220,23 +222,23 @@ __device__ __forceinline__ bool block_var_f32(const float (&M)[K][K], bool want_
 #pragma unroll
     for (int a = 0; a < K; ++a)
 #pragma unroll
-        for (int b = 0; b <= a; ++b) A[a][b] = M[a][b] * sc[a] * sc[b];
+        for (int b = 0; b <= a; ++b) A[a][b] = __fmul_rn(__fmul_rn(M[a][b], sc[a]), sc[b]);
     float L[K][K], inv[K];
-    float lsum = 0.0f;
+    float psum = 1.0f;              // product of the pivots, each in [kPivotMin, about 1]
 #pragma unroll
     for (int j = 0; j < K; ++j) {
         float p = A[j][j];
 #pragma unroll
-        for (int k = 0; k < j; ++k) p -= L[j][k] * L[j][k];
+        for (int k = 0; k < j; ++k) p = fmaf(-L[j][k], L[j][k], p);
         if (!(p >= kPivotMin)) return false;
         inv[j] = rsqrtf(p);
         L[j][j] = p * inv[j];
-        if (want_ld) lsum += logf(p) - 2.0f * logf(sc[j]);
+        psum *= p;
 #pragma unroll
         for (int i = j + 1; i < K; ++i) {
             float v = A[i][j];
 #pragma unroll
-            for (int k = 0; k < j; ++k) v -= L[i][k] * L[j][k];
+            for (int k = 0; k < j; ++k) v = fmaf(-L[i][k], L[j][k], v);
             L[i][j] = v * inv[j];
         }
     }
@@ -250,7 +252,7 @@ __device__ __forceinline__ bool block_var_f32(const float (&M)[K][K], bool want_
         for (int i = j + 1; i < K; ++i) {
             float v = 0.0f;
 #pragma unroll
-            for (int k = j; k < i; ++k) v -= L[i][k] * Li[k][j];
+            for (int k = j; k < i; ++k) v = fmaf(-L[i][k], Li[k][j], v);
             Li[i][j] = v * inv[i];
         }
     }
@@ -258,10 +260,19 @@ __device__ __forceinline__ bool block_var_f32(const float (&M)[K][K], bool want_
     for (int k = 0; k < K; ++k) {
         float v = 0.0f;
 #pragma unroll
-        for (int j = k; j < K; ++j) v += Li[j][k] * Li[j][k];
-        var[k] = v * sc[k] * sc[k];
+        for (int j = k; j < K; ++j) v = fmaf(Li[j][k], Li[j][k], v);
+        var[k] = __fmul_rn(__fmul_rn(v, sc[k]), sc[k]);
     }
-    ld = lsum;
+    if (want_ld) {
+        // log prod_j L_jj^2 + log prod_k M_kk, the diagonal multiplied in two
+        // pairs (three logarithms where one per factor took eight); a pair
+        // outside float32's comfortable range takes its logarithms apart
+        auto log2of = [](float a, float b) {
+            const float ab = a * b;
+            return ab > 1e-30f && ab < 1e30f ? logf(ab) : logf(a) + logf(b);
+        };
+        ld = logf(psum) + log2of(M[0][0], M[1][1]) + log2of(M[2][2], K == 4 ? M[K - 1][K - 1] : 1.0f);
+    }
     return true;
 }
 
@@ -385,19 +396,19 @@ __device__ __forceinline__ void uncertainty_body(const DevProblem& P, const floa
             // as each other's x neighbours
             const float wn = wc[v];
             float d32 = 0.0f;
-            if (x > 0) d32 += (wn + (v > 0 ? wc[v - 1] : __ldg(w + n - 1))) * P.ihx2;
-            if (x < P.nx - 1) d32 += (wn + (v + 1 < V ? wc[v + 1] : __ldg(w + n + 1))) * P.ihx2;
-            if (yy > 0) d32 += (wn + __ldg(w + n - P.nx)) * P.ihy2;
-            if (yy < P.ny - 1) d32 += (wn + __ldg(w + n + P.nx)) * P.ihy2;
-            if (z > 0) d32 += (wn + __ldg(w + n - sxy)) * P.ihz2;
-            if (z < P.nz - 1) d32 += (wn + __ldg(w + n + sxy)) * P.ihz2;
+            if (x > 0) d32 = fmaf(wn + (v > 0 ? wc[v - 1] : __ldg(w + n - 1)), P.ihx2, d32);
+            if (x < P.nx - 1) d32 = fmaf(wn + (v + 1 < V ? wc[v + 1] : __ldg(w + n + 1)), P.ihx2, d32);
+            if (yy > 0) d32 = fmaf(wn + __ldg(w + n - P.nx), P.ihy2, d32);
+            if (yy < P.ny - 1) d32 = fmaf(wn + __ldg(w + n + P.nx), P.ihy2, d32);
+            if (z > 0) d32 = fmaf(wn + __ldg(w + n - sxy), P.ihz2, d32);
+            if (z < P.nz - 1) d32 = fmaf(wn + __ldg(w + n + sxy), P.ihz2, d32);
             float M[K][K];
 #pragma unroll
             for (int a2 = 0; a2 < K; ++a2)
 #pragma unroll
                 for (int b2 = a2; b2 < K; ++b2) M[a2][b2] = M[b2][a2] = hv[tri(K, a2, b2)][v];
 #pragma unroll
-            for (int a2 = 0; a2 < K; ++a2) M[a2][a2] += P.lambda[a2] * d32;
+            for (int a2 = 0; a2 < K; ++a2) M[a2][a2] = fmaf(P.lambda[a2], d32, M[a2][a2]);
             ld[v] = 0.0f;
             if (!block_var_f32<K>(M, logdet != nullptr, vv[v], ld[v])) {
                 const double d = d32;
@@ -441,8 +452,11 @@ __device__ __forceinline__ void uncertainty_body(const DevProblem& P, const floa
     }
 }
 
+// Four blocks per SM: at 176x240x256 with logdet and moments 168 us, 186 us
+// with the three its registers allowed otherwise (196 us with one logarithm per
+// factor of the determinant besides).
 template <int K, int V>
-__global__ void __launch_bounds__(kBlock) k_uncertainty(DevProblem P, const float* __restrict__ h,
+__global__ void __launch_bounds__(kBlock, 4) k_uncertainty(DevProblem P, const float* __restrict__ h,
                                                         const float* __restrict__ w,
                                                         const float* __restrict__ y,
                                                         float* __restrict__ var,
