@@ -210,9 +210,11 @@ class ClockSampler:
 # ------------------------------------------------------------ roofline
 
 def step_bytes(j: int, K: int, cg_iters: int = None) -> int:
-    """Bytes PCG iteration j moves per voxel (pcg_step.cuh): j = 0 reads z_0, w,
-    H and writes p_0, v_0; later iterations read z, v, p, w, H and write z, v,
-    p; even j >= 2 also read p_{j-2} and write x, and read x when j > 2."""
+    """Bytes per voxel of PCG iteration j with the preconditioned residual z
+    stored, as a count of the method's operands: j = 0 reads z_0, w, H and
+    writes p_0, v_0; later iterations read z, v, p, w, H and write z, v, p; even
+    j >= 2 also read p_{j-2} and write x, and read x when j > 2.  The kernel
+    moves fewer (moved_step_bytes)."""
     T = K * (K + 1) // 2
     f = 4
     if j == 0:
@@ -220,6 +222,23 @@ def step_bytes(j: int, K: int, cg_iters: int = None) -> int:
     b = 3 * K * f + f + T * f + 3 * K * f
     if j >= 2 and j % 2 == 0:
         b += 2 * K * f + (K * f if j > 2 else 0)
+    return b
+
+
+def moved_step_bytes(j: int, K: int) -> int:
+    """Bytes per voxel of PCG iteration j as the kernel runs it (pcg_step.cuh:
+    z comes from the last two directions): j = 0 reads p_0, w, H and writes v_0;
+    j = 1 reads p_0, v_0, w, H and writes p, v; later ones also read p_{j-2};
+    even j >= 2 also write x, and read x when j > 2."""
+    T = K * (K + 1) // 2
+    f = 4
+    vec = 4 * f                                 # four floats per voxel whatever K is
+    b = f + T * f
+    if j == 0:
+        return b + 2 * vec
+    b += (2 if j == 1 else 3) * vec + 2 * vec
+    if j >= 2 and j % 2 == 0:
+        b += vec + (vec if j > 2 else 0)
     return b
 
 
@@ -254,7 +273,8 @@ def kernel_roofline(prof: dict, n_vox: int, steps: int, K: int, C: int, I: int, 
         if not v["launches"]:
             continue
         if kind == "pcg_step" and v["launches"] % CG_ITERS == 0:
-            total_bytes = ab["pcg_step_per_solve"] * n_vox * (v["launches"] // CG_ITERS)
+            per_solve = sum(moved_step_bytes(j, K) for j in range(CG_ITERS))
+            total_bytes = per_solve * n_vox * (v["launches"] // CG_ITERS)
         elif kind in ab:
             total_bytes = ab[kind] * n_vox * v["launches"]
         else:
@@ -284,7 +304,7 @@ def measured_peak():
 KIND_SOURCES = {
     "grad_hess": ["voxel_kernels.cu", "voxel_tma.cu", "voxel_model.cuh", "tma_common.cuh"],
     "uncertainty": ["voxel_kernels.cu"],
-    "jtv": ["stencil_kernels.cu"],
+    "jtv": ["stencil_kernels.cu", "tma_common.cuh"],
     "pcg_init": ["stencil_kernels.cu", "pcg_step.cuh"],
     "pcg_step": ["stencil_kernels.cu", "stencil_tma.cu", "pcg_step.cuh", "tma_common.cuh"],
     "pcg_final": ["stencil_kernels.cu", "pcg_step.cuh"],
@@ -322,11 +342,12 @@ def measured_traffic(kind: str, n_vox: int):
 # Kernel kind of each kernel function (the name before its template arguments).
 KERNEL_KIND = {
     "k_pcg_step_tma": "pcg_step", "k_pcg_step": "pcg_step", "k_pcg_init": "pcg_init",
-    "k_jtv": "jtv", "k_pcg_final": "pcg_final", "k_grad_hess": "grad_hess",
+    "k_jtv": "jtv", "k_jtv_staged": "jtv", "k_pcg_final": "pcg_final", "k_grad_hess": "grad_hess",
     "k_grad_hess_tma": "grad_hess", "k_uncertainty": "uncertainty",
     "k_grad_hess_proj": "grad_hess_proj", "k_push_all": "reslice",
     # the phase-batched forms (mpm_fit_batch with opts.graph = 2)
     "k_pcg_step_tma_batch": "pcg_step", "k_pcg_init_batch": "pcg_init", "k_jtv_batch": "jtv",
+    "k_jtv_staged_batch": "jtv",
     "k_pcg_final_batch": "pcg_final", "k_grad_hess_batch": "grad_hess",
     "k_grad_hess_tma_batch": "grad_hess", "k_uncertainty_batch": "uncertainty",
 }
