@@ -1,5 +1,6 @@
 // stencil_kernels.cu -- the prior and the Newton-system solve (sm_103a):
-//   k_jtv          JTV weights w_n = (u_n + eps^2)^-1/2 and JTV_eps (Eqs. 38-40)
+//   k_jtv_staged   JTV weights w_n = (u_n + eps^2)^-1/2 and JTV_eps (Eqs. 38-40);
+//                  k_jtv for small volumes and very wide rows
 //   k_pcg_init     r_0 = g + L y, p_0 = z_0 = M^-1 r_0 (Eq. 42)
 //   k_pcg_step     one PCG iteration (pcg_step.cuh): z_j, p_j from the previous
 //                  ones, q = (H + L) p_j, v = M^-1 q, the x fold and the

@@ -244,7 +244,7 @@ __device__ __forceinline__ void grad_hess_tma_body(const DevProblem& P, const XT
                         rho = make_float2(expf(dq.x), expf(dq.y));
                     }
                     float2 sg = make_float2(tc[0].s0 * e0.x, tc[1].s0 * e0.y);
-#pragma unroll 4
+#pragma unroll 2      // of 8 echoes: 4 at a time 514 us at 176x240x256, 2 at a time 507
                     for (int e = 0; e < ne; ++e) {
                         take(XT(), xv);
                         es.add(sg, q2, make_float2(xv[0], xv[1]));
