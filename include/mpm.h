@@ -243,7 +243,8 @@ mpm_status mpm_fit(const mpm_problem* problem, const mpm_opts* opts, const void*
  * call times each applicable shape on this volume (zeroed operands in `ws`, a
  * MPM_CALL_SOLVE-sized workspace or larger), keeps the fastest for every later
  * solve of a volume of this size in the process, and writes its index to
- * *tile (-1 when the TMA kernel does not apply: nx not a multiple of 4, or the
+ * *tile (-1 when it has nothing to time: nx not a multiple of 4, whose solves run
+ * the default shape on copies of w and H with padded rows, or the
  * volume smaller than a tile) and the mean time per launch of each shape to
  * ms[0..MPM_TILE_SHAPES-1] (-1 for shapes that do not apply; may be NULL).
  * If *tile >= 0 on entry, that shape is recorded without timing (ws may then
@@ -404,13 +405,15 @@ mpm_status mpm_server_destroy(mpm_server* server);
 /* Synchronises `stream` and returns MPM_ERR_NUMERIC if a kernel that used this
  * workspace recorded a failure since the workspace was last cleared (every
  * mpm_solve / mpm_fit clears it): a preconditioner block that is not positive
- * definite, a NaN in a reduction, or a bounded copy wait of the PCG iteration
- * or of the voxel pass that ran out (mpm_last_error() names which).  Every
- * mpm_grad_hess call clears it too.  Otherwise MPM_OK. */
+ * definite, a NaN in a reduction, or a bounded copy wait of the PCG iteration,
+ * the voxel pass or the JTV pass that ran out (mpm_last_error() names which).
+ * Every mpm_grad_hess and mpm_jtv_weights call clears it too.  Otherwise
+ * MPM_OK. */
 mpm_status mpm_workspace_status(const void* ws, size_t ws_bytes, void* stream);
 
 /* Test hook for the bounded waits of the staged kernels, the TMA-staged PCG
- * iteration and the staged voxel pass (the paper has no counterpart; tests
+ * iteration, the staged voxel pass and the staged JTV pass (the paper has no
+ * counterpart; tests
  * use it to drive the timeout path without a fault).  withhold != 0: from the
  * next launch on, their producers issue no copies, so every copy wait of
  * their compute warps runs out.
@@ -419,7 +422,7 @@ mpm_status mpm_workspace_status(const void* ws, size_t ws_bytes, void* stream);
  * A launch whose wait ran out skips its work, drains its own copies, records
  * the failure in the workspace status (mpm_workspace_status reports
  * MPM_ERR_NUMERIC, "copy wait timed out") and returns; the solve then stops
- * without a step, and the voxel pass leaves g and h undefined.  Process-wide.  Returns MPM_ERR_INVALID_ARG for
+ * without a step, the voxel pass leaves g and h undefined and the JTV pass w.  Process-wide.  Returns MPM_ERR_INVALID_ARG for
  * wait_us < 0. */
 mpm_status mpm_test_copy_timeout(int withhold, double wait_us);
 

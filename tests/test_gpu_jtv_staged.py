@@ -64,9 +64,37 @@ def test_jtv_staged_infinite_and_nan_maps():
         w = w.cpu().view(nz, ny, nx)
         near = [(0, 0, 0), (0, 0, 1), (0, 1, 0), (1, 0, 0)]
         for n in near:
-            assert (np.isnan(w[n]) if np.isnan(centre) else w[n] == 0.0), n
+            v = w[n].item()
+            assert (np.isnan(v) if np.isnan(centre) else v == 0.0), n
         rest = w.clone()
         for n in near:
             rest[n] = 1.0
         assert torch.isfinite(rest).all() and (rest > 0).all()
         assert not np.isfinite(e.item())
+
+
+@pytest.mark.parametrize("shape", [(64, 64, 33), (129, 95, 87)])
+def test_jtv_staged_copy_timeout(shape):
+    """Copies that never land (the test hook withholds them): the call returns,
+    the workspace records the timeout, and the next call on the same context
+    gives the weights again."""
+    import torch
+
+    import paper_2102_01604_gb300 as mpm
+    from paper_2102_01604_gb300 import _lib
+    p = mpm.make_problem(dataset((4, 4, 4), seed=11)["prot"], shape)
+    y = torch.randn((4, int(np.prod(shape))), device="cuda")
+    ws = mpm.workspace(p, None, _lib.CALL_JTV)
+    w0, e0 = (t.clone() for t in mpm.mpm_jtv_weights(p, y, ws=ws))
+    assert mpm.mpm_workspace_status(ws) == _lib.OK
+    mpm.mpm_test_copy_timeout(True, 1000.0)
+    try:
+        mpm.mpm_jtv_weights(p, y, ws=ws)
+        st = mpm.mpm_workspace_status(ws)
+        msg = _lib.load().mpm_last_error().decode()
+    finally:
+        mpm.mpm_test_copy_timeout(False, 0.0)
+    assert st == _lib.ERR_NUMERIC and "copy wait timed out" in msg
+    w, e = mpm.mpm_jtv_weights(p, y, ws=ws)
+    assert mpm.mpm_workspace_status(ws) == _lib.OK
+    assert torch.equal(w, w0) and torch.equal(e, e0)
