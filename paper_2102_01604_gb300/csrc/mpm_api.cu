@@ -261,7 +261,7 @@ static size_t al(size_t b) { return (b + 255) & ~(size_t)255; }
 
 constexpr int kMeanBlocksHost = 304;   // must match the launcher's cap
 
-FitWs layout(const DevProblem& P, int call, void* base)
+FitWs layout(const DevProblem& P, int call, void* base, bool padded)
 {
     FitWs L;
     memset(&L, 0, sizeof L);
@@ -287,18 +287,22 @@ FitWs layout(const DevProblem& P, int call, void* base)
         L.g = reinterpret_cast<float*>(take(vec));
         L.h = reinterpret_cast<float*>(take(sizeof(float) * (size_t)P.T * P.N));
     }
-    if (call == MPM_CALL_FIT || call == MPM_CALL_SOLVE) L.solve = take(solve_ws_bytes(P));
+    if (call == MPM_CALL_FIT || call == MPM_CALL_SOLVE) {
+        L.solve_bytes = padded ? solve_ws_bytes(P) : solve_ws_least(P);
+        L.solve = take(L.solve_bytes);
+    }
     L.total = off;
     return L;
 }
 
 mpm_status check_ws(const DevProblem& P, int call, void* ws, size_t ws_bytes, FitWs& L)
 {
-    const size_t need = layout(P, call, nullptr).total;
+    const size_t full = layout(P, call, nullptr).total;
+    const size_t need = layout(P, call, nullptr, false).total;
     if (ws_bytes < need)
         return fail(MPM_ERR_WORKSPACE_TOO_SMALL, "workspace of %zu bytes, %zu needed", ws_bytes, need);
     MPM_TRY(check_dev(ws, "ws", false, 256));
-    L = layout(P, call, ws);
+    L = layout(P, call, ws, ws_bytes >= full);
     return MPM_OK;
 }
 
@@ -378,7 +382,7 @@ static cudaError_t fit_enqueue_updates(const FitJob& j, cudaStream_t st, int* it
         if ((e = launch_lik(j, it, st))) return e;
         if (it >= j.opts.gn_iters) break;
         if ((e = launch_solve(P, solve_opts(j.opts), L.h, L.w, L.g, j.y, nullptr, j.y,
-                              nullptr, L.cg_rel + it, L.cg_it + it, L.solve, solve_ws_bytes(P), L.hdr, L.red, st)))
+                              nullptr, L.cg_rel + it, L.cg_it + it, L.solve, L.solve_bytes, L.hdr, L.red, st)))
             return e;
     }
     if (j.var) {
@@ -417,7 +421,7 @@ static mpm_status fit_run_adaptive(const FitJob& j, cudaStream_t st, int* iters_
         }
         F_prev = F;
         MPM_CUDA(launch_solve(P, solve_opts(j.opts), L.h, L.w, L.g, j.y, nullptr, j.y,
-                              nullptr, L.cg_rel + it, L.cg_it + it, L.solve, solve_ws_bytes(P), L.hdr, L.red, st));
+                              nullptr, L.cg_rel + it, L.cg_it + it, L.solve, L.solve_bytes, L.hdr, L.red, st));
     }
     if (j.var) {
         if (!w_fresh) MPM_CUDA(launch_jtv(P, j.y, L.w, L.jtv + MPM_MAX_REPORT + 1, L.red, &L.hdr->status, st));
@@ -1072,7 +1076,7 @@ mpm_status mpm_solve(const mpm_problem* problem, const mpm_opts* opts, const flo
     MPM_TRY(check_ws(P, MPM_CALL_SOLVE, ws, ws_bytes, L));
     MPM_CUDA(cudaMemsetAsync(L.hdr, 0, sizeof(WsHeader), st));
     MPM_CUDA(launch_solve(P, solve_opts(*opts), h, w, g, y, delta, nullptr, resid,
-                          nullptr, nullptr, L.solve, solve_ws_bytes(P), L.hdr, L.red, st));
+                          nullptr, nullptr, L.solve, L.solve_bytes, L.hdr, L.red, st));
     return MPM_OK;
 }
 
@@ -1116,7 +1120,12 @@ mpm_status mpm_autotune(const mpm_problem* problem, const mpm_opts* opts, void* 
     } else {
         FitWs L;
         MPM_TRY(check_ws(P, MPM_CALL_SOLVE, ws, ws_bytes, L));
-        MPM_CUDA(tma_autotune(P, L.solve, L.hdr, L.red, (cudaStream_t)stream, &best, t_ms));
+        if (L.solve_bytes < solve_ws_bytes(P)) {
+            // the solve takes the plain iteration in such a workspace
+            for (float& t : t_ms) t = -1.0f;
+        } else {
+            MPM_CUDA(tma_autotune(P, L.solve, L.hdr, L.red, (cudaStream_t)stream, &best, t_ms));
+        }
     }
     if (tile) *tile = best;
     if (ms)

@@ -198,10 +198,12 @@ struct FitWs {
     float* g;
     float* h;
     void* solve;
+    size_t solve_bytes;
     size_t total;
 };
 
-FitWs layout(const DevProblem& P, int call, void* base);   // base NULL: sizes only
+// base NULL: sizes only; without `padded`, no room for the solve's padded rows.
+FitWs layout(const DevProblem& P, int call, void* base, bool padded = true);
 
 // Spatial projection (projection.cu): per-contrast inputs on the acquisition
 // grids, and the opaque projection and workspace of one projected fit.

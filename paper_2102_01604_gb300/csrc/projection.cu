@@ -540,11 +540,11 @@ struct ProjWs {
     size_t total;
 };
 
-static ProjWs proj_layout(const DevProblem& P, const DevProj& Q, int call, void* base)
+static ProjWs proj_layout(const DevProblem& P, const DevProj& Q, int call, void* base, bool padded = true)
 {
     ProjWs W;
     memset(&W, 0, sizeof W);
-    W.L = layout(P, call, base);
+    W.L = layout(P, call, base, padded);
     size_t off = W.L.total;
     char* b = static_cast<char*>(base);
     auto take = [&](size_t bytes) -> char* {
@@ -764,12 +764,13 @@ mpm_status proj_prepare(const mpm_problem* problem, const mpm_projection* proj, 
     MPM_TRY(make_proj(problem, proj, *Q));
     MPM_TRY(check_proj_inputs(problem, *Q, x, b1p, b1m, pj.in));
     const DevProblem P = make_dev(problem);
-    const ProjWs need = proj_layout(P, *Q, MPM_CALL_FIT, nullptr);
+    const bool padded = ws_bytes >= proj_layout(P, *Q, MPM_CALL_FIT, nullptr).total;
+    const ProjWs need = proj_layout(P, *Q, MPM_CALL_FIT, nullptr, false);
     if (ws_bytes < need.total)
         return fail(MPM_ERR_WORKSPACE_TOO_SMALL, "workspace of %zu bytes, %zu needed", ws_bytes,
                     need.total);
     MPM_TRY(check_dev(ws, "ws", false, 256));
-    *W = proj_layout(P, *Q, MPM_CALL_FIT, ws);
+    *W = proj_layout(P, *Q, MPM_CALL_FIT, ws, padded);
     L = W->L;
     return MPM_OK;
 }

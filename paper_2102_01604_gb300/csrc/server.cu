@@ -43,6 +43,7 @@ struct Request {
     const float *b1p, *b1m;
     float *y, *var;
     size_t ws_off, ws_bytes;
+    bool padded;              // the workspace holds the solve's padded rows
     FitWs L;
     int slot;
     int overtaken;            // later requests admitted before this one
@@ -188,8 +189,11 @@ mpm_status mpm_server_submit(mpm_server* s, const mpm_problem* problem, const mp
     if ((st = check_dev(b1m, "b1m", true, 4)) != MPM_OK) return st;
     if ((st = check_dev(y, "y_inout", false, 4)) != MPM_OK) return st;
     if ((st = check_dev(var_out, "var_out", true, 4)) != MPM_OK) return st;
-    const size_t need = layout(P, MPM_CALL_FIT, nullptr).total;
     std::lock_guard<std::mutex> lk(s->mu);
+    // an arena without room for the padded rows of an odd x size still serves it
+    size_t need = layout(P, MPM_CALL_FIT, nullptr).total;
+    const bool padded = need <= s->arena.bytes;
+    if (!padded) need = layout(P, MPM_CALL_FIT, nullptr, false).total;
     if (need > s->arena.bytes)
         return fail(MPM_ERR_WORKSPACE_TOO_SMALL, "request needs %zu bytes, the arena holds %zu",
                     need, s->arena.bytes);
@@ -206,6 +210,7 @@ mpm_status mpm_server_submit(mpm_server* s, const mpm_problem* problem, const mp
     r.y = y;
     r.var = var_out;
     r.ws_bytes = need;
+    r.padded = padded;
     r.slot = -1;
     cudaError_t e = cudaEventCreateWithFlags(&r.ready, cudaEventDisableTiming);
     if (e != cudaSuccess) return fail(MPM_ERR_CUDA, "event: %s", cudaGetErrorString(e));
@@ -254,7 +259,7 @@ mpm_status mpm_server_step(mpm_server* s, int* n_active, int* n_queued, int* n_f
                 r.F_prev = F;
                 const FitWs& L = r.L;
                 SRV_CUDA(launch_solve(r.P, solve_opts(r.opts, false), L.h, L.w, L.g, r.y, nullptr,
-                                      r.y, nullptr, L.cg_rel + r.it, L.cg_it + r.it, L.solve, solve_ws_bytes(r.P), L.hdr,
+                                      r.y, nullptr, L.cg_rel + r.it, L.cg_it + r.it, L.solve, L.solve_bytes, L.hdr,
                                       L.red, r.stream));
                 r.it += 1;
                 st = srv_eval(s, r);
@@ -306,7 +311,7 @@ mpm_status mpm_server_step(mpm_server* s, int* n_active, int* n_queued, int* n_f
         for (auto q = s->queue.begin(); q != pick; ++q) s->reqs[*q].overtaken += 1;
         s->queue.erase(pick);
         a.ws_off = off;
-        a.L = layout(a.P, MPM_CALL_FIT, s->arena.base + off);
+        a.L = layout(a.P, MPM_CALL_FIT, s->arena.base + off, a.padded);
         a.slot = k;
         a.state = kActive;
         a.it = 0;
