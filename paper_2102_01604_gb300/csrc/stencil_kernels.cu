@@ -594,7 +594,11 @@ static SolveBufs carve(const DevProblem& P, void* ws)
 
 // --------------------------------------------------------------- PCG init
 
-template <int K>
+// PACKED: also writes the padded copies of w and H.  A template parameter,
+// because the test at run time took 58 registers instead of 48, one block per
+// SM less: 299 us instead of 233 at 176x240x256, where load latency bounds it
+// (bounds of 6 and 8 blocks per SM: 241 and 301 us).
+template <int K, bool PACKED>
 __device__ __forceinline__ void pcg_init_body(const DevProblem& P, int zc, const float* __restrict__ h,
                                               const float* __restrict__ w, const float* __restrict__ g,
                                               const float* __restrict__ y, float4* __restrict__ p0,
@@ -642,7 +646,7 @@ __device__ __forceinline__ void pcg_init_body(const DevProblem& P, int zc, const
             float hv[T], M[K][K];
 #pragma unroll
             for (int t = 0; t < T; ++t) hv[t] = __ldg(h + t * N + n);
-            if (rows.w) {
+            if constexpr (PACKED) {
                 const size_t np = x + (size_t)rows.pitch * (yy + (size_t)P.ny * z);
                 rows.w[np] = wn;
 #pragma unroll
@@ -686,7 +690,7 @@ __device__ __forceinline__ void pcg_init_body(const DevProblem& P, int zc, const
     }
 }
 
-template <int K>
+template <int K, bool PACKED>
 __global__ void __launch_bounds__(kBlock) k_pcg_init(DevProblem P, int zc, const float* __restrict__ h,
                                                      const float* __restrict__ w,
                                                      const float* __restrict__ g,
@@ -694,7 +698,7 @@ __global__ void __launch_bounds__(kBlock) k_pcg_init(DevProblem P, int zc, const
                                                      double tol2, WsHeader* hdr, double* resid,
                                                      Reduce red, PackedRows rows)
 {
-    pcg_init_body<K>(P, zc, h, w, g, y, p0, tol2, hdr, resid, red, rows, hw_grid());
+    pcg_init_body<K, PACKED>(P, zc, h, w, g, y, p0, tol2, hdr, resid, red, rows, hw_grid());
 }
 
 template <int K>
@@ -702,7 +706,7 @@ __global__ void __launch_bounds__(kBlock) k_pcg_init_batch(const __grid_constant
 {
     const int s = batch_subject(b.start, b.n);
     const InitArgs& a = b.a[s];
-    pcg_init_body<K>(a.P, a.zc, a.h, a.w, a.g, a.y, a.p0, a.tol2, a.hdr, a.resid, a.red, PackedRows{},
+    pcg_init_body<K, false>(a.P, a.zc, a.h, a.w, a.g, a.y, a.p0, a.tol2, a.hdr, a.resid, a.red, PackedRows{},
                      batch_grid(b.start[s], a.gx, a.gy, a.gz));
 }
 
@@ -1062,7 +1066,8 @@ static cudaError_t solve_k(const DevProblem& P, const SolveOpts& so, const float
     }
     {
         LaunchScope ls(MPM_KERNEL_PCG_INIT, st);
-        k_pcg_init<K><<<ig.grid, ig.block, 0, st>>>(P, ig.zc, h, w, g, y, B.p[0], tol2, hdr, resid, red, rows);
+        const auto init = rows.w ? k_pcg_init<K, true> : k_pcg_init<K, false>;
+        init<<<ig.grid, ig.block, 0, st>>>(P, ig.zc, h, w, g, y, B.p[0], tol2, hdr, resid, red, rows);
     }
     const StencilGrid tg = tma ? tma_grid(P, tile) : sg;
     const bool want_resid = resid != nullptr || tol2 > 0.0;
