@@ -55,10 +55,12 @@ struct InitArgs {
 };
 
 struct StepArgs {
-    CUtensorMap tp, tv, tp2, tw, th, tx;
+    CUtensorMap tp, tv, tp2, tz, tw, th, tx;
     DevProblem P;
     int nchunk, j, want_rr;
     float4 *vout, *pout, *xacc;
+    const float4* p2;
+    float4* zout;
     WsHeader* hdr;
     double* resid;
     Reduce red;

@@ -65,7 +65,8 @@ struct SolveScalars {
     int it;           // PCG iterations completed
     int xcount;       // iterations already folded into x (x is updated every other iteration)
     int done;         // 1 = no further iterations
-    int pad;
+    float pz;         // (p.M p) / (z.M z) of the next direction p and its z
+    int zin, zout;    // the next iteration reads z of the latest one; stores its own (pcg_step.cuh)
 };
 
 // Reduction scratch: per-block partials and an arrival counter.  The counter

@@ -695,7 +695,7 @@ static void plan_phased(FitJob* jobs, int n, std::vector<std::vector<PhasedSubje
         const int tile = tma_tile_choice(j.P);
         PhasedSubject ps;
         ps.j = &j;
-        ps.B = solve_bufs(j.P, j.L.solve);
+        ps.B = solve_bufs(j.P, j.L.solve, j.L.solve_bytes, j.L.red);
         if (!make_step_maps(j.P, j.L.h, j.L.w, j.P.nx, ps.B, tile, &ps.maps)) continue;
 
         rest[i] = 0;

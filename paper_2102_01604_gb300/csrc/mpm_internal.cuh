@@ -125,8 +125,8 @@ cudaError_t launch_solve_mg(const DevProblem& P, const SolveOpts& o, const float
 // when the volume or the pointers do not meet the copy engine's alignment
 // rules; the plain kernel is used then.
 struct StepMaps {
-    CUtensorMap v[2], p[3];   // halo boxes of the solve's vectors
-    CUtensorMap x;            // tile box (x fold)
+    CUtensorMap v[2], p[3], z[2];   // halo boxes of the solve's vectors
+    CUtensorMap x;                  // tile box (x fold)
     CUtensorMap w, h;
     SolveBufs B;
     int tile;          // index of the tile shape the maps were encoded for
@@ -153,7 +153,7 @@ cudaError_t launch_step_tma(const DevProblem& P, const StencilGrid& g, const Ste
                             cudaStream_t st);
 // Launches serving several subjects (batch.cuh): blocks[s] hardware blocks
 // for subject s, n <= kBatchMax.
-SolveBufs solve_bufs(const DevProblem& P, void* solve_ws);
+SolveBufs solve_bufs(const DevProblem& P, void* solve_ws, size_t ws_bytes, Reduce red);
 // share[s]: subject s's part of the group's voxels (the launch sets the grids).
 cudaError_t launch_jtv_batch(int K, const JtvArgs* a, const double* share, int n, cudaStream_t st);
 cudaError_t launch_grad_hess_batch(int K, int precond, int echo_dtype, const GradArgs* a,

@@ -18,23 +18,33 @@
 // wanted.  r.z is recomputed directly (z_j.M z_j) in every iteration, so the
 // expansion spans one step and errors do not accumulate.
 //
-// z itself is not stored: the last two directions hold it,
+// z itself is not stored while the last two directions hold it,
 //     z_j = p_j - beta_{j-1} p_{j-1},
-// with the beta that formed p_j, so an iteration reads p_j, p_{j-1} and v_j
+// with the beta that formed p_j: an iteration reads p_j, p_{j-1} and v_j
 // and writes p_{j+1} and v_{j+1}.  The iteration is bound by HBM: without z's
 // store it moves 124 B per voxel (K = 4) instead of 140, and the x fold, whose
 // two directions are both at hand, 16 B per iteration instead of 24.  The
-// difference of two roundings of p's size replaces one of z's; |p_j| stays
-// within a few |z_j| (1 to 3.3 on the Newton systems of a fit), and delta's
-// error against 64-bit arithmetic is the same (2.0e-7 either way after 30
-// iterations).
+// rounding of that z is 2^-24 |p_j|, of a stored one 2^-24 |z_j|.  On the
+// Newton systems of a fit |p_j| is within a few |z_j| (1 to 3.3), but on stiff
+// ones it reaches hundreds: at lambda = 1e5, 500 iterations, delta would end
+// 1.5e-4 from the 64-bit solution instead of 1.2e-6.  So the scalars carry
+//     (p_j.M p_j) / (z_j.M z_j) = 1 + beta_{j-1} (p_{j-1}.M p_{j-1}) / (z_{j-1}.M z_{j-1})
+// (z_j.M p_{j-1} = 0), and an iteration above kStoreZ also stores its z_j, which
+// the next one reads in place of p_{j-1}: 16 B per voxel more, and as much
+// again in the folding iterations, whose p_{j-2} is then read for itself.  With
+// 8^2 the errors are those of a z that is always stored (CPU restatement in
+// float32, 20x16x12, delta after the last iteration):
+//     lambda, iterations    z stored    never     above 4     8         16
+//     10, 400               3.6e-7      3.7e-7    3.7e-7      3.7e-7    3.7e-7
+//     1e3, 400              4.6e-7      2.1e-6    5.1e-7      5.1e-7    5.0e-7
+//     1e5, 500              1.2e-6      1.5e-4    2.0e-6      1.9e-6    7.1e-7
 //
 // The preconditioner block M_n = H_n + diag(lambda_k d_n), d_n = sum of the
 // six edge coefficients, is factorised in every iteration from H and the JTV
 // weights (its float32 Cholesky factor is the same each time), so the solve
 // stores no factor.
 //
-// The solve's own vectors (z, v, p and the accumulated x) are stored voxel
+// The solve's own vectors (v, p, the accumulated x and z where stored) are stored voxel
 // by voxel, four floats per voxel (K = 3 leaves the fourth zero), so one
 // 16-byte access moves all maps of a voxel; H, w and the caller's arrays stay
 // planar [component][N].
@@ -115,12 +125,16 @@ __device__ __forceinline__ float edge_sum(const float (&c)[6])
     return ((((c[0] + c[1]) + c[2]) + c[3]) + c[4]) + c[5];
 }
 
+// Largest (p.M p) / (z.M z) of an iteration that does not store z.
+constexpr float kStoreZ = 64.0f;
+
 // Per-solve workspace buffers: [N] float4 each (voxel-interleaved maps),
 // 256-byte aligned.
 struct SolveBufs {
     float4* v[2];    // v_j = M^-1 q_j in v[j & 1]
     float4* p[3];    // direction p_j in p[j % 3]
     float4* x;       // sum of the directions folded so far, alpha_i p_i
+    float4* z[2];    // preconditioned residual z_j in z[j & 1], where it is stored
 };
 
 template <int K>
@@ -175,6 +189,17 @@ __device__ __forceinline__ Maps axpy(float s, const Maps& v, const Maps& w)
 }
 __device__ __forceinline__ Maps minus(const Maps& v, const Maps& w) { return axpy(-1.0f, w, v); }
 
+// *at = v if `yes`, as one predicated store.  The tests for a stored z cost a
+// solve of 176x240x256 0.3% this way (7.41 -> 7.43 ms; a 64^3 fit 10.06 -> 10.01),
+// 0.8% with an if around the store (7.47), more with one branch around both
+// forms of z (7.60) or a second copy of the march (7.42, but the 64^3 fit 10.38).
+__device__ __forceinline__ void store_if(int yes, float4* at, const Maps& v)
+{
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.s32 q, %0, 0;\n\t@q st.global.v4.f32 [%1], {%2, %3, %4, %5};\n\t}"
+                 ::"r"(yes), "l"(at), "f"(v.a.x), "f"(v.a.y), "f"(v.b.x), "f"(v.b.y)
+                 : "memory");
+}
+
 // sum_k v_k w_k (the padding of K = 3 is zero).
 __device__ __forceinline__ float dot(const Maps& v, const Maps& w)
 {
@@ -183,18 +208,27 @@ __device__ __forceinline__ float dot(const Maps& v, const Maps& w)
 }
 
 // The scalars an iteration starts from: alpha_{j-1}, alpha_{j-2}, beta_{j-1}
-// and beta_{j-2} (those that exist).
+// and beta_{j-2} (those that exist), whether z_{j-1} was stored and whether z_j is.
 struct StepScalars {
     float alpha, alpha_prev, beta, beta_prev;
+    int zin, zout;
 };
 
-// z_j and p_j of one point from p1 = p_{j-1}, v = v_{j-1} and p2 = p_{j-2}
-// (j = 0: p1 is p_0 and v, p2 are not read; j = 1: p2 is not read).
+__device__ __forceinline__ StepScalars step_start(const SolveScalars& sc)
+{
+    return StepScalars{(float)sc.alpha, (float)sc.alpha_prev, (float)sc.beta, (float)sc.beta_prev,
+                       sc.zin, sc.zout};
+}
+
+// z_j and p_j of one point from p1 = p_{j-1}, v = v_{j-1} and pz = p_{j-2}, or
+// z_{j-1} where that was stored (j = 0: p1 is p_0 and v, pz are not read; j =
+// 1: pz is not read).
 template <int MODE>
 __device__ __forceinline__ void step_point(const StepScalars& s, const Maps& p1, const Maps& v,
-                                           const Maps& p2, Maps& zj, Maps& pj)
+                                           const Maps& pz, Maps& zj, Maps& pj)
 {
-    const Maps z = MODE >= kModeStep ? axpy(-s.beta_prev, p2, p1) : p1;   // z_{j-1}
+    Maps z = p1;                                                          // z_{j-1}
+    if (MODE >= kModeStep) z = s.zin ? pz : axpy(-s.beta_prev, pz, p1);
     zj = MODE == kModeFirst ? z : axpy(-s.alpha, v, z);
     pj = MODE == kModeFirst ? z : axpy(s.beta, p1, zj);
 }
@@ -291,6 +325,8 @@ __device__ __forceinline__ void step_scalars(const double (&s)[kStepSums], int j
 {
     SolveScalars& sc = hdr->sc;
     const double alpha_old = sc.alpha, beta_old = sc.beta;
+    const float pz_old = sc.pz;
+    const int zout_old = sc.zout;
     bool bad = false;
 #pragma unroll
     for (int i = 0; i < kStepSums; ++i) bad |= is_nan(s[i]);
@@ -308,6 +344,9 @@ __device__ __forceinline__ void step_scalars(const double (&s)[kStepSums], int j
     sc.beta_prev = beta_old;
     sc.beta = quot(rz_next, rz, irz);
     sc.rz = rz_next;
+    sc.pz = fmaf((float)sc.beta, pz_old, 1.0f);
+    sc.zin = zout_old;
+    sc.zout = !(sc.pz <= kStoreZ);
     sc.it = j + 1;
     if (resid_sums) {
         const double rr = s[kSumRR] - 2.0 * alpha * s[kSumRQ] + alpha * alpha * s[kSumQQ];

@@ -528,8 +528,8 @@ __global__ void __launch_bounds__(kBlock) k_jtv_batch(const __grid_constant__ Ba
 
 static size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 
-// v[2], p[3] and x, each [N] float4.
-static size_t pcg_bytes(const DevProblem& P) { return 6 * align256(sizeof(float4) * (size_t)P.N); }
+// v[2], p[3], x and z[2], each [N] float4.
+static size_t pcg_bytes(const DevProblem& P, int vecs = 8) { return vecs * align256(sizeof(float4) * (size_t)P.N); }
 
 // Copies of w and H with rows padded to a multiple of 4 floats (16 bytes), the
 // row pitch the copy engine needs, for volumes whose x size is not one: the
@@ -559,7 +559,9 @@ static bool wants_packed(const DevProblem& P)
     return P.nx % 4 != 0 && tma_tile_fits(P, tma_tile_choice(P));
 }
 
-size_t solve_ws_least(const DevProblem& P) { return std::max(pcg_bytes(P), mg_ws_bytes(P)); }
+// (The multigrid solver's need is the larger one but for volumes of up to 512
+// voxels, whose z[1] lies elsewhere where there is no room for it, see carve.)
+size_t solve_ws_least(const DevProblem& P) { return std::max(pcg_bytes(P, 7), mg_ws_bytes(P)); }
 
 // The larger of the two solvers' needs; with rows to pad, room for their copies.
 size_t solve_ws_bytes(const DevProblem& P)
@@ -581,7 +583,9 @@ SolveOpts solve_opts(const mpm_opts& o, bool overlap)
     return s;
 }
 
-static SolveBufs carve(const DevProblem& P, void* ws)
+// Without room for eight vectors (at most 512 voxels), z[1] takes the part of
+// the reduction partials that the iteration's seven sums leave.
+static SolveBufs carve(const DevProblem& P, void* ws, size_t ws_bytes, Reduce red)
 {
     SolveBufs b;
     char* c = static_cast<char*>(ws);
@@ -589,6 +593,9 @@ static SolveBufs carve(const DevProblem& P, void* ws)
     for (float4*& v : b.v) { v = reinterpret_cast<float4*>(c); c += vec; }
     for (float4*& v : b.p) { v = reinterpret_cast<float4*>(c); c += vec; }
     b.x = reinterpret_cast<float4*>(c);
+    b.z[0] = reinterpret_cast<float4*>(c + vec);
+    b.z[1] = ws_bytes >= pcg_bytes(P) ? reinterpret_cast<float4*>(c + 2 * vec)
+                                      : reinterpret_cast<float4*>(red.partials + (size_t)kStepSums * kMaxBlocks);
     return b;
 }
 
@@ -680,6 +687,8 @@ __device__ __forceinline__ void pcg_init_body(const DevProblem& P, int zc, const
         sc.alpha_prev = 0.0;
         sc.beta = 0.0;
         sc.beta_prev = 0.0;
+        sc.pz = 1.0f;
+        sc.zin = sc.zout = 0;
         sc.it = 0;
         sc.xcount = 0;
         sc.tol2 = tol2;
@@ -714,8 +723,8 @@ __global__ void __launch_bounds__(kBlock) k_pcg_init_batch(const __grid_constant
 
 // Plain form of one PCG iteration (pcg_step.cuh): a thread per (x, y) column
 // marching a run of z planes; each neighbour's p_j is formed from its own
-// p_{j-1}, v_{j-1} and p_{j-2} read from memory.  Used for volumes or pointers the TMA kernel
-// cannot take (a volume smaller than a tile, unaligned buffers).
+// p_{j-1}, v_{j-1} and p_{j-2} (or the stored z_{j-1}) read from memory.  Used
+// for volumes or pointers the TMA kernel cannot take (a volume smaller than a tile, unaligned buffers).
 template <int K, int MODE>
 __global__ void __launch_bounds__(kBlock) k_pcg_step(DevProblem P, int zc, int j, int want_rr,
                                                      const float* __restrict__ h,
@@ -723,9 +732,11 @@ __global__ void __launch_bounds__(kBlock) k_pcg_step(DevProblem P, int zc, int j
                                                      const float4* __restrict__ pin,
                                                      const float4* __restrict__ vin,
                                                      const float4* __restrict__ p2,
+                                                     const float4* __restrict__ zprev,
                                                      float4* __restrict__ vout,
                                                      float4* __restrict__ pout, float4* __restrict__ xacc,
-                                                     WsHeader* hdr, double* resid, Reduce red)
+                                                     float4* __restrict__ zout, WsHeader* hdr,
+                                                     double* resid, Reduce red)
 {
     constexpr int T = K * (K + 1) / 2;
     constexpr bool first = MODE == kModeFirst;
@@ -735,8 +746,7 @@ __global__ void __launch_bounds__(kBlock) k_pcg_step(DevProblem P, int zc, int j
     wait_predecessor();
     if (tid == 0) {
         s_done = hdr->sc.done;
-        s_sc = StepScalars{(float)hdr->sc.alpha, (float)hdr->sc.alpha_prev, (float)hdr->sc.beta,
-                           (float)hdr->sc.beta_prev};
+        s_sc = step_start(hdr->sc);
     }
     __syncthreads();
     if (s_done) return;
@@ -750,8 +760,9 @@ __global__ void __launch_bounds__(kBlock) k_pcg_step(DevProblem P, int zc, int j
     const int z1p = min(P.nz, z0p + zc);
     float part[kStepSums] = {};
     const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    const float4* __restrict__ pz = sc.zin ? zprev : p2;
     auto point = [&](long long m, Maps& zj, Maps& pj) {
-        step_point<MODE>(sc, pin[m], first ? zero : vin[m], MODE >= kModeStep ? p2[m] : zero, zj, pj);
+        step_point<MODE>(sc, pin[m], first ? zero : vin[m], MODE >= kModeStep ? pz[m] : zero, zj, pj);
     };
     if (x < P.nx && yy < P.ny) {
         for (int z = z0p; z < z1p; ++z) {
@@ -773,6 +784,7 @@ __global__ void __launch_bounds__(kBlock) k_pcg_step(DevProblem P, int zc, int j
             Maps v;
             step_voxel<K>(P, e.c, zj, pj, [&](int m) { return nb[m]; }, hv, want_rr, v, part);
             if (!first) pout[n] = pj.vec();
+            if (!first && sc.zout) zout[n] = zj.vec();
             vout[n] = v.vec();
             if (MODE >= kModeFold) xacc[n] = fold_x(MODE == kModeFoldX ? xacc[n] : zero, sc, p2[n], pin[n]).vec();
         }
@@ -1026,11 +1038,12 @@ static cudaError_t launch_step_plain(const DevProblem& P, const StencilGrid& sg,
 {
     const int jm = j > 0 ? j - 1 : 0;
     const float4 *pin = B.p[jm % 3], *vin = B.v[jm & 1], *p2 = B.p[(j + 1) % 3];
-    float4 *vout = B.v[j & 1], *pout = B.p[j % 3];
+    const float4* zprev = B.z[jm & 1];
+    float4 *vout = B.v[j & 1], *pout = B.p[j % 3], *zout = B.z[j & 1];
     cudaError_t e;
 #define MPM_STEP_PLAIN(M)                                                                          \
     e = launch_dependent(overlap, k_pcg_step<K, M>, sg.grid, sg.block, 0, st, P, sg.zc, j, want_rr, h, w, pin, vin, p2, \
-                         vout, pout, B.x, hdr, resid, red)
+                         zprev, vout, pout, B.x, zout, hdr, resid, red)
     switch (step_mode(j)) {
     case kModeFirst: MPM_STEP_PLAIN(kModeFirst); break;
     case kModeSecond: MPM_STEP_PLAIN(kModeSecond); break;
@@ -1050,7 +1063,7 @@ static cudaError_t solve_k(const DevProblem& P, const SolveOpts& so, const float
 {
     const StencilGrid sg = stencil_grid(P, kTileX, kTileY);
     const StencilGrid ig = stencil_grid(P, kTileX, kTileY, kInitWaves);
-    SolveBufs B = carve(P, solve_ws);
+    SolveBufs B = carve(P, solve_ws, ws_bytes, red);
     const int cg_iters = so.cg_iters;
     const double tol2 = so.tol_cg > 0.0 ? so.tol_cg * so.tol_cg : 0.0;
     StepMaps maps;
@@ -1087,7 +1100,7 @@ cudaError_t tma_autotune(const DevProblem& P, void* solve_ws, WsHeader* hdr, Red
                          cudaStream_t st, int* best, float* ms)
 {
     *best = -1;
-    // Timed on zeroed operands carved from the solve workspace's six vectors
+    // Timed on zeroed operands carved from six of the solve workspace's vectors
     // so that no buffer the launch writes is also read: iteration 3 reads p_2,
     // p_1 and v_2 from vectors 0-2 and writes p_3 and v_3 to 4 and 5; H and w
     // alias the read-only vectors 0-3 (T N floats fit in 0-2 for K = 3, 4).
@@ -1097,7 +1110,7 @@ cudaError_t tma_autotune(const DevProblem& P, void* solve_ws, WsHeader* hdr, Red
     SolveBufs B;
     B.p[2] = at(0); B.p[1] = at(1); B.p[0] = at(4);
     B.v[0] = at(2); B.v[1] = at(5);
-    B.x = at(3);       // not touched in iteration 3
+    B.x = B.z[0] = B.z[1] = at(3);       // not touched in iteration 3
     const float* h = reinterpret_cast<const float*>(at(0));
     const float* w = reinterpret_cast<const float*>(at(3));
     cudaError_t e;
@@ -1139,7 +1152,10 @@ cudaError_t tma_autotune(const DevProblem& P, void* solve_ws, WsHeader* hdr, Red
 
 // ------------------------------------------------- batched launches
 
-SolveBufs solve_bufs(const DevProblem& P, void* solve_ws) { return carve(P, solve_ws); }
+SolveBufs solve_bufs(const DevProblem& P, void* solve_ws, size_t ws_bytes, Reduce red)
+{
+    return carve(P, solve_ws, ws_bytes, red);
+}
 
 template <int K, bool RUNS, typename IT>
 static cudaError_t launch_jtv_batch_staged(int smem, const Batch<JtvArgs>& b, cudaStream_t st)

@@ -5,11 +5,13 @@
 // Iteration j reads p_{j-1}, v_{j-1} and p_{j-2} (with a one-voxel halo), the
 // JTV weights and H, and writes p_j and v_j once:
 //   z_j = (p_{j-1} - beta_{j-2} p_{j-2}) - alpha_{j-1} v_{j-1}
+// (where iteration j - 1 stored z_{j-1}, that takes the place of p_{j-2}, and
+// where the scalars ask for it z_j is written too; pcg_step.cuh)
 //   p_j = z_j + beta_{j-1} p_{j-1}
 //   q_j = (H + L) p_j,  v_j = M^-1 q_j,  and the sums for alpha_j and beta_j.
 // A block owns a TX x TY tile and marches up a run of z planes.  Per plane
 // one thread issues bulk tensor copies into a ring of "raw" stages:
-//   p, v, p_j-2  (TX+2) x (TY+2) voxels of 4 floats at (x0 - 1, y0 - 1, z)
+//   p, v, p_j-2 or z_j-1  (TX+2) x (TY+2) voxels of 4 floats at (x0 - 1, y0 - 1, z)
 //   w            (TX+8) x (TY+2) floats at (x0 - 4, y0 - 1, z)
 //   x            TX x TY voxels of 4 floats at (x0, y0, z) (even j > 2, x fold)
 // and H (TX x TY x T floats, planar) into a second ring.  The solve's own
@@ -135,8 +137,9 @@ __device__ __forceinline__ void compute_warps_sync()
 template <int K, int TX, int TY, int MODE>
 __device__ __forceinline__ void step_body(
     const DevProblem& P, int nchunk, int j, int want_rr, const CUtensorMap* tp, const CUtensorMap* tv,
-    const CUtensorMap* tp2, const CUtensorMap* tw, const CUtensorMap* th, const CUtensorMap* txm,
-    float4* __restrict__ vout, float4* __restrict__ pout, float4* __restrict__ xacc, WsHeader* hdr,
+    const CUtensorMap* tp2, const CUtensorMap* tz, const CUtensorMap* tw, const CUtensorMap* th,
+    const CUtensorMap* txm, float4* __restrict__ vout, float4* __restrict__ pout,
+    float4* __restrict__ xacc, const float4* __restrict__ p2, float4* __restrict__ zout, WsHeader* hdr,
     double* resid, Reduce red, long long wait_cycles, int withhold, const VGrid& vg)
 {
     using L = StepLayout<K, TX, TY, (MODE >= kModeFold)>;
@@ -167,7 +170,10 @@ __device__ __forceinline__ void step_body(
     if (tid == 32) {
         prefetch_map(tp);
         if (!first) prefetch_map(tv);
-        if (third) prefetch_map(tp2);
+        if (third) {
+            prefetch_map(tp2);
+            prefetch_map(tz);
+        }
         prefetch_map(tw);
         prefetch_map(th);
         if (readx) prefetch_map(txm);
@@ -187,8 +193,7 @@ __device__ __forceinline__ void step_body(
     wait_predecessor();
     if (tid == 0) {
         s_done = hdr->sc.done;
-        s_sc = StepScalars{(float)hdr->sc.alpha, (float)hdr->sc.alpha_prev, (float)hdr->sc.beta,
-                           (float)hdr->sc.beta_prev};
+        s_sc = step_start(hdr->sc);
     }
     __syncthreads();
     if (s_done) return;                                   // the same in every block
@@ -213,6 +218,7 @@ __device__ __forceinline__ void step_body(
     if (producer) {
         if (lane == 0 && !withhold) {
             int cb = 0, eb = 0;           // counters of the item's first planes
+            const CUtensorMap* tpz = sc.zin ? tz : tp2;
             for (int i = (int)vg.bx; i < items && !s_fail; i += (int)vg.gx) {
                 const int t = i % tiles, ch = i / tiles;
                 const int za = (int)((long long)ch * nz / nchunk), zb = (int)((long long)(ch + 1) * nz / nchunk);
@@ -236,7 +242,7 @@ __device__ __forceinline__ void step_body(
                     mbar_expect_tx(bar, bytes);
                     tma_load_3d(smem_u32(st + L::P_OFF), tp, 4 * (x0 - 1), y0 - 1, jj, bar);
                     if (!first) tma_load_3d(smem_u32(st + L::V_OFF), tv, 4 * (x0 - 1), y0 - 1, jj, bar);
-                    if (third) tma_load_3d(smem_u32(st + L::P2_OFF), tp2, 4 * (x0 - 1), y0 - 1, jj, bar);
+                    if (third) tma_load_3d(smem_u32(st + L::P2_OFF), tpz, 4 * (x0 - 1), y0 - 1, jj, bar);
                     tma_load_3d(smem_u32(st + L::W_OFF), tw, x0 - 4, y0 - 1, jj, bar);
                     if (readx && inner) tma_load_3d(smem_u32(st + L::X_OFF), txm, 4 * x0, y0, jj, bar);
                     raw_issued = c;
@@ -342,8 +348,8 @@ __device__ __forceinline__ void step_body(
                     const float4* bv = reinterpret_cast<const float4*>(st + L::V_OFF);
                     const float4* b2 = reinterpret_cast<const float4*>(st + L::P2_OFF);
                     const float* bw = reinterpret_cast<const float*>(st + L::W_OFF) + wcc;
-                    const Maps p1 = bp[bc], p2 = third ? Maps(b2[bc]) : zero;
-                    step_point<MODE>(sc, p1, first ? zero : Maps(bv[bc]), p2, zn, pn);
+                    const Maps p1 = bp[bc], pz = third ? Maps(b2[bc]) : zero;
+                    step_point<MODE>(sc, p1, first ? zero : Maps(bv[bc]), pz, zn, pn);
                     wn = bw[0];
                     cxyn[0] = okxm ? (wn + bw[-1]) * P.ihx2 : 0.f;
                     cxyn[1] = okxp ? (wn + bw[1]) * P.ihx2 : 0.f;
@@ -359,9 +365,11 @@ __device__ __forceinline__ void step_body(
                         }
                         if (inside) {
                             if (!first) pout[n] = pn.vec();
+                            if (!first) store_if(s_sc.zout, zout + n, zn);
                             if (fold) {
                                 const float4* bx = reinterpret_cast<const float4*>(st + L::X_OFF);
-                                xacc[n] = fold_x(readx ? Maps(bx[tc]) : zero, sc, p2, p1).vec();
+                                const Maps f = sc.zin ? Maps(p2[n]) : pz;         // p_{j-2}
+                                xacc[n] = fold_x(readx ? Maps(bx[tc]) : zero, sc, f, p1).vec();
                             }
                         }
                     }
@@ -426,13 +434,14 @@ template <int K, int TX, int TY, int MODE>
 __global__ void __launch_bounds__(StepLayout<K, TX, TY>::THREADS, StepLayout<K, TX, TY>::MINB) k_pcg_step_tma(
     DevProblem P, int nchunk, int j, int want_rr, const __grid_constant__ CUtensorMap tp,
     const __grid_constant__ CUtensorMap tv, const __grid_constant__ CUtensorMap tp2,
-    const __grid_constant__ CUtensorMap tw, const __grid_constant__ CUtensorMap th,
-    const __grid_constant__ CUtensorMap txm, float4* __restrict__ vout, float4* __restrict__ pout,
-    float4* __restrict__ xacc, WsHeader* hdr, double* resid, Reduce red, long long wait_cycles,
-    int withhold)
+    const __grid_constant__ CUtensorMap tz, const __grid_constant__ CUtensorMap tw,
+    const __grid_constant__ CUtensorMap th, const __grid_constant__ CUtensorMap txm,
+    float4* __restrict__ vout, float4* __restrict__ pout, float4* __restrict__ xacc,
+    const float4* __restrict__ p2, float4* __restrict__ zout, WsHeader* hdr, double* resid, Reduce red,
+    long long wait_cycles, int withhold)
 {
-    step_body<K, TX, TY, MODE>(P, nchunk, j, want_rr, &tp, &tv, &tp2, &tw, &th, &txm, vout, pout, xacc,
-                               hdr, resid, red, wait_cycles, withhold, hw_grid());
+    step_body<K, TX, TY, MODE>(P, nchunk, j, want_rr, &tp, &tv, &tp2, &tz, &tw, &th, &txm, vout, pout, xacc,
+                               p2, zout, hdr, resid, red, wait_cycles, withhold, hw_grid());
 }
 
 // Several subjects in one launch (mpm_fit_batch with opts.graph = 2).
@@ -442,8 +451,8 @@ __global__ void __launch_bounds__(StepLayout<K, TX, TY>::THREADS, StepLayout<K, 
 {
     const int s = batch_subject(b.start, b.n);
     const StepArgs& a = b.a[s];
-    step_body<K, TX, TY, MODE>(a.P, a.nchunk, a.j, a.want_rr, &a.tp, &a.tv, &a.tp2, &a.tw, &a.th, &a.tx,
-                               a.vout, a.pout, a.xacc, a.hdr, a.resid, a.red, a.wait_cycles, a.withhold, batch_grid(b.start[s], b.start[s + 1] - b.start[s], 1, 1));
+    step_body<K, TX, TY, MODE>(a.P, a.nchunk, a.j, a.want_rr, &a.tp, &a.tv, &a.tp2, &a.tz, &a.tw, &a.th, &a.tx,
+                               a.vout, a.pout, a.xacc, a.p2, a.zout, a.hdr, a.resid, a.red, a.wait_cycles, a.withhold, batch_grid(b.start[s], b.start[s + 1] - b.start[s], 1, 1));
 }
 
 // ------------------------------------------------------------------ host
@@ -523,6 +532,7 @@ bool make_step_maps(const DevProblem& P, const float* h, const float* w, int pit
                     reinterpret_cast<uintptr_t>(B.x);
     for (float4* v : B.v) any |= reinterpret_cast<uintptr_t>(v);
     for (float4* v : B.p) any |= reinterpret_cast<uintptr_t>(v);
+    for (float4* v : B.z) any |= reinterpret_cast<uintptr_t>(v);
     if (any % 16) return false;
     if (!encode_fn()) return false;
     const cuuint64_t nx = P.nx, ny = P.ny, nz = P.nz;
@@ -543,7 +553,7 @@ bool make_step_maps(const DevProblem& P, const float* h, const float* w, int pit
     bool ok = encode(&out->w, w, 3, d3, s3, wbox) && encode(&out->h, h, 4, dh, sh, hbox) &&
               encode(&out->x, f(B.x), 3, da, sa, tilebox);
     for (int i = 0; i < 2 && ok; ++i)
-        ok = encode(&out->v[i], f(B.v[i]), 3, da, sa, halo);
+        ok = encode(&out->v[i], f(B.v[i]), 3, da, sa, halo) && encode(&out->z[i], f(B.z[i]), 3, da, sa, halo);
     for (int i = 0; i < 3 && ok; ++i) ok = encode(&out->p[i], f(B.p[i]), 3, da, sa, halo);
     out->B = B;
     out->tile = tile;
@@ -566,8 +576,9 @@ static cudaError_t launch_step_m(const DevProblem& P, int nchunk, dim3 grid, con
     }
     const int jm = j > 0 ? j - 1 : 0;
     return launch_dependent(
-        overlap, k_pcg_step_tma<K, TX, TY, MODE>, grid, dim3(L::THREADS, 1, 1), L::SMEM, st, P, nchunk, j, want_rr, m.p[jm % 3], m.v[jm & 1], m.p[(j + 1) % 3], m.w, m.h, m.x,
-        m.B.v[j & 1], m.B.p[j % 3], m.B.x, hdr, resid, red,
+        overlap, k_pcg_step_tma<K, TX, TY, MODE>, grid, dim3(L::THREADS, 1, 1), L::SMEM, st, P, nchunk, j, want_rr, m.p[jm % 3], m.v[jm & 1],
+        m.p[(j + 1) % 3], m.z[jm & 1], m.w, m.h, m.x, m.B.v[j & 1], m.B.p[j % 3], m.B.x,
+        m.B.p[(j + 1) % 3], m.B.z[j & 1], hdr, resid, red,
         g_wait_cycles.load(std::memory_order_relaxed), g_withhold.load(std::memory_order_relaxed));
 }
 
@@ -593,6 +604,7 @@ StepArgs step_args(const DevProblem& P, const StepMaps& m, int nchunk, int j, in
     a.tp = m.p[jm % 3];
     a.tv = m.v[jm & 1];
     a.tp2 = m.p[(j + 1) % 3];
+    a.tz = m.z[jm & 1];
     a.tw = m.w;
     a.th = m.h;
     a.tx = m.x;
@@ -603,6 +615,8 @@ StepArgs step_args(const DevProblem& P, const StepMaps& m, int nchunk, int j, in
     a.vout = m.B.v[j & 1];
     a.pout = m.B.p[j % 3];
     a.xacc = m.B.x;
+    a.p2 = m.B.p[(j + 1) % 3];
+    a.zout = m.B.z[j & 1];
     a.hdr = hdr;
     a.resid = resid;
     a.red = red;
