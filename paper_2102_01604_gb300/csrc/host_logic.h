@@ -1,10 +1,12 @@
 // host_logic.h -- host-side decisions of the library that make no CUDA call:
 // the server's device arena and admission pick, the GPU-load rule shared by
-// the server and the batched graph, the lanes of a batched graph, and the z
-// split of the TMA PCG iteration.  Plain C++17, so the CPU tests compile and check it directly.
+// the server and the batched graph, the lanes of a batched graph, the z
+// split of the TMA PCG iteration and what is done once per device.  Plain
+// C++17, so the CPU tests compile and check it directly.
 #pragma once
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstddef>
 #include <iterator>
@@ -12,6 +14,25 @@
 #include <vector>
 
 namespace mpm {
+
+// Something to be done once on each device of the process: run(dev, f) calls f
+// unless f has returned 0 for `dev` before.  (Threads that come first together
+// may each call it.)  For kernel attributes, which hold for the device that was
+// current when they were set.
+class OncePerDevice {
+    std::atomic<unsigned long long> done_{0};
+
+public:
+    template <class F>
+    auto run(int dev, F f) -> decltype(f())
+    {
+        const unsigned long long bit = dev >= 0 && dev < 64 ? 1ull << dev : 0;
+        if (done_.load(std::memory_order_acquire) & bit) return static_cast<decltype(f())>(0);
+        const auto e = f();
+        if (static_cast<int>(e) == 0) done_.fetch_or(bit, std::memory_order_release);
+        return e;
+    }
+};
 
 // Share of the GPU one fit keeps busy: about 2^21 voxels keep every kernel of
 // a fit at a full wave, so larger volumes count as 1, smaller ones pro rata.

@@ -41,6 +41,22 @@ struct LaunchScope {
     void* rec;
 };
 
+template <class F>
+cudaError_t once_on_this_device(OncePerDevice& once, F f)
+{
+    int dev = 0;
+    const cudaError_t e = cudaGetDevice(&dev);
+    return e ? e : once.run(dev, f);
+}
+
+// Lets kernel f use `bytes` of dynamic shared memory on the current device.
+template <class F>
+cudaError_t smem_opt_in(OncePerDevice& once, F* f, int bytes)
+{
+    return once_on_this_device(
+        once, [&] { return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes); });
+}
+
 // Launches f; with `overlap`, so that it may start before its predecessor on
 // the stream has finished (programmatic dependent launch): f must call
 // wait_predecessor.

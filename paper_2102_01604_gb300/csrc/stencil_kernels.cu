@@ -965,15 +965,9 @@ static void jtv_grid(const DevProblem& P, int stages, double share, JtvArgs& a)
 template <int K, bool RUNS, typename IT>
 static cudaError_t jtv_smem_opt_in()
 {
-    static bool done = false;
-    if (done) return cudaSuccess;
-    cudaError_t e = cudaFuncSetAttribute(k_jtv_staged<K, RUNS, IT>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, kJtvSmemMax);
-    if (!e)
-        e = cudaFuncSetAttribute(k_jtv_staged_batch<K, RUNS, IT>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, kJtvSmemMax);
-    done = e == cudaSuccess;
-    return e;
+    static OncePerDevice solo, batch;
+    const cudaError_t e = smem_opt_in(solo, k_jtv_staged<K, RUNS, IT>, kJtvSmemMax);
+    return e ? e : smem_opt_in(batch, k_jtv_staged_batch<K, RUNS, IT>, kJtvSmemMax);
 }
 
 template <int K>

@@ -566,14 +566,9 @@ static cudaError_t launch_step_m(const DevProblem& P, int nchunk, dim3 grid, con
                                  cudaStream_t st)
 {
     using L = StepLayout<K, TX, TY, (MODE >= kModeFold)>;
-    static bool attr = false;
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(k_pcg_step_tma<K, TX, TY, MODE>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             step_smem_max<K, TX, TY>());
-        if (e != cudaSuccess) return e;
-        attr = true;
-    }
+    static OncePerDevice once;
+    const cudaError_t e = smem_opt_in(once, k_pcg_step_tma<K, TX, TY, MODE>, step_smem_max<K, TX, TY>());
+    if (e != cudaSuccess) return e;
     const int jm = j > 0 ? j - 1 : 0;
     return launch_dependent(
         overlap, k_pcg_step_tma<K, TX, TY, MODE>, grid, dim3(L::THREADS, 1, 1), L::SMEM, st, P, nchunk, j, want_rr, m.p[jm % 3], m.v[jm & 1],
@@ -629,14 +624,9 @@ template <int K, int TX, int TY, int MODE>
 static cudaError_t launch_step_batch_m(const Batch<StepArgs>& b, cudaStream_t st)
 {
     using L = StepLayout<K, TX, TY, (MODE >= kModeFold)>;
-    static bool attr = false;
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(k_pcg_step_tma_batch<K, TX, TY, MODE>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             step_smem_max<K, TX, TY>());
-        if (e != cudaSuccess) return e;
-        attr = true;
-    }
+    static OncePerDevice once;
+    const cudaError_t e = smem_opt_in(once, k_pcg_step_tma_batch<K, TX, TY, MODE>, step_smem_max<K, TX, TY>());
+    if (e != cudaSuccess) return e;
     return launch_dependent(true, k_pcg_step_tma_batch<K, TX, TY, MODE>, dim3(b.start[b.n]), dim3(L::THREADS, 1, 1),
                             L::SMEM, st, b);
 }
@@ -759,18 +749,18 @@ static cudaError_t prime_one()
 
 cudaError_t prime_tma_kernels()
 {
-    static bool done = false;
-    if (done) return cudaSuccess;
-    cudaError_t e = prime_voxel_kernels();
-    if (!e) e = prime_jtv_kernels();
-    if (!e) e = prime_one<4, 16, 16>();
-    if (!e) e = prime_one<4, 32, 8>();
-    if (!e) e = prime_one<4, 32, 16>();
-    if (!e) e = prime_one<3, 16, 16>();
-    if (!e) e = prime_one<3, 32, 8>();
-    if (!e) e = prime_one<3, 32, 16>();
-    if (!e) done = true;
-    return e;
+    static OncePerDevice once;
+    return once_on_this_device(once, [] {
+        cudaError_t e = prime_voxel_kernels();
+        if (!e) e = prime_jtv_kernels();
+        if (!e) e = prime_one<4, 16, 16>();
+        if (!e) e = prime_one<4, 32, 8>();
+        if (!e) e = prime_one<4, 32, 16>();
+        if (!e) e = prime_one<3, 16, 16>();
+        if (!e) e = prime_one<3, 32, 8>();
+        if (!e) e = prime_one<3, 32, 16>();
+        return e;
+    });
 }
 
 cudaError_t launch_step_tma(const DevProblem& P, const StencilGrid& g, const StepMaps& m, int j,

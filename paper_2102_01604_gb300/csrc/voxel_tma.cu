@@ -350,12 +350,9 @@ static cudaError_t launch_tma_k(const DevProblem& P, const void* x, const float*
                                 unsigned* status, cudaStream_t st)
 {
     auto* f = k_grad_hess_tma<K, PRE, XT>;
-    static bool attr = false;
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kGhSmem);
-        if (e != cudaSuccess) return e;
-        attr = true;
-    }
+    static OncePerDevice once;
+    const cudaError_t e = smem_opt_in(once, f, kGhSmem);
+    if (e != cudaSuccess) return e;
     const long long chunks = (P.N + kChunk - 1) / kChunk;
     const int grid = (int)std::min<long long>(chunks, 2LL * sm_count());
     f<<<grid, kGhThreads, kGhSmem, st>>>(P, static_cast<const XT*>(x), y, b1p, b1m, g, h, nll, red,
@@ -389,12 +386,9 @@ template <int K, int PRE, typename XT>
 static cudaError_t launch_tma_batch_k(Batch<GradArgs>& b, cudaStream_t st)
 {
     auto* f = k_grad_hess_tma_batch<K, PRE, XT>;
-    static bool attr = false;
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kGhSmem);
-        if (e != cudaSuccess) return e;
-        attr = true;
-    }
+    static OncePerDevice once;
+    const cudaError_t e = smem_opt_in(once, f, kGhSmem);
+    if (e != cudaSuccess) return e;
     f<<<b.start[b.n], kGhThreads, kGhSmem, st>>>(b, copy_wait_cycles(), copy_withhold());
     return cudaGetLastError();
 }
