@@ -190,6 +190,8 @@ __device__ __forceinline__ void jtv_staged_body(const DevProblem& P, int zc, int
         if (bytes) bulk_load(smem_u32(d + b), r + b, bytes, bar);
         for (int q = 0; q < b && q < len; ++q) d[q] = __ldg(r + q);
         for (int q = bytes ? e : max(b, 0); q < len; ++q) d[q] = __ldg(r + q);
+        // a later copy of this lane writes the same floats through the async proxy
+        if (b > 0 || e < len) fence_async_proxy();
     };
     if (tid == 0) {
         s_fail = 0;

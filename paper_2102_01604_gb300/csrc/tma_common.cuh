@@ -69,6 +69,13 @@ __device__ __forceinline__ bool mbar_wait_nap(uint32_t bar, uint32_t parity, lon
     return true;
 }
 
+// Orders this thread's earlier ordinary accesses to shared memory before the
+// bulk copies it issues later.
+__device__ __forceinline__ void fence_async_proxy()
+{
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+}
+
 // Fetch a tensor map ahead of the first copy that uses it.
 __device__ __forceinline__ void prefetch_map(const CUtensorMap* map)
 {
