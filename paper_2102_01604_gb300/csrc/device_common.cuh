@@ -72,7 +72,7 @@ struct SolveScalars {
 // Reduction scratch: per-block partials and an arrival counter.  The counter
 // is zero between launches (the last block resets it).
 struct Reduce {
-    double* partials;        // [kMaxBlocks * 2]
+    double* partials;        // [8][kMaxBlocks]
     unsigned int* counter;
 };
 

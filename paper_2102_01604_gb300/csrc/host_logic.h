@@ -187,6 +187,14 @@ inline int tma_chunks(long long tiles, int nz, long long wave)
     return best;
 }
 
+// The same split for a launch of tiles x nchunk blocks that reduces over them,
+// which may have at most `most` (>= tiles): volumes of billions of voxels would
+// take more (3364 tiles of 1221 planes on 304 resident blocks: 37004).
+inline int grid_chunks(long long tiles, int nz, long long wave, long long most)
+{
+    return (int)std::min<long long>(tma_chunks(tiles, nz, wave), std::max(1LL, most / tiles));
+}
+
 // Shares of one launch of the TMA PCG iteration between several volumes (a
 // phase-batched group): volume s, of tiles[s] tiles per plane and nz[s]
 // planes, gets blocks[s] blocks and chunks[s] z ranges.  Each of its blocks

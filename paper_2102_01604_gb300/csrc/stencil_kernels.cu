@@ -941,7 +941,7 @@ static int jtv_stages(const DevProblem& P, const float* y, const float* w)
 }
 
 // Grid of the JTV kernel.  Staged: blocks over the voxels of a plane times z
-// ranges, the split of tma_chunks over the resident blocks (a range also reads
+// ranges, the split of grid_chunks over the resident blocks (a range also reads
 // the planes below and above it, as an item of the PCG iteration does); a
 // subject that shares a launch takes `share` of the blocks.
 static void jtv_grid(const DevProblem& P, int stages, double share, JtvArgs& a)
@@ -957,7 +957,7 @@ static void jtv_grid(const DevProblem& P, int stages, double share, JtvArgs& a)
     }
     const long long bx = ((long long)P.nx * P.ny + kJtvRun - 1) / kJtvRun;
     const int per_sm = jtv_smem(P, stages) <= kJtvSmemHalf ? 2 : 1;
-    const int gz = tma_chunks(bx, P.nz, std::max(1LL, (long long)(share * per_sm * kNumSm)));
+    const int gz = grid_chunks(bx, P.nz, std::max(1LL, (long long)(share * per_sm * kNumSm)), kMaxBlocks);
     a.zc = (P.nz + gz - 1) / gz;
     a.gx = (unsigned)bx;
     a.gy = 1;
