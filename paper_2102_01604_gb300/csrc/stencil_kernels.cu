@@ -919,7 +919,7 @@ StencilGrid stencil_grid(const DevProblem& P, int tx, int ty, int waves, double 
 // Stages of the staged JTV kernel for this volume: as many as leave two blocks
 // per SM, at least three (plane z, plane z + 1 and one in flight) within a
 // block's shared memory; 0 (the tile kernel) where those do not fit, rows of
-// more than about 1900 voxels at K = 4, and for small volumes, where the staged
+// more than 1831 voxels at K = 4, and for small volumes, where the staged
 // kernel's longer start-up costs what it gives (64^3: 14.3 us staged, 14.6 not;
 // without runs of four, 61^3: 15.4 and 12.9; 181x217x181: 58 and 78).
 constexpr long long kJtvStagedMinRuns = 1LL << 17, kJtvStagedMin = 1LL << 20;
@@ -932,9 +932,9 @@ static bool jtv_runs(const DevProblem& P, const float* y, const float* w)
     return P.nx % 4 == 0 && (reinterpret_cast<uintptr_t>(y) | reinterpret_cast<uintptr_t>(w)) % 16 == 0;
 }
 
-static int jtv_stages(const DevProblem& P, const float* y, const float* w)
+static int jtv_stages(const DevProblem& P, bool runs)
 {
-    if (P.N < (jtv_runs(P, y, w) ? kJtvStagedMinRuns : kJtvStagedMin)) return 0;
+    if (P.N < (runs ? kJtvStagedMinRuns : kJtvStagedMin)) return 0;
     for (int n = kJtvStagesMax; n >= 3; --n)
         if (jtv_smem(P, n) <= (n > 3 ? kJtvSmemHalf : kJtvSmemMax)) return n;
     return 0;
@@ -1012,7 +1012,7 @@ cudaError_t launch_jtv(const DevProblem& P, const float* y, float* w, double* jt
                        unsigned* status, cudaStream_t st)
 {
     JtvArgs a{P, 0, 0, 0, 0, 0, y, w, jtv, red, status};
-    jtv_grid(P, jtv_stages(P, y, w), 1.0, a);
+    jtv_grid(P, jtv_stages(P, jtv_runs(P, y, w)), 1.0, a);
     LaunchScope ls(MPM_KERNEL_JTV, st);
     if (P.K == 4) return index32(P) ? launch_jtv_k<4, int>(a, st) : launch_jtv_k<4, long long>(a, st);
     return index32(P) ? launch_jtv_k<3, int>(a, st) : launch_jtv_k<3, long long>(a, st);
@@ -1176,20 +1176,21 @@ static cudaError_t launch_jtv_batch_k(bool staged, bool runs, int smem, const Ba
 
 cudaError_t launch_jtv_batch(int K, const JtvArgs* a, const double* share, int n, cudaStream_t st)
 {
-    // one kernel for the whole launch: staged if every subject can take it
+    // one kernel for the whole launch: runs of four if every subject has them,
+    // staged if every subject is large enough for that form
     static thread_local Batch<JtvArgs> b;
     unsigned blocks[kBatchMax];
     JtvArgs args[kBatchMax];
     bool i32 = true, staged = true, runs = true;
     for (int i = 0; i < n; ++i) {
         i32 = i32 && index32(a[i].P);
-        staged = staged && jtv_stages(a[i].P, a[i].y, a[i].w) > 0;
         runs = runs && jtv_runs(a[i].P, a[i].y, a[i].w);
     }
+    for (int i = 0; i < n; ++i) staged = staged && jtv_stages(a[i].P, runs) > 0;
     int smem = 0;
     for (int i = 0; i < n; ++i) {
         args[i] = a[i];
-        const int stages = staged ? jtv_stages(a[i].P, a[i].y, a[i].w) : 0;
+        const int stages = staged ? jtv_stages(a[i].P, runs) : 0;
         jtv_grid(a[i].P, stages, share[i], args[i]);
         blocks[i] = args[i].gx * args[i].gy * args[i].gz;
         smem = std::max(smem, jtv_smem(a[i].P, stages));

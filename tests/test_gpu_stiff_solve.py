@@ -52,7 +52,7 @@ def test_stiff_update_in_a_group():
     own solo update, each within the bound of the exact one."""
     import torch
     import paper_2102_01604_gb300 as mpm
-    opts = mpm.make_opts(gn_iters=1, cg_iters=ITERS, init=False, graph=2)
+    opts = mpm.make_opts(gn_iters=1, cg_iters=ITERS, init=False, graph="phased")
     subs = []
     for shape, seed in (((28, 18, 10), 3), ((32, 20, 7), 4)):
         d = dataset(shape, seed=seed, n_echoes=(6, 6, 6))
