@@ -339,6 +339,31 @@ __device__ __forceinline__ void release_dependents()
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
+// A volume cut into tiles of 2^lx x 2^ly x 2^lz voxels, one per thread of a
+// block; blocks take tiles in order.  (The shape comes from fit_tile.)
+struct VoxelTiles {
+    int lx, ly, lz;
+    int tx, ty;               // tiles along x and y
+    long long count;          // below 2^32
+    // first voxel of tile t
+    __device__ __forceinline__ void corner(long long t, int& x, int& y, int& z) const
+    {
+        const unsigned u = (unsigned)t, r = u / (unsigned)tx;
+        x = (int)(u - r * (unsigned)tx) << lx;
+        y = (int)(r % (unsigned)ty) << ly;
+        z = (int)(r / (unsigned)ty) << lz;
+    }
+    // this thread's voxel of tile t (it may lie outside the volume)
+    __device__ __forceinline__ void voxel(long long t, int& x, int& y, int& z) const
+    {
+        corner(t, x, y, z);
+        const int i = threadIdx.x;
+        x += i & ((1 << lx) - 1);
+        y += (i >> lx) & ((1 << ly) - 1);
+        z += i >> (lx + ly);
+    }
+};
+
 template <typename T>
 __device__ __forceinline__ float load_echo(const T* p, long long i);
 

@@ -34,6 +34,27 @@ public:
     }
 };
 
+// Extents 2^l[d] of the tiles that a volume of n[0] x n[1] x n[2] voxels is cut
+// into, one thread per voxel.  On entry l holds the shape wanted in a volume
+// large along every axis.  An axis that a half as long tile covers gives its
+// factor to the shortest side that does not cover its own axis yet (the first of
+// equals): a volume one voxel thick keeps whole blocks at work.
+inline void fit_tile(const int (&n)[3], int (&l)[3])
+{
+    int spare = 0;
+    for (int d = 0; d < 3; ++d)
+        while (l[d] > 0 && (1 << (l[d] - 1)) >= n[d]) {
+            --l[d];
+            ++spare;
+        }
+    for (; spare > 0; --spare) {
+        int s = -1;
+        for (int d = 0; d < 3; ++d)
+            if ((1LL << l[d]) < n[d] && (s < 0 || l[d] < l[s])) s = d;
+        ++l[s < 0 ? 2 : s];              // the whole volume is smaller than a tile
+    }
+}
+
 // Share of the GPU one fit keeps busy: about 2^21 voxels keep every kernel of
 // a fit at a full wave, so larger volumes count as 1, smaller ones pro rata.
 inline double gpu_load(long long n_vox)

@@ -57,6 +57,16 @@ cudaError_t smem_opt_in(OncePerDevice& once, F* f, int bytes)
         once, [&] { return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes); });
 }
 
+// Tiles of kBlock voxels, 2^lx x 2^ly x 2^lz where the volume is that large.
+inline VoxelTiles voxel_tiles(int nx, int ny, int nz, int lx, int ly, int lz)
+{
+    const int n[3] = {nx, ny, nz};
+    int l[3] = {lx, ly, lz};
+    fit_tile(n, l);
+    auto cut = [&](int d) { return (int)(((long long)n[d] + (1 << l[d]) - 1) >> l[d]); };
+    return VoxelTiles{l[0], l[1], l[2], cut(0), cut(1), (long long)cut(0) * cut(1) * cut(2)};
+}
+
 // Launches f; with `overlap`, so that it may start before its predecessor on
 // the stream has finished (programmatic dependent launch): f must call
 // wait_predecessor.

@@ -86,25 +86,32 @@ struct ProjBufs {
 // Blocks of the two kernels below take compact tiles, so that the neighbouring
 // rows and planes they gather from stay in L1 (both kernels at 176x240x256, three
 // scans: 2.16 ms with 8 x 4 x 8, 2.18 with 8 x 8 x 4, 2.23 with 16 x 8 x 2, 2.34
-// with 4 x 8 x 8, 2.39 with 32 x 4 x 2).
-constexpr int kTX = 8, kTY = 4, kTZ = 8;
+// with 4 x 8 x 8, 2.39 with 32 x 4 x 2).  Thin grids take other shapes of the same
+// size: with 8 x 4 x 8 for all, one warp in eight works where the grid is one
+// slice (both kernels at 512x512x1 234 us, 72 with 16 x 16 x 1; 1x256x256 105 and
+// 63; 320x320x4 142 and 101).
+constexpr int kProjLX = 3, kProjLY = 2, kProjLZ = 3;
 
-struct TileGrid {
-    int tx, ty;
-    long long tiles;
-    __host__ __device__ TileGrid(int nx, int ny, int nz)
-        : tx((nx + kTX - 1) / kTX), ty((ny + kTY - 1) / kTY),
-          tiles((long long)tx * ty * ((nz + kTZ - 1) / kTZ)) {}
-    // this thread's voxel of tile t
-    __device__ __forceinline__ void voxel(long long t, int& x, int& y, int& z) const
-    {
-        const unsigned u = (unsigned)t;                  // tiles of a grid with at most 2^31 voxels a plane
-        const unsigned r = u / (unsigned)tx;
-        x = (int)(u - r * (unsigned)tx) * kTX + (int)(threadIdx.x % kTX);
-        y = (int)(r % (unsigned)ty) * kTY + (int)(threadIdx.x / kTX % kTY);
-        z = (int)(r / (unsigned)ty) * kTZ + (int)(threadIdx.x / (kTX * kTY));
+static VoxelTiles proj_tiles(int nx, int ny, int nz)
+{
+    return voxel_tiles(nx, ny, nz, kProjLX, kProjLY, kProjLZ);
+}
+
+static bool usual_tiles(const VoxelTiles& g) { return g.lx == kProjLX && g.ly == kProjLY && g.lz == kProjLZ; }
+
+// This thread's voxel of tile t.  USUAL: the usual shape, as constants (as
+// variables they cost the two kernels 0.8% at 176x240x256).
+template <bool USUAL>
+__device__ __forceinline__ void proj_voxel(const VoxelTiles& g, long long t, int& x, int& y, int& z)
+{
+    VoxelTiles u = g;
+    if (USUAL) {
+        u.lx = kProjLX;
+        u.ly = kProjLY;
+        u.lz = kProjLZ;
     }
-};
+    u.voxel(t, x, y, z);
+}
 
 // Reconstruction coordinate of acquisition voxel (i, j, k); true when it lies
 // in [0, n_d - 1] on every axis.
@@ -266,24 +273,23 @@ __device__ __forceinline__ F gather_pullers(const ProjC& q, int x, int y, int z,
 // It took 419 us per contrast at 176x240x256 with 64-bit divisions for the
 // voxel's indices, all corners behind branches, four maps for every contrast
 // and 64 B records staged in shared memory.
-template <int K, int PRE, typename XT>
+template <int K, int PRE, typename XT, bool USUAL>
 __global__ void __launch_bounds__(kBlock) k_grad_hess_proj(DevProblem P, ProjC q, int c,
                                                            const float* __restrict__ y,
                                                            const XT* __restrict__ x,
                                                            const float* __restrict__ b1p,
                                                            const float* __restrict__ b1m,
                                                            float4* __restrict__ gh, double* nll,
-                                                           Reduce red)
+                                                           Reduce red, VoxelTiles tg)
 {
     constexpr int T = K * (K + 1) / 2;
     const long long M = q.M;
     const GhPlanes out = gh_planes(gh, M);
-    const TileGrid tg(q.mx, q.my, q.mz);
     Acc nll_acc;
-    for (long long t = blockIdx.x; t < tg.tiles; t += gridDim.x) {
+    for (long long t = blockIdx.x; t < tg.count; t += gridDim.x) {
         int i, j, k;
-        if (t + gridDim.x < tg.tiles) {   // the next tile's echoes and B1 values into L2
-            tg.voxel(t + gridDim.x, i, j, k);
+        if (t + gridDim.x < tg.count) {   // the next tile's echoes and B1 values into L2
+            proj_voxel<USUAL>(tg, t + gridDim.x, i, j, k);
             if (i < q.mx && j < q.my && k < q.mz) {
                 const long long mn = i + (long long)q.mx * (j + (long long)q.my * k);
                 for (int e = 0; e < P.n_echoes[c]; ++e) prefetch_l2(x + e * M + mn);
@@ -291,7 +297,7 @@ __global__ void __launch_bounds__(kBlock) k_grad_hess_proj(DevProblem P, ProjC q
                 if (b1m) prefetch_l2(b1m + mn);
             }
         }
-        tg.voxel(t, i, j, k);
+        proj_voxel<USUAL>(tg, t, i, j, k);
         if (i >= q.mx || j >= q.my || k >= q.mz) continue;
         const long long m = i + (long long)q.mx * (j + (long long)q.my * k);
         float G[K], H[T];
@@ -373,10 +379,11 @@ struct PushInto {
 // records, 64-bit divisions, linear blocks and every point of the box tested;
 // both passes together took 2.73 ms, 2.16 ms now.
 // IT: an index type that holds every acquisition voxel's index.
-template <int K, typename IT>
+template <int K, typename IT, bool USUAL>
 __global__ void __launch_bounds__(kBlock, 4) k_push_all(DevProblem P, DevProj Q, ProjBufs B,
                                                      float* __restrict__ g, float* __restrict__ h,
-                                                     const double* nll_parts, double* nll)
+                                                     const double* nll_parts, double* nll,
+                                                     VoxelTiles tg)
 {
     constexpr int T = K * (K + 1) / 2;
     constexpr int CH = K + T;                     // channels: g, then the packed H
@@ -386,10 +393,9 @@ __global__ void __launch_bounds__(kBlock, 4) k_push_all(DevProblem P, DevProj Q,
         for (int c = 0; c < Q.C; ++c) s += nll_parts[c];
         *nll = s;
     }
-    const TileGrid tg(P.nx, P.ny, P.nz);
-    for (long long t = blockIdx.x; t < tg.tiles; t += gridDim.x) {
+    for (long long t = blockIdx.x; t < tg.count; t += gridDim.x) {
         int x, y, z;
-        tg.voxel(t, x, y, z);
+        proj_voxel<USUAL>(tg, t, x, y, z);
         if (x >= P.nx || y >= P.ny || z >= P.nz) continue;
         const long long n = x + (long long)P.nx * (y + (long long)P.ny * z);
         float A[CH];
@@ -560,9 +566,9 @@ static ProjWs proj_layout(const DevProblem& P, const DevProj& Q, int call, void*
     return W;
 }
 
-static int tile_blocks(const TileGrid& g)
+static int tile_blocks(const VoxelTiles& g)
 {
-    return (int)std::max(1LL, std::min(g.tiles, 8LL * kNumSm));
+    return (int)std::max(1LL, std::min(g.count, 8LL * kNumSm));
 }
 
 // The pass of contrast c, which depends on K maps.
@@ -571,16 +577,21 @@ static cudaError_t grad_hess_proj_c(const DevProblem& P, const DevProj& Q, int c
                                     const float* y, const ProjWs& W, Reduce red, cudaStream_t st)
 {
     const ProjC& q = Q.c[c];
-    const int grid = tile_blocks(TileGrid(q.mx, q.my, q.mz));
+    const VoxelTiles tg = proj_tiles(q.mx, q.my, q.mz);
+    const int grid = tile_blocks(tg);
     LaunchScope ls(MPM_KERNEL_GRAD_HESS_PROJ, st);
-    if (in.echo_dtype == 1)
-        k_grad_hess_proj<K, PRE, __nv_bfloat16><<<grid, kBlock, 0, st>>>(
-            P, q, c, y, static_cast<const __nv_bfloat16*>(in.x[c]), in.b1p[c], in.b1m[c], W.gh[c],
-            W.nll_parts + c, red);
-    else
-        k_grad_hess_proj<K, PRE, float><<<grid, kBlock, 0, st>>>(
-            P, q, c, y, static_cast<const float*>(in.x[c]), in.b1p[c], in.b1m[c], W.gh[c],
-            W.nll_parts + c, red);
+    auto launch = [&](auto* x, auto f) {
+        f<<<grid, kBlock, 0, st>>>(P, q, c, y, x, in.b1p[c], in.b1m[c], W.gh[c], W.nll_parts + c, red, tg);
+    };
+    const bool usual = usual_tiles(tg);
+    if (in.echo_dtype == 1) {
+        using XT = __nv_bfloat16;
+        launch(static_cast<const XT*>(in.x[c]),
+               usual ? k_grad_hess_proj<K, PRE, XT, true> : k_grad_hess_proj<K, PRE, XT, false>);
+    } else {
+        launch(static_cast<const float*>(in.x[c]),
+               usual ? k_grad_hess_proj<K, PRE, float, true> : k_grad_hess_proj<K, PRE, float, false>);
+    }
     return cudaGetLastError();
 }
 
@@ -602,9 +613,11 @@ static cudaError_t grad_hess_proj_k(const DevProblem& P, const DevProj& Q, const
     LaunchScope ls(MPM_KERNEL_RESLICE, st);
     bool i32 = true;
     for (int c = 0; c < Q.C; ++c) i32 = i32 && Q.c[c].M <= 0xffffffffLL;
-    const int grid = tile_blocks(TileGrid(P.nx, P.ny, P.nz));
-    if (i32) k_push_all<K, unsigned><<<grid, kBlock, 0, st>>>(P, Q, B, g, h, W.nll_parts, nll);
-    else k_push_all<K, long long><<<grid, kBlock, 0, st>>>(P, Q, B, g, h, W.nll_parts, nll);
+    const VoxelTiles tg = proj_tiles(P.nx, P.ny, P.nz);
+    const int grid = tile_blocks(tg);
+    const auto push = usual_tiles(tg) ? (i32 ? k_push_all<K, unsigned, true> : k_push_all<K, long long, true>)
+                                      : (i32 ? k_push_all<K, unsigned, false> : k_push_all<K, long long, false>);
+    push<<<grid, kBlock, 0, st>>>(P, Q, B, g, h, W.nll_parts, nll, tg);
     return cudaGetLastError();
 }
 
