@@ -22,8 +22,11 @@
 // cycle symmetric, so plain CG may use it.
 //
 // Every kernel below takes tiles of 32 x 4 x 2 voxels, one per thread: no
-// division per voxel, and the rows and planes a stencil shares stay in L1.  An
-// iteration at the finest level is four launches: the matvec, the update with
+// division per voxel, and the rows and planes a stencil shares stay in L1.
+// Levels shorter than that along an axis take other shapes of the same size (with
+// 32 x 4 x 2 for all, 12 iterations at 8x512x512 took 8.13 ms, 3.47 with 8 x 8 x
+// 4; 1x256x256 2.45 and 0.96).  An iteration at the finest level is four
+// launches: the matvec, the update with
 // the first smoothing sweep (it has the residual at hand), the residual's
 // restriction, and the last sweep with the coarse correction (each neighbour's
 // parent added as it is read) and r . z.  They are bound by the latency of
@@ -46,6 +49,7 @@ namespace mpm {
 
 constexpr long long kMgMinVoxels = 512;
 constexpr int kMgMaxLevels = 16;
+constexpr int kMgLX = 5, kMgLY = 2, kMgLZ = 1;      // tiles of 32 x 4 x 2 voxels
 
 struct MgLevel {
     int nx, ny, nz;
@@ -55,6 +59,7 @@ struct MgLevel {
     float4* r;          // right-hand side of this level's cycle
     float4* x;          // result of this level's cycle
     float4* t;          // ping-pong partner of x for the sweeps
+    VoxelTiles tiles;
 };
 
 struct MgBufs {
@@ -103,6 +108,7 @@ static size_t mg_carve(const DevProblem& P, int levels, void* ws, MgBufs* B)
         v.ny = dims[l][1];
         v.nz = dims[l][2];
         v.N = (long long)v.nx * v.ny * v.nz;
+        v.tiles = voxel_tiles(v.nx, v.ny, v.nz, kMgLX, kMgLY, kMgLZ);
         v.h = l == 0 ? nullptr : static_cast<const float*>(take(sizeof(float) * P.T * v.N));
         v.kap = static_cast<float*>(take(sizeof(float) * 3 * v.N));
         v.r = static_cast<float4*>(take(sizeof(float4) * v.N));
@@ -144,30 +150,17 @@ __device__ __forceinline__ void level_edges(const MgLevel& L, int x, int y, int 
     for (int m = 0; m < 6; ++m) c[m] = ok[m] ? k[m] : 0.0f;
 }
 
-// Blocks take tiles of 32 x 4 x 2 voxels in order, one voxel per thread.
-constexpr int kMgTX = 32, kMgTY = 4, kMgTZ = 2;
-
-struct MgTiles {
-    int tx, ty;
-    long long count;
-    __host__ __device__ explicit MgTiles(const MgLevel& L)
-        : tx((L.nx + kMgTX - 1) / kMgTX), ty((L.ny + kMgTY - 1) / kMgTY),
-          count((long long)tx * ty * ((L.nz + kMgTZ - 1) / kMgTZ)) {}
-    // This thread's voxel of tile t; false where it lies outside the level.
-    __device__ __forceinline__ bool voxel(const MgLevel& L, long long t, int& x, int& y, int& z, long long& n) const
-    {
-        const unsigned u = (unsigned)t, r = u / (unsigned)tx;      // tiles < 2^32: N < 2^40
-        x = (int)(u - r * (unsigned)tx) * kMgTX + (int)(threadIdx.x % kMgTX);
-        y = (int)(r % (unsigned)ty) * kMgTY + (int)(threadIdx.x / kMgTX % kMgTY);
-        z = (int)(r / (unsigned)ty) * kMgTZ + (int)(threadIdx.x / (kMgTX * kMgTY));
-        n = x + (long long)L.nx * (y + (long long)L.ny * z);
-        return x < L.nx && y < L.ny && z < L.nz;
-    }
-};
+// This thread's voxel of tile t; false where it lies outside the level.
+__device__ __forceinline__ bool tile_voxel(const MgLevel& L, long long t, int& x, int& y, int& z, long long& n)
+{
+    L.tiles.voxel(t, x, y, z);
+    n = x + (long long)L.nx * (y + (long long)L.ny * z);
+    return x < L.nx && y < L.ny && z < L.nz;
+}
 
 static int mg_grid(const MgLevel& L)
 {
-    const long long cap = 8LL * kNumSm, t = MgTiles(L).count;
+    const long long cap = 8LL * kNumSm, t = L.tiles.count;
     return (int)(t < cap ? t : cap);
 }
 
@@ -223,11 +216,10 @@ __device__ __forceinline__ bool solve_done(const WsHeader* hdr) { return hdr->sc
 __global__ void __launch_bounds__(kBlock) k_mg_kappa0(DevProblem P, MgLevel L, const float* __restrict__ w)
 {
     const long long sxy = (long long)L.nx * L.ny;
-    const MgTiles tiles(L);
-    for (long long t = blockIdx.x; t < tiles.count; t += gridDim.x) {
+    for (long long t = blockIdx.x; t < L.tiles.count; t += gridDim.x) {
         int x, y, z;
         long long n;
-        if (!tiles.voxel(L, t, x, y, z, n)) continue;
+        if (!tile_voxel(L, t, x, y, z, n)) continue;
         const float wn = __ldg(w + n);
         L.kap[n] = x + 1 < L.nx ? (wn + __ldg(w + n + 1)) * P.ihx2 : 0.0f;
         L.kap[L.N + n] = y + 1 < L.ny ? (wn + __ldg(w + n + L.nx)) * P.ihy2 : 0.0f;
@@ -243,11 +235,10 @@ __global__ void __launch_bounds__(kBlock) k_mg_coarsen(DevProblem P, MgLevel F, 
     const int T = P.T;
     const float* fh = F.h ? F.h : h0;
     float* ch = const_cast<float*>(C.h);
-    const MgTiles tiles(C);
-    for (long long t = blockIdx.x; t < tiles.count; t += gridDim.x) {
+    for (long long t = blockIdx.x; t < C.tiles.count; t += gridDim.x) {
         int cx, cy, cz;
         long long c;
-        if (!tiles.voxel(C, t, cx, cy, cz, c)) continue;
+        if (!tile_voxel(C, t, cx, cy, cz, c)) continue;
         float hs[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
         float ks[3] = {0, 0, 0};
         for (int dz = 0; dz < 2; ++dz)
@@ -310,11 +301,10 @@ __global__ void __launch_bounds__(kBlock, 4) k_mg_sweep(DevProblem P, MgLevel L,
     constexpr int T = K * (K + 1) / 2;
     if (solve_done(hdr)) return;
     Acc acc;
-    const MgTiles tiles(L);
-    for (long long t = blockIdx.x; t < tiles.count; t += gridDim.x) {
+    for (long long t = blockIdx.x; t < L.tiles.count; t += gridDim.x) {
         int x, y, z;
         long long n;
-        if (!tiles.voxel(L, t, x, y, z, n)) continue;
+        if (!tile_voxel(L, t, x, y, z, n)) continue;
         float c[6];
         long long off[6];
         level_edges(L, x, y, z, n, c, off);
@@ -361,25 +351,30 @@ __global__ void __launch_bounds__(kBlock, 4) k_mg_sweep(DevProblem P, MgLevel L,
     }
 }
 
-// Restricted residual: C.r = P' (F.r - A_F x).  One fine voxel per thread; a
-// tile's 16 x 2 x 1 coarse voxels are summed in the warp (the pair along x) and
-// in shared memory (y, then z).
+// Restricted residual: C.r = P' (F.r - A_F x).  One fine voxel per thread; the
+// children of a coarse voxel lie in one tile and are summed in the warp (the pair
+// along x) and in shared memory (y, then z).  Along an axis on which the tile is
+// one voxel long there is one voxel, and nothing to pair.
 template <int K>
 __global__ void __launch_bounds__(kBlock, 4) k_mg_restrict(DevProblem P, MgLevel F, MgLevel C, const float* h0,
                                                         const float4* __restrict__ xf, const WsHeader* hdr)
 {
     constexpr int T = K * (K + 1) / 2;
-    __shared__ float4 part[kMgTZ][kMgTY][kMgTX / 2];
+    __shared__ float4 part[kBlock];
     if (solve_done(hdr)) return;
-    const MgTiles tiles(F);
-    const int lane = threadIdx.x % kMgTX, ty = threadIdx.x / kMgTX % kMgTY, tz = threadIdx.x / (kMgTX * kMgTY);
-    for (long long t = blockIdx.x; t < tiles.count; t += gridDim.x) {
+    const int tid = threadIdx.x;
+    const int px = F.tiles.lx > 0, py = F.tiles.ly > 0, pz = F.tiles.lz > 0;    // pairs along an axis
+    const int lx = F.tiles.lx - px, ly = F.tiles.ly - py, lz = F.tiles.lz - pz;     // the tile's coarse voxels
+    const int u = tid & ((1 << lx) - 1), v = (tid >> lx) & ((1 << ly) - 1), s = tid >> (lx + ly);
+    const int sy = 1 << lx, sz = sy << F.tiles.ly;                                  // strides of part
+    const int p0 = u + (v << py) * sy + (s << pz) * sz;
+    for (long long t = blockIdx.x; t < F.tiles.count; t += gridDim.x) {
         int x, y, z;
         long long n;
         float d[K];
 #pragma unroll
         for (int a = 0; a < K; ++a) d[a] = 0.0f;
-        if (tiles.voxel(F, t, x, y, z, n)) {
+        if (tile_voxel(F, t, x, y, z, n)) {
             float c[6];
             long long off[6];
             level_edges(F, x, y, z, n, c, off);
@@ -390,17 +385,20 @@ __global__ void __launch_bounds__(kBlock, 4) k_mg_restrict(DevProblem P, MgLevel
 #pragma unroll
             for (int a = 0; a < K; ++a) d[a] = r[a] - ax[a];
         }
+        if (px) {
 #pragma unroll
-        for (int a = 0; a < K; ++a) d[a] += __shfl_down_sync(0xffffffffu, d[a], 1);
-        if (!(lane & 1)) part[tz][ty][lane >> 1] = pack4<K>(d);
+            for (int a = 0; a < K; ++a) d[a] += __shfl_down_sync(0xffffffffu, d[a], 1);
+        }
+        if (!px || !(tid & 1)) part[tid >> px] = pack4<K>(d);
         __syncthreads();
-        if (threadIdx.x < kMgTX / 2 * (kMgTY / 2)) {
-            const int u = threadIdx.x % (kMgTX / 2), v = threadIdx.x / (kMgTX / 2);
-            const float4 s = add4(add4(part[0][2 * v][u], part[0][2 * v + 1][u]),
-                                  add4(part[1][2 * v][u], part[1][2 * v + 1][u]));
-            // thread 0's voxel is the tile's corner
-            const int cx = ((x - lane) >> 1) + u, cy = ((y - ty) >> 1) + v, cz = (z - tz) >> 1;
-            if (cx < C.nx && cy < C.ny && cz < C.nz) C.r[cx + (long long)C.nx * (cy + (long long)C.ny * cz)] = s;
+        if (tid < 1 << (lx + ly + lz)) {
+            auto line = [&](int p) { return py ? add4(part[p], part[p + sy]) : part[p]; };
+            const float4 sum = pz ? add4(line(p0), line(p0 + sz)) : line(p0);
+            // the tile's corner, halved, is its first coarse voxel
+            int bx, by, bz;
+            F.tiles.corner(t, bx, by, bz);
+            const int cx = (bx >> 1) + u, cy = (by >> 1) + v, cz = (bz >> 1) + s;
+            if (cx < C.nx && cy < C.ny && cz < C.nz) C.r[cx + (long long)C.nx * (cy + (long long)C.ny * cz)] = sum;
         }
         __syncthreads();
     }
@@ -505,11 +503,10 @@ __global__ void __launch_bounds__(kBlock) k_mgcg_init(DevProblem P, MgLevel L0, 
                                                       WsHeader* hdr, double* resid, Reduce red)
 {
     Acc rr;
-    const MgTiles tiles(L0);
-    for (long long t = blockIdx.x; t < tiles.count; t += gridDim.x) {
+    for (long long t = blockIdx.x; t < L0.tiles.count; t += gridDim.x) {
         int x, yy, z;
         long long n;
-        if (!tiles.voxel(L0, t, x, yy, z, n)) continue;
+        if (!tile_voxel(L0, t, x, yy, z, n)) continue;
         float c[6];
         long long off[6];
         level_edges(L0, x, yy, z, n, c, off);
@@ -607,11 +604,10 @@ __global__ void __launch_bounds__(kBlock, 4) k_mgcg_matvec(DevProblem P, MgLevel
         }
     };
     Acc acc;
-    const MgTiles tiles(L0);
-    for (long long t = blockIdx.x; t < tiles.count; t += gridDim.x) {
+    for (long long t = blockIdx.x; t < L0.tiles.count; t += gridDim.x) {
         int x, y, zz;
         long long n;
-        if (!tiles.voxel(L0, t, x, y, zz, n)) continue;
+        if (!tile_voxel(L0, t, x, y, zz, n)) continue;
         float c[6];
         long long off[6];
         level_edges(L0, x, y, zz, n, c, off);
@@ -673,11 +669,10 @@ __global__ void __launch_bounds__(kBlock, 4) k_mgcg_update(DevProblem P, MgLevel
     if (s_done) return;
     const float alpha = s_alpha;
     Acc acc;
-    const MgTiles tiles(L0);
-    for (long long t = blockIdx.x; t < tiles.count; t += gridDim.x) {
+    for (long long t = blockIdx.x; t < L0.tiles.count; t += gridDim.x) {
         int x, y, z;
         long long n;
-        if (!tiles.voxel(L0, t, x, y, z, n)) continue;
+        if (!tile_voxel(L0, t, x, y, z, n)) continue;
         float xv[K], pv[K], qv[K], rv[K];
         unpack4<K>(p[n], pv);
         unpack4<K>(q[n], qv);
