@@ -222,14 +222,17 @@ __device__ __forceinline__ bool block_var_f32(const float (&M)[K][K], bool want_
 #pragma unroll
     for (int a = 0; a < K; ++a)
 #pragma unroll
-        for (int b = 0; b <= a; ++b) A[a][b] = __fmul_rn(__fmul_rn(M[a][b], sc[a]), sc[b]);
+        for (int b = 0; b < a; ++b) A[a][b] = __fmul_rn(__fmul_rn(M[a][b], sc[a]), sc[b]);
     float L[K][K], inv[K];
     float psum = 1.0f;              // product of the pivots, each in [kPivotMin, about 1]
 #pragma unroll
     for (int j = 0; j < K; ++j) {
-        float p = A[j][j];
+        // the diagonal's last product is not rounded by itself (rounded, the
+        // variance of the last map was 1.17e-7 off instead of 1.14e-7)
+        const float t = __fmul_rn(M[j][j], sc[j]);
+        float p = j == 0 ? __fmul_rn(t, sc[j]) : fmaf(t, sc[j], -__fmul_rn(L[j][0], L[j][0]));
 #pragma unroll
-        for (int k = 0; k < j; ++k) p = fmaf(-L[j][k], L[j][k], p);
+        for (int k = 1; k < j; ++k) p = fmaf(-L[j][k], L[j][k], p);
         if (!(p >= kPivotMin)) return false;
         inv[j] = rsqrtf(p);
         L[j][j] = p * inv[j];
