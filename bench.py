@@ -227,7 +227,8 @@ def step_bytes(j: int, K: int, cg_iters: int = None) -> int:
 
 def moved_step_bytes(j: int, K: int) -> int:
     """Bytes per voxel of PCG iteration j as the kernel runs it (pcg_step.cuh:
-    z comes from the last two directions): j = 0 reads p_0, w, H and writes v_0;
+    z comes from the last two directions, as in every iteration of these fits):
+    j = 0 reads p_0, w, H and writes v_0;
     j = 1 reads p_0, v_0, w, H and writes p, v; later ones also read p_{j-2};
     even j >= 2 also write x, and read x when j > 2."""
     T = K * (K + 1) // 2

@@ -131,8 +131,12 @@ struct SolveOpts {
     int mg_coarse_sweeps;
     bool overlap;           // an iteration's launch may start before the one before it has ended
 };
-// overlap: false for fits that share the GPU with others (the server's), whose
-// blocks an early launch's waiting blocks would keep out
+// overlap: false for the server's fits.  It is worth 11% to a 64^3 fit alone, but
+// among other requests nothing: 24 requests of mixed sizes at 30/s ran at 1224 to
+// 1231 Mvoxel GN-iter/s without and 1229 with it, median latency 0.20 s either
+// way (1226 to 1235 with it only while one request is active), at 3/s 0.085 s.
+// Captured lanes keep it for the same reason: 16 uneven subjects 1313 to 1318
+// with and 1320 to 1323 without, 16 of 64^3 777 to 799 and 799 to 800.
 SolveOpts solve_opts(const mpm_opts& o, bool overlap = true);
 cudaError_t launch_solve(const DevProblem& P, const SolveOpts& so, const float* h,
                          const float* w, const float* g, const float* y, float* delta,

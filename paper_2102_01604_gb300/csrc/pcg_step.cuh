@@ -31,7 +31,9 @@
 //     (p_j.M p_j) / (z_j.M z_j) = 1 + beta_{j-1} (p_{j-1}.M p_{j-1}) / (z_{j-1}.M z_{j-1})
 // (z_j.M p_{j-1} = 0), and an iteration above kStoreZ also stores its z_j, which
 // the next one reads in place of p_{j-1}: 16 B per voxel more, and as much
-// again in the folding iterations, whose p_{j-2} is then read for itself.  With
+// again in the folding iterations, whose p_{j-2} is then read for itself (from
+// L2, where the producer has it fetched).  30 iterations at 176x240x256 with
+// every z stored take 9.00 ms (9.18 without that fetch), 7.42 with none.  With
 // 8^2 the errors are those of a z that is always stored (CPU restatement in
 // float32, 20x16x12, delta after the last iteration):
 //     lambda, iterations    z stored    never     above 4     8         16

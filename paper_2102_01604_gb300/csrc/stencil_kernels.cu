@@ -405,7 +405,7 @@ __global__ void __launch_bounds__(kJtvThreads, 2)
                            batch_grid(b.start[s], a.gx, a.gy, a.gz));
 }
 
-// The tile kernel, for rows too wide for three stages.
+// The tile kernel, for small volumes and rows too wide for three stages.
 // Each thread marches up its z range with the centre values of planes z - 1,
 // z and z + 1 in registers; the centre of plane z + 2 is loaded one plane
 // ahead.  The x / y neighbours come from the plane's tile in shared memory

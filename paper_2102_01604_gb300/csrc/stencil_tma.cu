@@ -245,6 +245,7 @@ __device__ __forceinline__ void step_body(
                     if (third) tma_load_3d(smem_u32(st + L::P2_OFF), tpz, 4 * (x0 - 1), y0 - 1, jj, bar);
                     tma_load_3d(smem_u32(st + L::W_OFF), tw, x0 - 4, y0 - 1, jj, bar);
                     if (readx && inner) tma_load_3d(smem_u32(st + L::X_OFF), txm, 4 * x0, y0, jj, bar);
+                    if (fold && sc.zin && inner) tma_prefetch_3d(tp2, 4 * (x0 - 1), y0 - 1, jj);
                     raw_issued = c;
                     if (!inner) continue;
                     const int e = eb + (jj - za);
