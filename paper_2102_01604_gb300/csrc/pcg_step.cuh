@@ -223,14 +223,14 @@ __device__ __forceinline__ StepScalars step_start(const SolveScalars& sc)
 }
 
 // z_j and p_j of one point from p1 = p_{j-1}, v = v_{j-1} and pz = p_{j-2}, or
-// z_{j-1} where that was stored (j = 0: p1 is p_0 and v, pz are not read; j =
+// z_{j-1} where that was stored (zin; j = 0: p1 is p_0 and v, pz are not read; j =
 // 1: pz is not read).
 template <int MODE>
-__device__ __forceinline__ void step_point(const StepScalars& s, const Maps& p1, const Maps& v,
+__device__ __forceinline__ void step_point(const StepScalars& s, bool zin, const Maps& p1, const Maps& v,
                                            const Maps& pz, Maps& zj, Maps& pj)
 {
     Maps z = p1;                                                          // z_{j-1}
-    if (MODE >= kModeStep) z = s.zin ? pz : axpy(-s.beta_prev, pz, p1);
+    if (MODE >= kModeStep) z = zin ? pz : axpy(-s.beta_prev, pz, p1);
     zj = MODE == kModeFirst ? z : axpy(-s.alpha, v, z);
     pj = MODE == kModeFirst ? z : axpy(s.beta, p1, zj);
 }

@@ -727,8 +727,11 @@ __global__ void __launch_bounds__(kBlock) k_pcg_init_batch(const __grid_constant
 // marching a run of z planes; each neighbour's p_j is formed from its own
 // p_{j-1}, v_{j-1} and p_{j-2} (or the stored z_{j-1}) read from memory.  Used
 // for volumes or pointers the TMA kernel cannot take (a volume smaller than a tile, unaligned buffers).
+// Three blocks per SM, with a few registers spilled: bound by the latency of its
+// neighbours' loads (30 iterations of 2x1024x512 with four maps 11.1 ms, 11.5 with
+// the two that 106 registers leave; three maps 9.9 and 13.0).
 template <int K, int MODE>
-__global__ void __launch_bounds__(kBlock) k_pcg_step(DevProblem P, int zc, int j, int want_rr,
+__global__ void __launch_bounds__(kBlock, 3) k_pcg_step(DevProblem P, int zc, int j, int want_rr,
                                                      const float* __restrict__ h,
                                                      const float* __restrict__ w,
                                                      const float4* __restrict__ pin,
@@ -762,11 +765,15 @@ __global__ void __launch_bounds__(kBlock) k_pcg_step(DevProblem P, int zc, int j
     const int z1p = min(P.nz, z0p + zc);
     float part[kStepSums] = {};
     const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-    const float4* __restrict__ pz = sc.zin ? zprev : p2;
-    auto point = [&](long long m, Maps& zj, Maps& pj) {
-        step_point<MODE>(sc, pin[m], first ? zero : vin[m], MODE >= kModeStep ? pz[m] : zero, zj, pj);
-    };
-    if (x < P.nx && yy < P.ny) {
+    // A copy of the loop for each case of a stored z: with a test at each of a
+    // voxel's seven points, 30 iterations of 2x1024x512 with three maps took 13.6
+    // ms, with the test of zout alone 12.0, where without either they took 10.9.
+    auto march = [&](auto zin_c, auto zout_c) {
+        constexpr bool ZIN = decltype(zin_c)::value, ZOUT = decltype(zout_c)::value;
+        const float4* __restrict__ pz = ZIN ? zprev : p2;
+        auto point = [&](long long m, Maps& zj, Maps& pj) {
+            step_point<MODE>(sc, ZIN, pin[m], first ? zero : vin[m], MODE >= kModeStep ? pz[m] : zero, zj, pj);
+        };
         for (int z = z0p; z < z1p; ++z) {
             const long long n = x + (long long)P.nx * yy + sxy * z;
             const float wn = __ldg(w + n);
@@ -786,9 +793,22 @@ __global__ void __launch_bounds__(kBlock) k_pcg_step(DevProblem P, int zc, int j
             Maps v;
             step_voxel<K>(P, e.c, zj, pj, [&](int m) { return nb[m]; }, hv, want_rr, v, part);
             if (!first) pout[n] = pj.vec();
-            if (!first && sc.zout) zout[n] = zj.vec();
+            if (ZOUT) zout[n] = zj.vec();
             vout[n] = v.vec();
             if (MODE >= kModeFold) xacc[n] = fold_x(MODE == kModeFoldX ? xacc[n] : zero, sc, p2[n], pin[n]).vec();
+        }
+    };
+    if (x < P.nx && yy < P.ny) {
+        using Zin = std::bool_constant<(MODE >= kModeStep)>;      // z_{j-1} may have been stored
+        using Zout = std::bool_constant<!first>;
+        using No = std::false_type;
+        if (Zin::value && sc.zin) {
+            if (sc.zout) march(Zin(), Zout());
+            else march(Zin(), No());
+        } else if (Zout::value && sc.zout) {
+            march(No(), Zout());
+        } else {
+            march(No(), No());
         }
     }
     release_dependents();

@@ -350,7 +350,7 @@ __device__ __forceinline__ void step_body(
                     const float4* b2 = reinterpret_cast<const float4*>(st + L::P2_OFF);
                     const float* bw = reinterpret_cast<const float*>(st + L::W_OFF) + wcc;
                     const Maps p1 = bp[bc], pz = third ? Maps(b2[bc]) : zero;
-                    step_point<MODE>(sc, p1, first ? zero : Maps(bv[bc]), pz, zn, pn);
+                    step_point<MODE>(sc, sc.zin, p1, first ? zero : Maps(bv[bc]), pz, zn, pn);
                     wn = bw[0];
                     cxyn[0] = okxm ? (wn + bw[-1]) * P.ihx2 : 0.f;
                     cxyn[1] = okxp ? (wn + bw[1]) * P.ihx2 : 0.f;
@@ -360,7 +360,7 @@ __device__ __forceinline__ void step_body(
                         fp[bc] = pn.vec();
                         if (tid < L::NH) {
                             Maps hz, hpj;
-                            step_point<MODE>(sc, bp[hb], first ? zero : Maps(bv[hb]),
+                            step_point<MODE>(sc, sc.zin, bp[hb], first ? zero : Maps(bv[hb]),
                                              third ? Maps(b2[hb]) : zero, hz, hpj);
                             fp[hb] = hpj.vec();
                         }
