@@ -941,7 +941,8 @@ StencilGrid stencil_grid(const DevProblem& P, int tx, int ty, int waves, double 
 // block's shared memory; 0 (the tile kernel) where those do not fit, rows of
 // more than 1831 voxels at K = 4, and for small volumes, where the staged
 // kernel's longer start-up costs what it gives (64^3: 14.3 us staged, 14.6 not;
-// without runs of four, 61^3: 15.4 and 12.9; 181x217x181: 58 and 78).
+// without runs of four, 61^3: 15.4 and 12.9; 181x217x181: 58 and 78), and for
+// planes that leave a block's 1024 voxels mostly empty.
 constexpr long long kJtvStagedMinRuns = 1LL << 17, kJtvStagedMin = 1LL << 20;
 constexpr int kJtvSmemHalf = 110 * 1024, kJtvSmemMax = 220 * 1024;
 
@@ -952,9 +953,22 @@ static bool jtv_runs(const DevProblem& P, const float* y, const float* w)
     return P.nx % 4 == 0 && (reinterpret_cast<uintptr_t>(y) | reinterpret_cast<uintptr_t>(w)) % 16 == 0;
 }
 
+// Whether a plane has work enough for the staged kernel's blocks: one of them
+// takes as long as 2.3 tiles of 32 x 8 (2.9 without runs of four), so planes of
+// one or two tiles are faster in the tile kernel (8x8x8192 31.3 us, 48.8 staged;
+// 13x15x7000 43.1 and 53.1; 16x16x10000 54.2 and 57.0; but 16x20x6000 48.4 and
+// 37.1), those of two in long volumes only (16x16x4096 30.7 and 29.0; 16x16x1024
+// 21.0 and 15.2).
+static bool jtv_plane_fills(const DevProblem& P, bool runs)
+{
+    const long long tiles = (long long)((P.nx + kTileX - 1) / kTileX) * ((P.ny + kTileY - 1) / kTileY);
+    const long long blocks = ((long long)P.nx * P.ny + kJtvRun - 1) / kJtvRun;
+    return 10 * tiles >= (runs ? 23 : 29) * blocks || (runs && tiles >= 2 * blocks && P.N <= kJtvStagedMin);
+}
+
 static int jtv_stages(const DevProblem& P, bool runs)
 {
-    if (P.N < (runs ? kJtvStagedMinRuns : kJtvStagedMin)) return 0;
+    if (P.N < (runs ? kJtvStagedMinRuns : kJtvStagedMin) || !jtv_plane_fills(P, runs)) return 0;
     for (int n = kJtvStagesMax; n >= 3; --n)
         if (jtv_smem(P, n) <= (n > 3 ? kJtvSmemHalf : kJtvSmemMax)) return n;
     return 0;

@@ -101,7 +101,13 @@ def test_fit_without_padded_rows_matches_the_oracle():
     ((129, 95, 87), 0, True),
     ((129, 95, 87), 2, True),
     ((129, 95, 85), 0, False),          # below 2^20
-    ((3, 5, 70001), 1, True),
+    ((3, 5, 70001), 1, False),          # planes of one tile
+    ((8, 8, 4096), 0, False),
+    ((16, 16, 4096), 0, True),          # two, and not longer than 2^20 voxels
+    ((16, 16, 4097), 0, False),
+    ((16, 20, 4097), 0, True),          # three
+    ((15, 17, 4200), 0, True),
+    ((13, 15, 5500), 0, False),
     ((1500, 7, 101), 0, True),
     ((1828, 3, 200), 0, True),          # the widest row of its kind
     ((1832, 3, 200), 0, False),
