@@ -345,22 +345,14 @@ struct VoxelTiles {
     int lx, ly, lz;
     int tx, ty;               // tiles along x and y
     long long count;          // below 2^32
-    // first voxel of tile t
-    __device__ __forceinline__ void corner(long long t, int& x, int& y, int& z) const
-    {
-        const unsigned u = (unsigned)t, r = u / (unsigned)tx;
-        x = (int)(u - r * (unsigned)tx) << lx;
-        y = (int)(r % (unsigned)ty) << ly;
-        z = (int)(r / (unsigned)ty) << lz;
-    }
     // this thread's voxel of tile t (it may lie outside the volume)
     __device__ __forceinline__ void voxel(long long t, int& x, int& y, int& z) const
     {
-        corner(t, x, y, z);
+        const unsigned u = (unsigned)t, r = u / (unsigned)tx;
         const int i = threadIdx.x;
-        x += i & ((1 << lx) - 1);
-        y += (i >> lx) & ((1 << ly) - 1);
-        z += i >> (lx + ly);
+        x = ((int)(u - r * (unsigned)tx) << lx) + (i & ((1 << lx) - 1));
+        y = ((int)(r % (unsigned)ty) << ly) + ((i >> lx) & ((1 << ly) - 1));
+        z = ((int)(r / (unsigned)ty) << lz) + (i >> (lx + ly));
     }
 };
 

@@ -25,7 +25,7 @@
 // division per voxel, and the rows and planes a stencil shares stay in L1.
 // Levels shorter than that along an axis take other shapes of the same size (with
 // 32 x 4 x 2 for all, 12 iterations at 8x512x512 took 8.13 ms, 3.47 with 8 x 8 x
-// 4; 1x256x256 2.45 and 0.96).  An iteration at the finest level is four
+// 4; 1x256x256 2.45 and 0.95).  An iteration at the finest level is four
 // launches: the matvec, the update with
 // the first smoothing sweep (it has the residual at hand), the residual's
 // restriction, and the last sweep with the coarse correction (each neighbour's
@@ -33,7 +33,7 @@
 // their loads: all of a voxel's are issued at once, none behind a test of an
 // edge coefficient, and 64 registers keep four blocks on an SM (without that,
 // 15.5 ms; hints of the next tile into L2, 14.3).  Solve of 176x240x256, 12
-// iterations: 18.1 ms as seven kernels over linear 64-bit voxel indices, 14.0 ms.
+// iterations: 18.1 ms as seven kernels over linear 64-bit voxel indices, 13.7 ms.
 //
 // Vectors are voxel-interleaved (float4 per voxel, the fourth component zero
 // for K = 3); H and kappa are planar.  CG scalars stay on the device (last
@@ -150,10 +150,31 @@ __device__ __forceinline__ void level_edges(const MgLevel& L, int x, int y, int 
     for (int m = 0; m < 6; ++m) c[m] = ok[m] ? k[m] : 0.0f;
 }
 
+// A level's tiles.  USUAL: their shape as constants.  (As variables, and without
+// the bounds on the update's and the coarsening's registers, 11 iterations at
+// 45x62x49 took 930 us, 904 this way; 176x240x256 12.76 and 12.59 ms.)
+template <bool USUAL>
+__device__ __forceinline__ VoxelTiles tiles_of(const MgLevel& L)
+{
+    VoxelTiles t = L.tiles;
+    if (USUAL) {
+        t.lx = kMgLX;
+        t.ly = kMgLY;
+        t.lz = kMgLZ;
+    }
+    return t;
+}
+
+static bool usual_tiles(const MgLevel& L)
+{
+    return L.tiles.lx == kMgLX && L.tiles.ly == kMgLY && L.tiles.lz == kMgLZ;
+}
+
 // This thread's voxel of tile t; false where it lies outside the level.
+template <bool USUAL>
 __device__ __forceinline__ bool tile_voxel(const MgLevel& L, long long t, int& x, int& y, int& z, long long& n)
 {
-    L.tiles.voxel(t, x, y, z);
+    tiles_of<USUAL>(L).voxel(t, x, y, z);
     n = x + (long long)L.nx * (y + (long long)L.ny * z);
     return x < L.nx && y < L.ny && z < L.nz;
 }
@@ -213,13 +234,14 @@ __device__ __forceinline__ bool solve_done(const WsHeader* hdr) { return hdr->sc
 // ------------------------------------------------------------ hierarchy
 
 // Level 0 edge coefficients from the JTV weights.
+template <bool USUAL>
 __global__ void __launch_bounds__(kBlock) k_mg_kappa0(DevProblem P, MgLevel L, const float* __restrict__ w)
 {
     const long long sxy = (long long)L.nx * L.ny;
     for (long long t = blockIdx.x; t < L.tiles.count; t += gridDim.x) {
         int x, y, z;
         long long n;
-        if (!tile_voxel(L, t, x, y, z, n)) continue;
+        if (!tile_voxel<USUAL>(L, t, x, y, z, n)) continue;
         const float wn = __ldg(w + n);
         L.kap[n] = x + 1 < L.nx ? (wn + __ldg(w + n + 1)) * P.ihx2 : 0.0f;
         L.kap[L.N + n] = y + 1 < L.ny ? (wn + __ldg(w + n + L.nx)) * P.ihy2 : 0.0f;
@@ -229,7 +251,8 @@ __global__ void __launch_bounds__(kBlock) k_mg_kappa0(DevProblem P, MgLevel L, c
 
 // Galerkin coarse level: H summed over the children, each coarse edge the
 // sum of the fine edges crossing it (those of the children on the +a side).
-__global__ void __launch_bounds__(kBlock) k_mg_coarsen(DevProblem P, MgLevel F, MgLevel C,
+template <bool USUAL>
+__global__ void __launch_bounds__(kBlock, 4) k_mg_coarsen(DevProblem P, MgLevel F, MgLevel C,
                                                        const float* h0)
 {
     const int T = P.T;
@@ -238,7 +261,7 @@ __global__ void __launch_bounds__(kBlock) k_mg_coarsen(DevProblem P, MgLevel F, 
     for (long long t = blockIdx.x; t < C.tiles.count; t += gridDim.x) {
         int cx, cy, cz;
         long long c;
-        if (!tile_voxel(C, t, cx, cy, cz, c)) continue;
+        if (!tile_voxel<USUAL>(C, t, cx, cy, cz, c)) continue;
         float hs[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
         float ks[3] = {0, 0, 0};
         for (int dz = 0; dz < 2; ++dz)
@@ -292,7 +315,7 @@ __device__ __forceinline__ void direction_scalars(double rz, int first, WsHeader
 
 // One damped block-Jacobi sweep on a level; DOT: the result is z, and r . z is
 // reduced (`first`: of the first cycle).
-template <int K, int FROM, bool DOT>
+template <int K, int FROM, bool DOT, bool USUAL>
 __global__ void __launch_bounds__(kBlock, 4) k_mg_sweep(DevProblem P, MgLevel L, MgLevel C, const float* h0,
                                                      float omega, const float4* __restrict__ xin,
                                                      float4* __restrict__ xout, int first, WsHeader* hdr,
@@ -304,7 +327,7 @@ __global__ void __launch_bounds__(kBlock, 4) k_mg_sweep(DevProblem P, MgLevel L,
     for (long long t = blockIdx.x; t < L.tiles.count; t += gridDim.x) {
         int x, y, z;
         long long n;
-        if (!tile_voxel(L, t, x, y, z, n)) continue;
+        if (!tile_voxel<USUAL>(L, t, x, y, z, n)) continue;
         float c[6];
         long long off[6];
         level_edges(L, x, y, z, n, c, off);
@@ -355,7 +378,7 @@ __global__ void __launch_bounds__(kBlock, 4) k_mg_sweep(DevProblem P, MgLevel L,
 // children of a coarse voxel lie in one tile and are summed in the warp (the pair
 // along x) and in shared memory (y, then z).  Along an axis on which the tile is
 // one voxel long there is one voxel, and nothing to pair.
-template <int K>
+template <int K, bool USUAL>
 __global__ void __launch_bounds__(kBlock, 4) k_mg_restrict(DevProblem P, MgLevel F, MgLevel C, const float* h0,
                                                         const float4* __restrict__ xf, const WsHeader* hdr)
 {
@@ -363,18 +386,21 @@ __global__ void __launch_bounds__(kBlock, 4) k_mg_restrict(DevProblem P, MgLevel
     __shared__ float4 part[kBlock];
     if (solve_done(hdr)) return;
     const int tid = threadIdx.x;
-    const int px = F.tiles.lx > 0, py = F.tiles.ly > 0, pz = F.tiles.lz > 0;    // pairs along an axis
-    const int lx = F.tiles.lx - px, ly = F.tiles.ly - py, lz = F.tiles.lz - pz;     // the tile's coarse voxels
+    const VoxelTiles tl = tiles_of<USUAL>(F);
+    const int px = tl.lx > 0, py = tl.ly > 0, pz = tl.lz > 0;    // pairs along an axis
+    const int lx = tl.lx - px, ly = tl.ly - py, lz = tl.lz - pz;     // the tile's coarse voxels
     const int u = tid & ((1 << lx) - 1), v = (tid >> lx) & ((1 << ly) - 1), s = tid >> (lx + ly);
-    const int sy = 1 << lx, sz = sy << F.tiles.ly;                                  // strides of part
+    const int sy = 1 << lx, sz = sy << tl.ly;                                  // strides of part
     const int p0 = u + (v << py) * sy + (s << pz) * sz;
+    const int ix = tid & ((1 << tl.lx) - 1), iy = (tid >> tl.lx) & ((1 << tl.ly) - 1),
+              iz = tid >> (tl.lx + tl.ly);                                // this thread's place
     for (long long t = blockIdx.x; t < F.tiles.count; t += gridDim.x) {
         int x, y, z;
         long long n;
         float d[K];
 #pragma unroll
         for (int a = 0; a < K; ++a) d[a] = 0.0f;
-        if (tile_voxel(F, t, x, y, z, n)) {
+        if (tile_voxel<USUAL>(F, t, x, y, z, n)) {
             float c[6];
             long long off[6];
             level_edges(F, x, y, z, n, c, off);
@@ -395,9 +421,7 @@ __global__ void __launch_bounds__(kBlock, 4) k_mg_restrict(DevProblem P, MgLevel
             auto line = [&](int p) { return py ? add4(part[p], part[p + sy]) : part[p]; };
             const float4 sum = pz ? add4(line(p0), line(p0 + sz)) : line(p0);
             // the tile's corner, halved, is its first coarse voxel
-            int bx, by, bz;
-            F.tiles.corner(t, bx, by, bz);
-            const int cx = (bx >> 1) + u, cy = (by >> 1) + v, cz = (bz >> 1) + s;
+            const int cx = ((x - ix) >> 1) + u, cy = ((y - iy) >> 1) + v, cz = ((z - iz) >> 1) + s;
             if (cx < C.nx && cy < C.ny && cz < C.nz) C.r[cx + (long long)C.nx * (cy + (long long)C.ny * cz)] = sum;
         }
         __syncthreads();
@@ -497,7 +521,7 @@ __global__ void __launch_bounds__(512) k_mg_coarsest_small(DevProblem P, MgLevel
 // ------------------------------------------------------------ CG
 
 // r = g + L y (L from the JTV weights), |r_0|^2; scalars reset.
-template <int K>
+template <int K, bool USUAL>
 __global__ void __launch_bounds__(kBlock) k_mgcg_init(DevProblem P, MgLevel L0, const float* __restrict__ g,
                                                       const float* __restrict__ y, double tol2,
                                                       WsHeader* hdr, double* resid, Reduce red)
@@ -506,7 +530,7 @@ __global__ void __launch_bounds__(kBlock) k_mgcg_init(DevProblem P, MgLevel L0, 
     for (long long t = blockIdx.x; t < L0.tiles.count; t += gridDim.x) {
         int x, yy, z;
         long long n;
-        if (!tile_voxel(L0, t, x, yy, z, n)) continue;
+        if (!tile_voxel<USUAL>(L0, t, x, yy, z, n)) continue;
         float c[6];
         long long off[6];
         level_edges(L0, x, yy, z, n, c, off);
@@ -573,7 +597,7 @@ __global__ void __launch_bounds__(kBlock) k_mgcg_rz(long long N, const float4* _
 
 // p = z + beta p_old (at the voxel and its neighbours), q = (H + L) p, p . q;
 // alpha = rz / p.q.
-template <int K>
+template <int K, bool USUAL>
 __global__ void __launch_bounds__(kBlock, 4) k_mgcg_matvec(DevProblem P, MgLevel L0, const float* h0,
                                                         const float4* __restrict__ pold,
                                                         float4* __restrict__ pnew, float4* __restrict__ q,
@@ -607,7 +631,7 @@ __global__ void __launch_bounds__(kBlock, 4) k_mgcg_matvec(DevProblem P, MgLevel
     for (long long t = blockIdx.x; t < L0.tiles.count; t += gridDim.x) {
         int x, y, zz;
         long long n;
-        if (!tile_voxel(L0, t, x, y, zz, n)) continue;
+        if (!tile_voxel<USUAL>(L0, t, x, y, zz, n)) continue;
         float c[6];
         long long off[6];
         level_edges(L0, x, y, zz, n, c, off);
@@ -652,8 +676,8 @@ __global__ void __launch_bounds__(kBlock, 4) k_mgcg_matvec(DevProblem P, MgLevel
 
 // x += alpha p, r -= alpha q, |r|^2; the iteration counter and the tolerance.
 // SWEEP: also the next cycle's first sweep, t = omega D^-1 r.
-template <int K, bool SWEEP>
-__global__ void __launch_bounds__(kBlock, 4) k_mgcg_update(DevProblem P, MgLevel L0, const float* h0, float omega,
+template <int K, bool SWEEP, bool USUAL>
+__global__ void __launch_bounds__(kBlock, 5) k_mgcg_update(DevProblem P, MgLevel L0, const float* h0, float omega,
                                                         int j, float4* __restrict__ xacc,
                                                         const float4* __restrict__ p,
                                                         const float4* __restrict__ q, WsHeader* hdr,
@@ -672,7 +696,7 @@ __global__ void __launch_bounds__(kBlock, 4) k_mgcg_update(DevProblem P, MgLevel
     for (long long t = blockIdx.x; t < L0.tiles.count; t += gridDim.x) {
         int x, y, z;
         long long n;
-        if (!tile_voxel(L0, t, x, y, z, n)) continue;
+        if (!tile_voxel<USUAL>(L0, t, x, y, z, n)) continue;
         float xv[K], pv[K], qv[K], rv[K];
         unpack4<K>(p[n], pv);
         unpack4<K>(q[n], qv);
@@ -760,12 +784,14 @@ static void vcycle(const DevProblem& P, const MgBufs& B, int l, const float* h0,
 {
     const MgLevel& Lv = B.lv[l];
     const int grid = mg_grid(Lv);
+    const bool usual = usual_tiles(Lv);
     const float om = o.mg_omega;
     auto sweep = [&](auto from, bool dot, const MgLevel& C, const float4* xin, float4* xout) {
         constexpr int FROM = decltype(from)::value;
         LaunchScope ls(MPM_KERNEL_MG, st);
-        if (dot) k_mg_sweep<K, FROM, true><<<grid, kBlock, 0, st>>>(P, Lv, C, h0, om, xin, xout, first, hdr, red);
-        else k_mg_sweep<K, FROM, false><<<grid, kBlock, 0, st>>>(P, Lv, C, h0, om, xin, xout, first, hdr, red);
+        const auto f = dot ? (usual ? k_mg_sweep<K, FROM, true, true> : k_mg_sweep<K, FROM, true, false>)
+                           : (usual ? k_mg_sweep<K, FROM, false, true> : k_mg_sweep<K, FROM, false, false>);
+        f<<<grid, kBlock, 0, st>>>(P, Lv, C, h0, om, xin, xout, first, hdr, red);
     };
     using Zero = std::integral_constant<int, kFromZero>;
     using FromX = std::integral_constant<int, kFromX>;
@@ -805,7 +831,8 @@ static void vcycle(const DevProblem& P, const MgBufs& B, int l, const float* h0,
     const MgLevel& C = B.lv[l + 1];
     {
         LaunchScope ls(MPM_KERNEL_MG, st);
-        k_mg_restrict<K><<<grid, kBlock, 0, st>>>(P, Lv, C, h0, cur, hdr);
+        const auto f = usual ? k_mg_restrict<K, true> : k_mg_restrict<K, false>;
+        f<<<grid, kBlock, 0, st>>>(P, Lv, C, h0, cur, hdr);
     }
     vcycle<K>(P, B, l + 1, h0, o, false, first, hdr, red, st);
     for (int s = 0; s < o.mg_nu; ++s) {
@@ -831,18 +858,21 @@ static cudaError_t solve_mg_k(const DevProblem& P, const SolveOpts& o, const flo
     MgLevel L0 = B.lv[0];
     const int grid = voxel_grid(P.N), tgrid = mg_grid(L0);
     const double tol2 = o.tol_cg > 0.0 ? o.tol_cg * o.tol_cg : 0.0;
-    const bool one_level = B.L == 1;
+    const bool one_level = B.L == 1, usual = usual_tiles(L0);
     {
         LaunchScope ls(MPM_KERNEL_MG, st);
-        k_mg_kappa0<<<tgrid, kBlock, 0, st>>>(P, L0, w);
+        const auto f = usual ? k_mg_kappa0<true> : k_mg_kappa0<false>;
+        f<<<tgrid, kBlock, 0, st>>>(P, L0, w);
     }
     for (int l = 0; l + 1 < B.L; ++l) {
         LaunchScope ls(MPM_KERNEL_MG, st);
-        k_mg_coarsen<<<mg_grid(B.lv[l + 1]), kBlock, 0, st>>>(P, B.lv[l], B.lv[l + 1], h);
+        const auto f = usual_tiles(B.lv[l + 1]) ? k_mg_coarsen<true> : k_mg_coarsen<false>;
+        f<<<mg_grid(B.lv[l + 1]), kBlock, 0, st>>>(P, B.lv[l], B.lv[l + 1], h);
     }
     {
         LaunchScope ls(MPM_KERNEL_PCG_INIT, st);
-        k_mgcg_init<K><<<tgrid, kBlock, 0, st>>>(P, L0, g, y, tol2, hdr, resid, red);
+        const auto f = usual ? k_mgcg_init<K, true> : k_mgcg_init<K, false>;
+        f<<<tgrid, kBlock, 0, st>>>(P, L0, g, y, tol2, hdr, resid, red);
     }
     auto cycle = [&](bool swept, int first) {
         vcycle<K>(P, B, 0, h, o, swept, first, hdr, red, st);
@@ -857,16 +887,15 @@ static cudaError_t solve_mg_k(const DevProblem& P, const SolveOpts& o, const flo
         const bool more = j + 1 < o.cg_iters;
         {
             LaunchScope ls(MPM_KERNEL_PCG_STEP, st);
-            k_mgcg_matvec<K><<<tgrid, kBlock, 0, st>>>(P, L0, h, pold, pnew, B.cq, j == 0, hdr, red);
+            const auto f = usual ? k_mgcg_matvec<K, true> : k_mgcg_matvec<K, false>;
+            f<<<tgrid, kBlock, 0, st>>>(P, L0, h, pold, pnew, B.cq, j == 0, hdr, red);
         }
         {
             LaunchScope ls(MPM_KERNEL_PCG_STEP, st);
-            if (more && !one_level)
-                k_mgcg_update<K, true><<<tgrid, kBlock, 0, st>>>(P, L0, h, o.mg_omega, j, B.cx, pnew, B.cq, hdr,
-                                                                 resid, red);
-            else
-                k_mgcg_update<K, false><<<tgrid, kBlock, 0, st>>>(P, L0, h, o.mg_omega, j, B.cx, pnew, B.cq, hdr,
-                                                                  resid, red);
+            const auto f = more && !one_level
+                               ? (usual ? k_mgcg_update<K, true, true> : k_mgcg_update<K, true, false>)
+                               : (usual ? k_mgcg_update<K, false, true> : k_mgcg_update<K, false, false>);
+            f<<<tgrid, kBlock, 0, st>>>(P, L0, h, o.mg_omega, j, B.cx, pnew, B.cq, hdr, resid, red);
         }
         if (more) cycle(!one_level, 0);
     }
