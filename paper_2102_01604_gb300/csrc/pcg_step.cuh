@@ -192,13 +192,23 @@ __device__ __forceinline__ Maps axpy(float s, const Maps& v, const Maps& w)
 __device__ __forceinline__ Maps minus(const Maps& v, const Maps& w) { return axpy(-1.0f, w, v); }
 
 // *at = v if `yes`, as one predicated store.  The tests for a stored z cost a
-// solve of 176x240x256 0.3% this way (7.41 -> 7.43 ms; a 64^3 fit 10.06 -> 10.01),
+// solve of 176x240x256 0.3% this way (7.41 -> 7.43 ms; a 64^3 fit 10.05 -> 10.02;
+// three maps, 136x141x109, 28 iterations 1.66 -> 1.68, 64^3 none),
 // 0.8% with an if around the store (7.47), more with one branch around both
 // forms of z (7.60) or a second copy of the march (7.42, but the 64^3 fit 10.38).
 __device__ __forceinline__ void store_if(int yes, float4* at, const Maps& v)
 {
     asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.s32 q, %0, 0;\n\t@q st.global.v4.f32 [%1], {%2, %3, %4, %5};\n\t}"
                  ::"r"(yes), "l"(at), "f"(v.a.x), "f"(v.a.y), "f"(v.b.x), "f"(v.b.y)
+                 : "memory");
+}
+
+// v = *at if `yes`, as one predicated load.
+__device__ __forceinline__ void load_if(int yes, Maps& v, const float4* at)
+{
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.s32 q, %4, 0;\n\t@q ld.global.v4.f32 {%0, %1, %2, %3}, [%5];\n\t}"
+                 : "+f"(v.a.x), "+f"(v.a.y), "+f"(v.b.x), "+f"(v.b.y)
+                 : "r"(yes), "l"(at)
                  : "memory");
 }
 

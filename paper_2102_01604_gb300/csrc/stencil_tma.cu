@@ -366,10 +366,11 @@ __device__ __forceinline__ void step_body(
                         }
                         if (inside) {
                             if (!first) pout[n] = pn.vec();
-                            if (!first) store_if(s_sc.zout, zout + n, zn);
+                            if (!first) store_if(K == 3 ? sc.zout : s_sc.zout, zout + n, zn);
                             if (fold) {
                                 const float4* bx = reinterpret_cast<const float4*>(st + L::X_OFF);
-                                const Maps f = sc.zin ? Maps(p2[n]) : pz;         // p_{j-2}
+                                Maps f = pz;                                      // p_{j-2}
+                                load_if(sc.zin, f, p2 + n);
                                 xacc[n] = fold_x(readx ? Maps(bx[tc]) : zero, sc, f, p1).vec();
                             }
                         }
