@@ -727,11 +727,13 @@ __global__ void __launch_bounds__(kBlock) k_pcg_init_batch(const __grid_constant
 // marching a run of z planes; each neighbour's p_j is formed from its own
 // p_{j-1}, v_{j-1} and p_{j-2} (or the stored z_{j-1}) read from memory.  Used
 // for volumes or pointers the TMA kernel cannot take (a volume smaller than a tile, unaligned buffers).
-// Three blocks per SM, with a few registers spilled: bound by the latency of its
-// neighbours' loads (30 iterations of 2x1024x512 with four maps 11.1 ms, 11.5 with
-// the two that 106 registers leave; three maps 9.9 and 13.0).
-template <int K, int MODE>
-__global__ void __launch_bounds__(kBlock, 3) k_pcg_step(DevProblem P, int zc, int j, int want_rr,
+// MINB blocks per SM: three, with a few registers spilled, where the launch has as
+// many, because the latency of the neighbours' loads bounds it (30 iterations of
+// 2x1024x512 with four maps 11.1 ms, 11.5 with the two that 106 registers leave;
+// three maps 9.9 and 13.0); two, without spills, for smaller launches (17x16x15
+// 30 iterations 297 us, 313 with three).
+template <int K, int MODE, int MINB>
+__global__ void __launch_bounds__(kBlock, MINB) k_pcg_step(DevProblem P, int zc, int j, int want_rr,
                                                      const float* __restrict__ h,
                                                      const float* __restrict__ w,
                                                      const float4* __restrict__ pin,
@@ -1071,8 +1073,9 @@ static cudaError_t launch_step_plain(const DevProblem& P, const StencilGrid& sg,
     const float4* zprev = B.z[jm & 1];
     float4 *vout = B.v[j & 1], *pout = B.p[j % 3], *zout = B.z[j & 1];
     cudaError_t e;
+    const bool few = (long long)sg.grid.x * sg.grid.y * sg.grid.z <= 2 * kNumSm;
 #define MPM_STEP_PLAIN(M)                                                                          \
-    e = launch_dependent(overlap, k_pcg_step<K, M>, sg.grid, sg.block, 0, st, P, sg.zc, j, want_rr, h, w, pin, vin, p2, \
+    e = launch_dependent(overlap, few ? k_pcg_step<K, M, 2> : k_pcg_step<K, M, 3>, sg.grid, sg.block, 0, st, P, sg.zc, j, want_rr, h, w, pin, vin, p2, \
                          zprev, vout, pout, B.x, zout, hdr, resid, red)
     switch (step_mode(j)) {
     case kModeFirst: MPM_STEP_PLAIN(kModeFirst); break;
