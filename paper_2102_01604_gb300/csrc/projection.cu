@@ -276,9 +276,13 @@ __device__ __forceinline__ F gather_pullers(const ProjC& q, int x, int y, int z,
 // gathers' latency and instruction issue (about 900 instructions per voxel).
 // It took 419 us per contrast at 176x240x256 with 64-bit divisions for the
 // voxel's indices, all corners behind branches, four maps for every contrast
-// and 64 B records staged in shared memory.
+// and 64 B records staged in shared memory.  Four blocks per SM (60 to 64
+// registers) for more of a voxel's loads in flight: left to itself the compiler
+// takes 40 or 48 registers as it happens, and this pass and the push take 2.05 ms
+// at 176x240x256 instead of 1.97, 1.35 instead of 1.31 at 188x195x184 with bfloat16
+// echoes and the row-sum loading.
 template <int K, int PRE, typename XT, bool USUAL>
-__global__ void __launch_bounds__(kBlock) k_grad_hess_proj(DevProblem P, ProjC q, int c,
+__global__ void __launch_bounds__(kBlock, 4) k_grad_hess_proj(DevProblem P, ProjC q, int c,
                                                            const float* __restrict__ y,
                                                            const XT* __restrict__ x,
                                                            const float* __restrict__ b1p,
@@ -381,7 +385,7 @@ struct PushInto {
 // Bound: instruction issue and the gathers' L1 traffic (about 8 contributing
 // voxels per contrast).  Three scans of 176x240x256 took 1468 us with 64 B
 // records, 64-bit divisions, linear blocks and every point of the box tested;
-// both passes together took 2.73 ms, 2.04 ms now.
+// both passes together took 2.73 ms, 1.97 ms now.
 // IT: an index type that holds every acquisition voxel's index.
 template <int K, typename IT, bool USUAL>
 __global__ void __launch_bounds__(kBlock, 4) k_push_all(DevProblem P, DevProj Q, ProjBufs B,
